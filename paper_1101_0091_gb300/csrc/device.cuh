@@ -112,6 +112,42 @@ __device__ __forceinline__ float ldcs(const float* p) { return __ldcs(p); }
 __device__ __forceinline__ f32n ldcs(const f32n* p) { return f32n{__ldcs(reinterpret_cast<const float*>(p))}; }
 __device__ __forceinline__ int32_t ldcs(const int32_t* p) { return __ldcs(p); }
 
+// Columns per lane of the column-split kernels (k_crs_cols, k_sell_cols) for k right-hand sides: 4 or
+// 2 when k divides by it and every row of B and C starts on 16 bytes (16-byte accesses), else 1 (odd k,
+// odd leading dimensions, blocks 8 bytes off).  These products are bound by the FP64 pipe (one warp
+// FMA occupies an SM for 16 cycles), so a lane per column costs nothing that the pipe does not hide,
+// while a masked kernel of 4, 8 or 16 columns on one lane issued the masked FMAs as well.  Measured,
+// masked -> lanes: k = 3 on a 131 x 127 x 129 Poisson matrix 107.9 -> 86.3 us (FP64 floor 71); k = 6,
+// ld = 8 on a 600,011-row eigenproblem matrix 173.1 -> 111.4 us (floor 79); k = 16, ld = 17 up to 8 x.
+inline int cols_per_lane(int k, const double* B, int64_t ldb, const double* C, int64_t ldc) {
+  const bool a16 = ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0;
+  return !a16 || k % 2 ? 1 : (k % 4 ? 2 : 4);
+}
+
+// W consecutive columns of a block row: 16-byte accesses for W = 2, 4.
+template <int W>
+__device__ __forceinline__ void load_cols(const double* __restrict__ b, double (&g)[W]) {
+  if constexpr (W == 1) {
+    g[0] = __ldg(b);
+  } else {
+#pragma unroll
+    for (int q = 0; q < W; q += 2) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(b + q));
+      g[q] = x.x;
+      g[q + 1] = x.y;
+    }
+  }
+}
+template <int W>
+__device__ __forceinline__ void store_cols(double* c, const double (&a)[W]) {
+  if constexpr (W == 1) {
+    c[0] = a[0];
+  } else {
+#pragma unroll
+    for (int q = 0; q < W; q += 2) reinterpret_cast<double2*>(c)[q / 2] = make_double2(a[q], a[q + 1]);
+  }
+}
+
 __device__ __forceinline__ double warp_sum_xor(double x, int width) {
   for (int off = width >> 1; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
   return x;

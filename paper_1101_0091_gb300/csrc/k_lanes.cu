@@ -7,12 +7,12 @@
 // scalar CRS kernel.  The same kernel with a row list and accumulate = 1 is the
 // halo pass of the local/halo split: C[rows[t]] += (halo row t) * B.
 //
-// CRS_L1 on a full, 16-byte aligned block of K >= 2 columns runs k_crs_cols
-// instead: the row's entries still go to one lane each in order, but the K
-// columns are split over G = K / W lanes (W = 4 columns per lane for K >= 8,
-// all K below), so every gather is a 16-byte load and the G lanes of a row
-// read one contiguous piece of its B row.  Each column's sum is formed in the
-// same order as in the scalar form, so the bits are the same.
+// CRS_L1 on a block of k >= 2 columns runs k_crs_cols instead: the row's entries
+// still go to one lane each in order, but the k columns are split over G = k / W
+// lanes (cols_per_lane: W = 4 or 2 with 16-byte gathers and stores, W = 1 for odd
+// or unaligned blocks), and the G lanes of a row read one contiguous piece of its
+// B row.  Each column's sum is formed in the same order whatever W is, so the bits
+// are the same.
 #include "device.cuh"
 
 namespace spmv {
@@ -105,25 +105,19 @@ __global__ void __launch_bounds__(kThreads, (K == 1 ? 8 : 1))
   }
 }
 
-// Columns per lane of the column-split form.
-template <int K>
-struct ColsPerLane {
-  static constexpr int value = K >= 8 ? 4 : K;
-};
-
-template <typename VT, int K>
-__global__ void __launch_bounds__(kThreads, 6)
+// k columns of a row on G = k / W lanes, W columns each (W = 4 or 2 with 16-byte accesses, else 1).
+template <typename VT, int W>
+__global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_crs_cols(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
-               int64_t ldc, int prefetch) {
-  constexpr int W = ColsPerLane<K>::value;
-  constexpr int G = K / W;           // lanes per row
-  constexpr int RPC = kThreads / G;  // rows per CTA
+               int64_t ldc, int G, int prefetch) {
+  const int rpc = kThreads / G;  // rows per CTA
   if (threadIdx.x == 0 && prefetch > 0)
-    prefetch_rows(((int64_t)blockIdx.x + prefetch) * RPC, RPC, n_rows, row_ptr, col, val);
-  const int64_t g = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G;
-  if (g >= n_rows) return;
-  const int c0 = (int)(threadIdx.x % G) * W;  // first column of this lane
+    prefetch_rows(((int64_t)blockIdx.x + prefetch) * rpc, rpc, n_rows, row_ptr, col, val);
+  const int r = (int)threadIdx.x / G;
+  const int64_t g = (int64_t)blockIdx.x * rpc + r;
+  if (r >= rpc || g >= n_rows) return;
+  const int c0 = ((int)threadIdx.x - r * G) * W;  // first column of this lane
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   double acc[W];
 #pragma unroll
@@ -131,39 +125,27 @@ __global__ void __launch_bounds__(kThreads, 6)
   const double* Bc = B + c0;
   for (int j = rs; j < re; ++j) {
     const double v = to_f64(ldg(val + j));
-    const double* b = Bc + (int64_t)ldg(col + j) * ldb;
     double gv[W];
-#pragma unroll
-    for (int q = 0; q < W; q += 2) {
-      const double2 x = __ldg(reinterpret_cast<const double2*>(b + q));
-      gv[q] = x.x;
-      gv[q + 1] = x.y;
-    }
+    load_cols(Bc + (int64_t)ldg(col + j) * ldb, gv);
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[q] = fma(v, gv[q], acc[q]);
   }
-  double2* out = reinterpret_cast<double2*>(C + g * ldc + c0);
-#pragma unroll
-  for (int q = 0; q < W; q += 2) out[q / 2] = make_double2(acc[q], acc[q + 1]);
+  store_cols(C + g * ldc + c0, acc);
+}
+
+template <typename VT, int W>
+static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int32_t* col, const VT* val,
+                               const double* B, int64_t ldb, double* C, int64_t ldc, int k, int pf, cudaStream_t s) {
+  const int G = k / W, rpc = kThreads / G;
+  const int64_t grid = (n_rows + rpc - 1) / rpc;
+  k_crs_cols<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, row_ptr, col, val, B, ldb, C, ldc, G, pf);
+  return cudaGetLastError();
 }
 
 template <typename VT, int L, int K>
 static cudaError_t launch_lanes_t(int64_t n_rows, const int32_t* rows, const int32_t* row_ptr,
                                   const int32_t* col, const VT* val, const double* B, int64_t ldb, double* C,
                                   int64_t ldc, int k, bool acc, int pf, cudaStream_t s) {
-  if (n_rows == 0) return cudaSuccess;
-  if constexpr (L == 1 && K >= 2) {
-    // a full block of K columns with 16-byte aligned rows, not accumulating: the column-split
-    // form (16-byte gathers and stores; these products are FP64-pipe-bound, and halving the
-    // gather instructions, then sharing each B row among G lanes, took the 3D Poisson product
-    // at K = 2 / 16 from 0.82 / 0.81 to 0.95 / 0.98 of the FP64 peak)
-    if (k == K && !acc && !rows && ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0) {
-      constexpr int G = K / ColsPerLane<K>::value;
-      const int64_t grid = (n_rows * G + kThreads - 1) / kThreads;
-      k_crs_cols<VT, K><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, row_ptr, col, val, B, ldb, C, ldc, pf);
-      return cudaGetLastError();
-    }
-  }
   const int64_t rows_per_cta = kThreads / L;
   const int64_t grid = (n_rows + rows_per_cta - 1) / rows_per_cta;
   if constexpr (L > 1 && K >= 2) {
@@ -183,11 +165,20 @@ template <typename VT, int L>
 static cudaError_t lanes_k(int64_t n, const int32_t* rows, const int32_t* rp, const int32_t* col, const VT* val,
                            const double* B, int64_t ldb, double* C, int64_t ldc, int k, bool acc,
                            int pf, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
   if (k <= 1) return launch_lanes_t<VT, L, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  if (k <= 2) return launch_lanes_t<VT, L, 2>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  if (k <= 4) return launch_lanes_t<VT, L, 4>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  if (k <= 8) return launch_lanes_t<VT, L, 8>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  return launch_lanes_t<VT, L, 16>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
+  if constexpr (L == 1) {  // k >= 2 never comes with a row list (the halo pass has k = 1)
+    switch (cols_per_lane(k, B, ldb, C, ldc)) {
+      case 4: return launch_cols<VT, 4>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+      case 2: return launch_cols<VT, 2>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+      default: return launch_cols<VT, 1>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    }
+  } else {
+    if (k <= 2) return launch_lanes_t<VT, L, 2>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
+    if (k <= 4) return launch_lanes_t<VT, L, 4>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
+    if (k <= 8) return launch_lanes_t<VT, L, 8>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
+    return launch_lanes_t<VT, L, 16>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
+  }
 }
 
 template <typename VT>

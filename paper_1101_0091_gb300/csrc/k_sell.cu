@@ -9,11 +9,10 @@
 // rows by length inside sigma-windows keeps the padding (idle FP64 issue
 // slots) small.
 //
-// A full, 16-byte aligned block of K >= 2 columns runs k_sell_cols: each
-// sorted row is shared by G = K / W lanes (W = 4 columns per lane for K >= 8,
-// all K below), every gather is a 16-byte load, and the G lanes of a row read
-// one contiguous piece of its B row; a row's slots are still summed in order,
-// so the bits equal the scalar form's.
+// A block of k >= 2 columns runs k_sell_cols: each sorted row is shared by
+// G = k / W lanes with W columns each (cols_per_lane), and the G lanes of a row
+// read one contiguous piece of its B row; a row's slots are still summed in
+// order, so every W gives the same bits.
 #include "device.cuh"
 
 namespace spmv {
@@ -33,12 +32,12 @@ __device__ __forceinline__ void prefetch_chunks(int64_t c0, int64_t chunks, int6
   }
 }
 
-template <typename VT, int K>
+template <typename VT>
 __global__ void __launch_bounds__(kThreads)
     k_sell(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm,
            const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
            const int32_t* __restrict__ col, const VT* __restrict__ val, const double* __restrict__ B,
-           int64_t ldb, double* __restrict__ C, int64_t ldc, int k, int prefetch) {
+           int64_t ldb, double* __restrict__ C, int64_t ldc, int prefetch) {
   constexpr int CPC = kThreads / kSellC;  // chunks per CTA
   // bring the slots of the CTA `prefetch` positions ahead into L2
   if (threadIdx.x == 0 && prefetch > 0)
@@ -49,11 +48,9 @@ __global__ void __launch_bounds__(kThreads)
   const int t = threadIdx.x & 31;
   const int len = __ldg(chunk_len + c);
   const int64_t base = __ldg(chunk_ptr + c) + t;
-  double acc[K];
-#pragma unroll
-  for (int q = 0; q < K; ++q) acc[q] = 0.0;
+  double acc = 0.0;
   // batches of NB slots: all gathers of a batch are issued before its FMAs
-  constexpr int NB = K >= 4 ? 1 : 2;
+  constexpr int NB = 2;
   for (int j = 0; j < len; j += NB) {
     double v[NB];
     const double* b[NB];
@@ -63,46 +60,36 @@ __global__ void __launch_bounds__(kThreads)
       v[u] = to_f64(ldcs(val + slot));
       b[u] = B + (int64_t)ldcs(col + slot) * ldb;
     }
-    double g[NB][K];
+    double g[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) g[u] = j + u < len ? __ldg(b[u]) : 0.0;
 #pragma unroll
     for (int u = 0; u < NB; ++u)
-#pragma unroll
-      for (int q = 0; q < K; ++q) g[u][q] = (j + u < len && q < k) ? __ldg(b[u] + q) : 0.0;
-#pragma unroll
-    for (int u = 0; u < NB; ++u)
-#pragma unroll
-      for (int q = 0; q < K; ++q)
-        if (j + u < len && q < k) acc[q] = fma(v[u], g[u][q], acc[q]);
+      if (j + u < len) acc = fma(v[u], g[u], acc);
   }
   if (r >= n_rows) return;
-  double* out = C + (int64_t)__ldg(perm + r) * ldc;
-#pragma unroll
-  for (int q = 0; q < K; ++q)
-    if (q < k) out[q] = acc[q];
+  C[(int64_t)__ldg(perm + r) * ldc] = acc;
 }
 
-// Columns per lane of the column-split form.
-template <int K>
-struct SellColsPerLane {
-  static constexpr int value = K >= 8 ? 4 : K;
-};
-
-template <typename VT, int K>
-__global__ void __launch_bounds__(kThreads, 6)
+// k columns of a sorted row on G = k / W lanes, W columns each (as k_crs_cols).
+template <typename VT, int W>
+__global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm,
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
                 const int32_t* __restrict__ col, const VT* __restrict__ val, const double* __restrict__ B,
-                int64_t ldb, double* __restrict__ C, int64_t ldc, int prefetch) {
-  constexpr int W = SellColsPerLane<K>::value;
-  constexpr int G = K / W;                      // lanes per row
-  constexpr int CPC = kThreads / (kSellC * G);  // chunks per CTA
-  if (threadIdx.x == 0 && prefetch > 0)
-    prefetch_chunks(((int64_t)blockIdx.x + prefetch) * CPC, CPC, n_chunks, chunk_ptr, col, val);
-  const int64_t ra = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const int64_t r = ra / G;  // sorted row
+                int64_t ldb, double* __restrict__ C, int64_t ldc, int G, int prefetch) {
+  const int rpc = kThreads / G;  // sorted rows per CTA
+  if (threadIdx.x == 0 && prefetch > 0) {
+    // the chunks that start in the rows of the CTA `prefetch` positions ahead
+    const int64_t f0 = (((int64_t)blockIdx.x + prefetch) * rpc + kSellC - 1) / kSellC;
+    const int64_t f1 = (((int64_t)blockIdx.x + prefetch + 1) * rpc + kSellC - 1) / kSellC;
+    if (f1 > f0) prefetch_chunks(f0, f1 - f0, n_chunks, chunk_ptr, col, val);
+  }
+  const int rl = (int)threadIdx.x / G;
+  const int64_t r = (int64_t)blockIdx.x * rpc + rl;  // sorted row
+  if (rl >= rpc || r >= n_rows) return;
   const int64_t c = r >> 5;
-  if (c >= n_chunks) return;
-  const int c0 = (int)(ra % G) * W;  // first column of this lane
+  const int c0 = ((int)threadIdx.x - rl * G) * W;  // first column of this lane
   const int len = __ldg(chunk_len + c);
   const int64_t base = __ldg(chunk_ptr + c) + (r & (kSellC - 1));
   double acc[W];
@@ -112,54 +99,39 @@ __global__ void __launch_bounds__(kThreads, 6)
   for (int j = 0; j < len; ++j) {
     const int64_t slot = base + (int64_t)j * kSellC;
     const double v = to_f64(ldcs(val + slot));
-    const double* b = Bc + (int64_t)ldcs(col + slot) * ldb;
     double g[W];
-#pragma unroll
-    for (int q = 0; q < W; q += 2) {
-      const double2 x = __ldg(reinterpret_cast<const double2*>(b + q));
-      g[q] = x.x;
-      g[q + 1] = x.y;
-    }
+    load_cols(Bc + (int64_t)ldcs(col + slot) * ldb, g);
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
   }
-  if (r >= n_rows) return;
-  double2* out = reinterpret_cast<double2*>(C + (int64_t)__ldg(perm + r) * ldc + c0);
-#pragma unroll
-  for (int q = 0; q < W; q += 2) out[q / 2] = make_double2(acc[q], acc[q + 1]);
+  store_cols(C + (int64_t)__ldg(perm + r) * ldc + c0, acc);
 }
 
-template <typename VT, int K>
-static cudaError_t launch_sell_t(const SellDev& S, const VT* val, const double* B, int64_t ldb, double* C,
-                                 int64_t ldc, int k, cudaStream_t s) {
-  if (S.n_chunks == 0) return cudaSuccess;
-  if constexpr (K >= 2) {
-    // a full block of K columns with 16-byte aligned rows: the column-split form (these
-    // products are FP64-pipe-bound; on the eigenproblem-shaped matrix it took K = 2 / 4 / 16
-    // from 0.59 / 0.71 / 0.88 to 0.82 / 0.94 / 0.97 of the FP64 peak)
-    if (k == K && ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0) {
-      constexpr int G = K / SellColsPerLane<K>::value;
-      const int64_t grid = (S.n_chunks * kSellC * G + kThreads - 1) / kThreads;
-      k_sell_cols<VT, K><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr,
-                                                              S.chunk_len, S.col, val, B, ldb, C, ldc, S.prefetch);
-      return cudaGetLastError();
-    }
-  }
-  const int64_t threads = S.n_chunks * kSellC;
-  const int64_t grid = (threads + kThreads - 1) / kThreads;
-  k_sell<VT, K><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len, S.col,
-                                                     val, B, ldb, C, ldc, k, S.prefetch);
+template <typename VT, int W>
+static cudaError_t launch_cols(const SellDev& S, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
+                               int k, cudaStream_t s) {
+  const int G = k / W, rpc = kThreads / G;
+  const int64_t grid = (S.n_rows + rpc - 1) / rpc;
+  k_sell_cols<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len,
+                                                         S.col, val, B, ldb, C, ldc, G, S.prefetch);
   return cudaGetLastError();
 }
 
 template <typename VT>
 static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                           int k, cudaStream_t s) {
-  if (k <= 1) return launch_sell_t<VT, 1>(S, val, B, ldb, C, ldc, k, s);
-  if (k <= 2) return launch_sell_t<VT, 2>(S, val, B, ldb, C, ldc, k, s);
-  if (k <= 4) return launch_sell_t<VT, 4>(S, val, B, ldb, C, ldc, k, s);
-  if (k <= 8) return launch_sell_t<VT, 8>(S, val, B, ldb, C, ldc, k, s);
-  return launch_sell_t<VT, 16>(S, val, B, ldb, C, ldc, k, s);
+  if (S.n_chunks == 0) return cudaSuccess;
+  if (k > 1) {
+    switch (cols_per_lane(k, B, ldb, C, ldc)) {
+      case 4: return launch_cols<VT, 4>(S, val, B, ldb, C, ldc, k, s);
+      case 2: return launch_cols<VT, 2>(S, val, B, ldb, C, ldc, k, s);
+      default: return launch_cols<VT, 1>(S, val, B, ldb, C, ldc, k, s);
+    }
+  }
+  const int64_t grid = (S.n_chunks * kSellC + kThreads - 1) / kThreads;
+  k_sell<VT><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len, S.col, val,
+                                                 B, ldb, C, ldc, S.prefetch);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sell(const SellDev& S, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
