@@ -95,6 +95,7 @@ struct spmv_plan {
   double scattered = 0.0;
   double fill256 = 1.0;
   bool auto_sell = false;
+  LongRows long_rows;   // built on AUTO's first resolution to CRS_L1 on a matrix with long rows
   HostCsr host;
   DevArena arena;
   CsrDev A;            // the whole matrix
@@ -291,7 +292,37 @@ static spmv_status build_sym_dev(spmv_plan* p) {
   return SPMV_OK;
 }
 
+// The rows of more than kShortRow entries; none when no row exceeds kAutoLongestRow or when they are
+// more than kAutoLongShare of the rows.
+static spmv_status build_long_rows(spmv_plan* p) {
+  if (p->long_rows.rows) return SPMV_OK;
+  const int32_t* rp = p->host.row_ptr.data();
+  const int64_t n = p->host.n_rows;
+  int32_t longest = 0;
+  int64_t n_long = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    longest = std::max(longest, rp[i + 1] - rp[i]);
+    n_long += rp[i + 1] - rp[i] > kShortRow;
+  }
+  if (longest <= kAutoLongestRow || n_long > kAutoLongShare * n) return SPMV_OK;
+  std::vector<int32_t> list, warp_rows;
+  for (int64_t i = 0; i < n; ++i) {
+    const int32_t len = rp[i + 1] - rp[i];
+    if (len > kShortRow) (len > kWarpRow ? list : warp_rows).push_back((int32_t)i);
+  }
+  LongRows lr;
+  lr.n_cta = (int)list.size();
+  lr.n_warp = (int)warp_rows.size();
+  list.insert(list.end(), warp_rows.begin(), warp_rows.end());
+  int32_t* d;
+  SPMV_CUDA(upload(p->arena, &d, list.data(), (int64_t)list.size(), 0));
+  lr.rows = d;
+  p->long_rows = lr;
+  return SPMV_OK;
+}
+
 static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
+  const bool is_auto = variant == SPMV_VARIANT_AUTO;
   if (variant == SPMV_VARIANT_AUTO) {
     variant = p->auto_sell ? SPMV_SELL : SPMV_CRS_L1;
     sigma = p->auto_sell ? 256 : sigma;
@@ -311,6 +342,13 @@ static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
     spmv_status st = build_sym_dev(p);
     if (st != SPMV_OK) return st;
   }
+  LongRows lr;
+  if (is_auto && variant == SPMV_CRS_L1) {
+    spmv_status st = build_long_rows(p);
+    if (st != SPMV_OK) return st;
+    lr = p->long_rows;
+  }
+  p->A.long_rows = lr;
   p->variant = variant;
   ++p->generation;
   return SPMV_OK;

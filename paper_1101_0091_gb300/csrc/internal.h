@@ -90,6 +90,16 @@ constexpr int kDefaultPrefetch = 456;
 // that format stores at least kAutoSellFill nonzeros per slot.
 constexpr double kAutoScattered = 0.3;
 constexpr double kAutoSellFill = 0.85;
+// AUTO's CRS_L1 gives the rows of more than kShortRow entries a warp or a CTA each when the longest
+// row exceeds kAutoLongestRow and they are at most kAutoLongShare of the rows; an explicit CRS_L1 keeps
+// every row on one thread.  Both sides, one thread per row -> long rows split: power-law lengths, 200,000
+// rows, longest row 40 / 64 / 96 / 256 at k = 1: 14.5 -> 14.0 / 16.6 -> 12.6 / 20.7 -> 14.3 /
+// 39.0 -> 14.4 us (2,000,000 rows: 69.7 -> 69.0 / 82.8 -> 73.4 / 95.7 -> 74.3 / 135.6 -> 77.6).  300,000
+// banded rows of which a share has 96 entries, the others 7: share 0.1 / 0.25 / 0.5 / 1 at k = 1 57.7 ->
+// 25.1 / 65.7 -> 49.6 / 70.3 -> 88.9 / 95.4 -> 164.4 us, at k = 4 204.8 -> 48.0 / 209.8 -> 94.7 / 212.0 ->
+// 168.5 / 209.1 -> 302.7 us.
+constexpr int kAutoLongestRow = 48;
+constexpr double kAutoLongShare = 0.25;
 
 // Share of a row sample's entries gathered at scattered addresses by consecutive rows (see host.cpp).
 double scattered_fraction(const int32_t* row_ptr, const int32_t* col, int64_t n_rows);

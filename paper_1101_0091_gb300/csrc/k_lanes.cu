@@ -142,6 +142,121 @@ static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int
   return cudaGetLastError();
 }
 
+// One row on NT threads (a warp or the CTA; thread t of them): EP entry lanes, a power of two, times
+// k column lanes.  Entry lane e adds entries rs + e, rs + e + EP, ...; a tree over sh (NT sums) adds
+// the entry lanes in a fixed order.  One column per lane for every k: the tree's FP64 adds are what
+// a row of a few dozen entries spends most on, and each step of it adds 32 useful sums this way.
+template <typename VT, int NT>
+__device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* __restrict__ row_ptr,
+                                         const int32_t* __restrict__ col, const VT* __restrict__ val,
+                                         const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+                                         int64_t ldc, double* sh) {
+  const int rs = __ldg(row_ptr + row), re = __ldg(row_ptr + row + 1);
+  const int ep = 1 << (31 - __clz(NT / k));
+  const int e = t / k, c = t - e * k;
+  double acc = 0.0;
+  if (e < ep) {
+    constexpr int U = 4;  // entries in flight per lane
+    for (int j = rs + e; j < re; j += U * ep) {
+      double v[U], g[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int jj = j + u * ep < re ? j + u * ep : j;
+        v[u] = to_f64(ldcs(val + jj));
+        g[u] = __ldg(B + (int64_t)ldcs(col + jj) * ldb + c);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u * ep < re) acc = fma(v[u], g[u], acc);
+    }
+  }
+  sh[t] = acc;
+  for (int h = ep >> 1; h > 0; h >>= 1) {
+    if (NT == 32) __syncwarp(); else __syncthreads();
+    if (e < h) sh[t] = acc += sh[t + h * k];
+  }
+  if (e == 0) C[(int64_t)row * ldc + c] = acc;
+}
+
+// CRS_L1 as AUTO runs it on matrices with long rows: the listed long rows first, each on a CTA or a
+// warp, then the others as in k_crs_cols.  What bounded these products was the longest row, walked by
+// one thread with one or eight gathers in flight: a 200,000-row matrix with power-law lengths up to 2000
+// took 212.9 us at k = 1 and takes 14.4 now (k = 4, 32 entries and more per row and lane: 86 -> 32 us at
+// lengths up to 256); what is left is three dependent loads per wave and, back to back, the host's
+// launch.  A warp covers up to 512 entries in 16 steps of which four are in flight; longer rows take
+// a CTA, and both come first so that the short rows fill their tail.
+template <typename VT, int W>
+__global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 5))
+    k_crs_long(LongRows lr, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+               int64_t ldc, int G, int prefetch) {
+  __shared__ double sh[kThreads];
+  constexpr int WARPS = kThreads / 32;
+  const int tid = (int)threadIdx.x;
+  int64_t blk = blockIdx.x;
+  if (blk < lr.n_cta) {
+    long_row<VT, kThreads>(__ldg(lr.rows + blk), tid, G * W, row_ptr, col, val, B, ldb, C, ldc, sh);
+    return;
+  }
+  blk -= lr.n_cta;
+  const int warp_ctas = (lr.n_warp + WARPS - 1) / WARPS;
+  if (blk < warp_ctas) {
+    const int i = (int)blk * WARPS + tid / 32;
+    if (i < lr.n_warp)
+      long_row<VT, 32>(__ldg(lr.rows + lr.n_cta + i), tid % 32, G * W, row_ptr, col, val, B, ldb, C, ldc,
+                       sh + (tid & ~31));
+    return;
+  }
+  blk -= warp_ctas;
+  const int rpc = kThreads / G;
+  if (tid == 0 && prefetch > 0) prefetch_rows((blk + prefetch) * rpc, rpc, n_rows, row_ptr, col, val);
+  const int r = tid / G;
+  const int64_t g = blk * rpc + r;
+  if (r >= rpc || g >= n_rows) return;
+  const int c0 = (tid - r * G) * W;
+  const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
+  if (re - rs > kShortRow) return;
+  double acc[W];
+#pragma unroll
+  for (int q = 0; q < W; ++q) acc[q] = 0.0;
+  const double* Bc = B + c0;
+  // NB entries in flight, then one by one: these products are bound by the FP64 pipe on large
+  // matrices, and a batch padded with masked multiply-adds issues them (3,000,000 rows of 5 entries,
+  // k = 3: 127.5 us padded, 94.6 us so)
+  constexpr int NB = W == 4 ? 2 : 4;
+  int j = rs;
+  for (; j + NB <= re; j += NB) {
+    double v[NB], gv[NB][W];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      v[u] = to_f64(ldg(val + j + u));
+      load_cols(Bc + (int64_t)ldg(col + j + u) * ldb, gv[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u)
+#pragma unroll
+      for (int q = 0; q < W; ++q) acc[q] = fma(v[u], gv[u][q], acc[q]);
+  }
+  for (; j < re; ++j) {
+    const double v = to_f64(ldg(val + j));
+    double gv[W];
+    load_cols(Bc + (int64_t)ldg(col + j) * ldb, gv);
+#pragma unroll
+    for (int q = 0; q < W; ++q) acc[q] = fma(v, gv[q], acc[q]);
+  }
+  store_cols(C + g * ldc + c0, acc);
+}
+
+template <typename VT, int W>
+static cudaError_t launch_long(const LongRows& lr, int64_t n_rows, const int32_t* row_ptr, const int32_t* col,
+                               const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
+                               int pf, cudaStream_t s) {
+  const int G = k / W, rpc = kThreads / G, warps = kThreads / 32;
+  const int64_t grid = lr.n_cta + (lr.n_warp + warps - 1) / warps + (n_rows + rpc - 1) / rpc;
+  k_crs_long<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(lr, n_rows, row_ptr, col, val, B, ldb, C, ldc, G, pf);
+  return cudaGetLastError();
+}
+
 template <typename VT, int L, int K>
 static cudaError_t launch_lanes_t(int64_t n_rows, const int32_t* rows, const int32_t* row_ptr,
                                   const int32_t* col, const VT* val, const double* B, int64_t ldb, double* C,
@@ -196,16 +311,25 @@ static cudaError_t lanes_dispatch(int lanes, int64_t n, const int32_t* rows, con
   }
 }
 
+template <typename VT>
+static cudaError_t crs_dispatch(const CsrDev& A, int lanes, const VT* val, const double* B, int64_t ldb, double* C,
+                                int64_t ldc, int k, cudaStream_t s) {
+  const LongRows& lr = A.long_rows;
+  if (lanes == 1 && lr.n_cta + lr.n_warp > 0) {
+    switch (cols_per_lane(k, B, ldb, C, ldc)) {
+      case 4: return launch_long<VT, 4>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
+      case 2: return launch_long<VT, 2>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
+      default: return launch_long<VT, 1>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
+    }
+  }
+  return lanes_dispatch<VT>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, val, B, ldb, C, ldc, k, false, A.prefetch, s);
+}
+
 cudaError_t launch_crs_lanes(const CsrDev& A, bool fp32, int lanes, const double* B, int64_t ldb, double* C,
                              int64_t ldc, int k, cudaStream_t s) {
-  if (fp32 && A.val32_special)
-    return lanes_dispatch<float>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, A.val32, B, ldb, C, ldc, k, false,
-                                 A.prefetch, s);
-  if (fp32)
-    return lanes_dispatch<f32n>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, reinterpret_cast<const f32n*>(A.val32),
-                                B, ldb, C, ldc, k, false, A.prefetch, s);
-  return lanes_dispatch<double>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, A.val, B, ldb, C, ldc, k, false,
-                                A.prefetch, s);
+  if (fp32 && A.val32_special) return crs_dispatch<float>(A, lanes, A.val32, B, ldb, C, ldc, k, s);
+  if (fp32) return crs_dispatch<f32n>(A, lanes, reinterpret_cast<const f32n*>(A.val32), B, ldb, C, ldc, k, s);
+  return crs_dispatch<double>(A, lanes, A.val, B, ldb, C, ldc, k, s);
 }
 
 cudaError_t launch_halo(const HaloDev& H, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc, int k,

@@ -20,6 +20,15 @@ constexpr int kWarpRowsPerBlock = kThreads / 32;
 constexpr int kSellC = 32;           // SELL chunk height
 constexpr uint32_t kBlockWarpFlag = 0x80000000u;  // high bit of a row-block entry: warp-per-row block
 
+// Rows of more than kShortRow entries, for the kernel that gives them a warp or a CTA each: those of
+// more than kWarpRow entries first (n_cta of them), then the others (n_warp).
+constexpr int kShortRow = 32;
+constexpr int kWarpRow = 512;
+struct LongRows {
+  const int32_t* rows = nullptr;
+  int n_cta = 0, n_warp = 0;
+};
+
 // Device view of one CRS matrix (values in FP64 and, optionally, FP32).
 struct CsrDev {
   int64_t n_rows = 0, n_cols = 0, nnz = 0;
@@ -32,6 +41,7 @@ struct CsrDev {
   int tile = 0;                     // nonzero capacity of a CRS_STAGED tile
   int prefetch = 0;                 // CTAs ahead whose val/col slices are prefetched into L2 (0 = off)
   bool val32_special = false;       // val32 holds a subnormal, infinite or NaN float
+  LongRows long_rows;               // listed (n_cta + n_warp > 0) when AUTO splits the long rows off CRS_L1
 };
 
 struct SellDev {
