@@ -192,7 +192,8 @@ spmv_status spmv_set_variant(spmv_handle h, int32_t variant, int32_t sell_sigma)
 spmv_status spmv_get_info(spmv_handle h, spmv_info* info);
 
 /* Launch parameters a tuner may change without touching the result.
- * prefetch_distance: each CTA of the row and SELL kernels asks the TMA engine
+ * prefetch_distance: each CTA of the row and SELL kernels (those of CRS_L1 on rows of
+ * eight and more entries on average excepted, which it slows) asks the TMA engine
  * to prefetch into L2 the matrix slice of the CTA this many positions ahead
  * (cp.async.bulk.prefetch.L2); 0 disables it.  Default: 456 (three per SM), and
  * 0 on matrices whose gathers are scattered (the test of SPMV_VARIANT_AUTO):

@@ -218,7 +218,7 @@ static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n
   double* dval;
   SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, 0));
   SPMV_CUDA(upload(p->arena, &dcol, col, nnz, pad_to(nnz, 4)));
-  SPMV_CUDA(upload(p->arena, &dval, val, nnz, pad_to(nnz, 2)));
+  SPMV_CUDA(upload(p->arena, &dval, val, nnz, pad_to(nnz, 4)));
   M->n_rows = n_rows;
   M->n_cols = n_cols;
   M->nnz = nnz;

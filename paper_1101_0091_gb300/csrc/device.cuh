@@ -112,6 +112,25 @@ __device__ __forceinline__ float ldcs(const float* p) { return __ldcs(p); }
 __device__ __forceinline__ f32n ldcs(const f32n* p) { return f32n{__ldcs(reinterpret_cast<const float*>(p))}; }
 __device__ __forceinline__ int32_t ldcs(const int32_t* p) { return __ldcs(p); }
 
+// Four consecutive entries from a 16-byte (col, float) or 32-byte (double) aligned address.
+__device__ __forceinline__ void ldg4(const double* p, double (&x)[4]) {
+  asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3])
+               : "l"(p));
+}
+__device__ __forceinline__ void ldg4(const float* p, float (&x)[4]) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  x[0] = t.x, x[1] = t.y, x[2] = t.z, x[3] = t.w;
+}
+__device__ __forceinline__ void ldg4(const f32n* p, f32n (&x)[4]) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  x[0].v = t.x, x[1].v = t.y, x[2].v = t.z, x[3].v = t.w;
+}
+__device__ __forceinline__ void ldg4(const int32_t* p, int32_t (&x)[4]) {
+  const int4 t = __ldg(reinterpret_cast<const int4*>(p));
+  x[0] = t.x, x[1] = t.y, x[2] = t.z, x[3] = t.w;
+}
+
 // Columns per lane of the column-split kernels (k_crs_cols, k_sell_cols) for k right-hand sides: 4 or
 // 2 when k divides by it and every row of B and C starts on 16 bytes (16-byte accesses), else 1 (odd k,
 // odd leading dimensions, blocks 8 bytes off).  These products are bound by the FP64 pipe (one warp

@@ -105,6 +105,20 @@ __global__ void __launch_bounds__(kThreads, (K == 1 ? 8 : 1))
   }
 }
 
+// The last 0..3 entries of a row (r of them, gathers x): no multiply-add is issued that no lane of the
+// warp needs.  A masked-off warp instruction occupies the FP64 pipe (16 cycles of an SM) like any other.
+template <typename VT, int W>
+__device__ __forceinline__ void add_tail(int r, const VT* v, const double (*x)[W], double (&acc)[W]) {
+  const unsigned lanes = __activemask();
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    if (!__any_sync(lanes, u < r)) break;
+    if (u < r)
+#pragma unroll
+      for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v[u]), x[u][q], acc[q]);
+  }
+}
+
 // k columns of a row on G = k / W lanes, W columns each (W = 4 or 2 with 16-byte accesses, else 1).
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
@@ -139,6 +153,94 @@ static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (n_rows + rpc - 1) / rpc;
   k_crs_cols<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, row_ptr, col, val, B, ldb, C, ldc, G, pf);
+  return cudaGetLastError();
+}
+
+// out[i] = (a, b)[i + phase], i < 4, phase < 4: four consecutive entries that straddle two aligned groups.
+template <typename T>
+__device__ __forceinline__ void realign(const T (&a)[4], const T (&b)[4], int phase, T (&out)[4]) {
+  const bool one = phase & 1, two = phase & 2;
+  T t[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const T x = i < 4 ? a[i % 4] : b[i % 4], y = i < 3 ? a[(i + 1) % 4] : b[(i + 1) % 4];
+    t[i] = one ? y : x;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) out[i] = two ? t[i + 2] : t[i];
+}
+
+// CRS_L1 on matrices of longer rows, k = W columns on the row's one lane: val and col_idx are read in
+// aligned groups of four entries (32 and 16 bytes), realigned in registers to the row's own start, so
+// that no multiply-add is issued for an entry of another row and the order of the sum is the scalar
+// kernel's.  One entry at a time, the 32 lanes of a load touch 32 lines of which each gives 8 or 4
+// bytes, and at 27 entries a row L1 loses most of them before their next use: 569 MB came from DRAM for
+// 330 MB of matrix.  Now every sector is used by the load that fetches it.  On a 27-point stencil of
+// 999,900 rows 131.0 -> 78.5 us (HBM floor 50, FP64 floor 42): the gathers' latency at 40 warps
+// per SM bounds it (FP64 pipe 60 %, DRAM 54 % busy).  Staging a warp's 32 rows in shared memory instead
+// (one bulk copy) took 75 us, but 248 against 93 us at 32 entries a row, where the lanes meet in one
+// bank, and rows of 60 entries left 8 warps on an SM.  An L2 prefetch of the CTAs ahead slows it
+// (77.7 -> 100 us), and so does a second group in flight (48 -> 59 registers: 79.2 us).
+template <typename VT, int W>
+__global__ void __launch_bounds__(kThreads, (W == 4 ? 3 : 5))
+    k_crs_wide(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+               int64_t ldc) {
+  const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (g >= n_rows) return;
+  const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
+  double acc[W];
+#pragma unroll
+  for (int q = 0; q < W; ++q) acc[q] = 0.0;
+  const int phase = rs & 3;
+  // the next four entries straddle the aligned groups a and b (a group is read only if it holds an
+  // entry of the row)
+  VT va[4] = {}, vb[4] = {};
+  int32_t ca[4] = {}, cb[4] = {};
+  int at = rs & ~3;
+  if (at < re) {
+    ldg4(val + at, va);
+    ldg4(col + at, ca);
+  }
+  for (int n = re - rs; n > 0; n -= 4) {
+    at += 4;
+    if (at < re) {
+      ldg4(col + at, cb);
+      ldg4(val + at, vb);
+    }
+    VT v[4];
+    int32_t c[4];
+    realign(ca, cb, phase, c);
+    double x[4][W];
+    if (n >= 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) load_cols(B + (int64_t)c[u] * ldb, x[u]);
+      realign(va, vb, phase, v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v[u]), x[u][q], acc[q]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (u < n) load_cols(B + (int64_t)c[u] * ldb, x[u]);
+      realign(va, vb, phase, v);
+      add_tail(n, v, x, acc);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      va[u] = vb[u];
+      ca[u] = cb[u];
+    }
+  }
+  store_cols(C + g * ldc, acc);
+}
+
+template <typename VT, int W>
+static cudaError_t launch_wide(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
+                               cudaStream_t s) {
+  const int64_t grid = (A.n_rows + kThreads - 1) / kThreads;
+  k_crs_wide<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc);
   return cudaGetLastError();
 }
 
@@ -321,6 +423,12 @@ static cudaError_t crs_dispatch(const CsrDev& A, int lanes, const VT* val, const
       case 2: return launch_long<VT, 2>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
       default: return launch_long<VT, 1>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
     }
+  }
+  if (lanes == 1 && A.nnz >= kWideRow * A.n_rows && A.n_rows > 0) {
+    const int w = cols_per_lane(k, B, ldb, C, ldc);
+    if (k == 1) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
+    if (w == k && A.nnz >= kWideRowCols * A.n_rows)
+      return k == 2 ? launch_wide<VT, 2>(A, val, B, ldb, C, ldc, s) : launch_wide<VT, 4>(A, val, B, ldb, C, ldc, s);
   }
   return lanes_dispatch<VT>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, val, B, ldb, C, ldc, k, false, A.prefetch, s);
 }

@@ -29,12 +29,17 @@ struct LongRows {
   int n_cta = 0, n_warp = 0;
 };
 
+// CRS_L1 reads the rows in aligned groups of four entries from this many entries per row on average
+// (kWideRowCols for blocks of two or four columns).
+constexpr int64_t kWideRow = 8;
+constexpr int64_t kWideRowCols = 16;
+
 // Device view of one CRS matrix (values in FP64 and, optionally, FP32).
 struct CsrDev {
   int64_t n_rows = 0, n_cols = 0, nnz = 0;
   const int32_t* row_ptr = nullptr;
   const int32_t* col = nullptr;     // padded to a multiple of 4 entries + 4
-  const double* val = nullptr;      // padded to a multiple of 2 entries + 2
+  const double* val = nullptr;      // padded to a multiple of 4 entries + 4
   const float* val32 = nullptr;     // padded to a multiple of 4 entries + 4
   const uint32_t* blk = nullptr;    // row blocks of CRS_STAGED (n_blk + 1 entries)
   int64_t n_blk = 0;
