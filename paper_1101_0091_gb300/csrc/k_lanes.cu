@@ -119,6 +119,49 @@ __device__ __forceinline__ void add_tail(int r, const VT* v, const double (*x)[W
   }
 }
 
+// CRS_L1, one vector: thread per row, four entries at a time (their gathers in flight together), then
+// the last 0..3.  Padding each row's last batch of eight (FP32 values: four) with masked multiply-adds
+// cost what it padded: 280^3 Poisson (7 entries a row) 326.5 -> 323.2 us (HBM-bound), with FP32 values
+// 303.9 -> 272.4 us; 1500^2 Laplacian 39.0 -> 33.2 us; 3,000,000 rows of 5 entries 48.9 -> 41.1 us.  The
+// two pipes together bound it: 7 multiply-adds per row are 0.74 of the HBM time at 280^3, with FP32
+// values 0.99 of it.
+template <typename VT, bool UNIT>  // UNIT: ldb = 1 (its multiplication and two registers saved)
+__global__ void __launch_bounds__(kThreads, 8)
+    k_crs_row(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+              const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+              int64_t ldc, int prefetch) {
+  if (threadIdx.x == 0 && prefetch > 0)
+    prefetch_rows(((int64_t)blockIdx.x + prefetch) * kThreads, kThreads, n_rows, row_ptr, col, val);
+  const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (g >= n_rows) return;
+  int j = __ldg(row_ptr + g);
+  const int re = __ldg(row_ptr + g + 1);
+  double acc[1] = {0.0};
+  for (; j + 4 <= re; j += 4) {
+    const VT* vj = val + j;
+    const int32_t* cj = col + j;
+    double v[4], x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = to_f64(ldg(vj + u));
+      x[u] = __ldg(UNIT ? B + ldg(cj + u) : B + (int64_t)ldg(cj + u) * ldb);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[0] = fma(v[u], x[u], acc[0]);
+  }
+  double v[3], x[3][1];
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    v[u] = x[u][0] = 0.0;
+    if (j + u < re) {
+      v[u] = to_f64(ldg(val + j + u));
+      x[u][0] = __ldg(UNIT ? B + ldg(col + j + u) : B + (int64_t)ldg(col + j + u) * ldb);
+    }
+  }
+  add_tail(re - j, v, x, acc);
+  C[g * ldc] = acc[0];
+}
+
 // k columns of a row on G = k / W lanes, W columns each (W = 4 or 2 with 16-byte accesses, else 1).
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
@@ -383,6 +426,14 @@ static cudaError_t lanes_k(int64_t n, const int32_t* rows, const int32_t* rp, co
                            const double* B, int64_t ldb, double* C, int64_t ldc, int k, bool acc,
                            int pf, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
+  if constexpr (L == 1) {
+    if (k == 1 && !rows) {
+      const int64_t grid = (n + kThreads - 1) / kThreads;
+      (ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>)<<<(unsigned)grid, kThreads, 0, s>>>(
+          n, rp, col, val, B, ldb, C, ldc, pf);
+      return cudaGetLastError();
+    }
+  }
   if (k <= 1) return launch_lanes_t<VT, L, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
   if constexpr (L == 1) {  // k >= 2 never comes with a row list (the halo pass has k = 1)
     switch (cols_per_lane(k, B, ldb, C, ldc)) {
