@@ -49,23 +49,24 @@ __global__ void __launch_bounds__(kThreads)
   const int len = __ldg(chunk_len + c);
   const int64_t base = __ldg(chunk_ptr + c) + t;
   double acc = 0.0;
-  // batches of NB slots: all gathers of a batch are issued before its FMAs
+  // batches of NB slots: all gathers of a batch are issued before its FMAs (len is the warp's, so
+  // the last slots take a branch, not masked multiply-adds)
   constexpr int NB = 2;
-  for (int j = 0; j < len; j += NB) {
-    double v[NB];
-    const double* b[NB];
+  int j = 0;
+  for (; j + NB <= len; j += NB) {
+    double v[NB], g[NB];
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const int64_t slot = base + (int64_t)((j + u < len) ? j + u : j) * kSellC;
+      const int64_t slot = base + (int64_t)(j + u) * kSellC;
       v[u] = to_f64(ldcs(val + slot));
-      b[u] = B + (int64_t)ldcs(col + slot) * ldb;
+      g[u] = __ldg(B + (int64_t)ldcs(col + slot) * ldb);
     }
-    double g[NB];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) g[u] = j + u < len ? __ldg(b[u]) : 0.0;
-#pragma unroll
-    for (int u = 0; u < NB; ++u)
-      if (j + u < len) acc = fma(v[u], g[u], acc);
+    for (int u = 0; u < NB; ++u) acc = fma(v[u], g[u], acc);
+  }
+  for (; j < len; ++j) {
+    const int64_t slot = base + (int64_t)j * kSellC;
+    acc = fma(to_f64(ldcs(val + slot)), __ldg(B + (int64_t)ldcs(col + slot) * ldb), acc);
   }
   if (r >= n_rows) return;
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
