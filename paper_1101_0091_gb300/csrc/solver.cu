@@ -5,15 +5,15 @@
 // dominates).
 //
 // Vectors are row-major n x k blocks (ld = k, 16-byte aligned: the vector
-// kernels move 16 bytes per access).  The vector work of an iteration is a few
-// fused grid-stride kernels on a grid of one wave; each reduces
-// its per-column inner products to one partial per CTA, and the CTA that
-// finishes last (threadfence + ticket, no waiting) adds the partials in a
-// fixed order and updates the per-column scalars in device memory.  Reductions are
+// kernels move 16 bytes per access).  The vector work of an iteration is three
+// fused grid-stride kernels on a grid of at most one wave; each writes
+// its per-column inner products as one partial per CTA, and every CTA of the kernel
+// that uses them adds the partials again in a fixed order.  Reductions are
 // therefore deterministic for a given solver.  Columns freeze on the device the
 // iteration they converge (or break down), so the host only polls a counter
 // every `check_every` iterations; those iterations are replayed from a CUDA
 // graph captured once per (B, X, check_every).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -23,46 +23,56 @@
 
 namespace spmv {
 
-constexpr int kSolverCtasPerSm = 8;  // upper limit; the occupancy of the update kernel decides
+constexpr int kVecCtasPerSm = 2;  // CTAs of the vector kernels per SM (their launch bounds hold them resident)
 constexpr int kMaxCols = 16;
 
+// Per-column scalars.  Every CTA of a kernel reads them and CTA 0 writes, so no kernel writes a field
+// that it reads: k_cg_direction writes rr, active, iters and n_active, k_cg_update the others, with
+// copies (rr_old) or working sets (running) of what k_cg_direction needs; in the Lanczos kernels
+// k_lz_scale writes live_next and b_prev, k_lz_alpha live.
 struct CgScalars {
-  double rr[kMaxCols], tol2[kMaxCols], alpha[kMaxCols], beta[kMaxCols];
-  int active[kMaxCols], next_active[kMaxCols], iters[kMaxCols], breakdown[kMaxCols];
+  double rr[kMaxCols], rr_old[kMaxCols], tol2[kMaxCols], alpha[kMaxCols];
+  int active[kMaxCols], running[kMaxCols], iters[kMaxCols], breakdown[kMaxCols];
   int n_active;
 };
 
 struct LzScalars {
-  double b_prev[kMaxCols], inv_b[kMaxCols], alpha[kMaxCols];
-  int live[kMaxCols];
+  double b_prev[kMaxCols];
+  int live[kMaxCols], live_next[kMaxCols];
 };
 
 // ---------------------------------------------------------------- block walking
-// How a thread walks a row-major n x k block, one unit per grid-stride step:
+// How the threads of a kernel walk a row-major n x k block, one unit per thread and grid stride:
 //  PAIRS (k = 1): two consecutive entries, one 16-byte access;
 //  VROWS (k = K = 2, 4): one row of K values, K/2 16-byte accesses;
-//  VGROUPS (k = K = 8, 16): a group of 4 columns of one row (K/4 units per
-//    row), two 16-byte accesses; a thread keeps 4 accumulators instead of K,
-//    which keeps these kernels at several CTAs per SM;
-//  ROWS (other k): one row, k scalar accesses (K >= k, masked).
-// PAIRS, VROWS and VGROUPS need 16-byte aligned blocks (checked on the host).
-enum { ROWS = 0, VROWS = 1, PAIRS = 2, VGROUPS = 3 };
+//  VGROUPS (k = K = 8, 16): a group of 4 columns of one row (K/4 units per row), two 16-byte accesses;
+//  FLAT (other k): one entry; the largest multiple of k threads of a CTA take part, so that a thread
+//    stays on its column and a warp reads consecutive entries.
+// In every mode the stride keeps a thread on the same columns.  PAIRS, VROWS and VGROUPS need 16-byte
+// aligned blocks (checked on the host).
+enum { FLAT = 0, VROWS = 1, PAIRS = 2, VGROUPS = 3 };
+
+constexpr int kVecThreads = 512;  // threads per CTA of the vector kernels
 
 template <int K, int MODE>
 struct Seg {
-  static constexpr int NG = MODE == VGROUPS ? K / 4 : 1;                    // units per row
-  static constexpr int W = MODE == PAIRS ? 2 : (MODE == VGROUPS ? 4 : K);  // values per unit
-  static constexpr int KC = MODE == PAIRS ? 1 : W;                         // accumulators per thread
-  static constexpr int KP = MODE == PAIRS ? 1 : K;                         // columns of the sums
-  static_assert(kThreads % NG == 0, "a thread's units must share one column group");
-  __device__ static int64_t units(int64_t n) { return MODE == PAIRS ? (n + 1) / 2 : n * NG; }
-  // accumulator of value w, and the block column it belongs to in unit u
-  __device__ static int acol(int w) { return MODE == PAIRS ? 0 : w; }
-  __device__ static int gcol(int64_t u, int w) {
-    return MODE == PAIRS ? 0 : (MODE == VGROUPS ? (int)(u % NG) * 4 + w : w);
+  static constexpr int NG = MODE == VGROUPS ? K / 4 : 1;                                        // units per row
+  static constexpr int W = MODE == FLAT ? 1 : MODE == PAIRS ? 2 : (MODE == VGROUPS ? 4 : K);  // values per unit
+  static constexpr int KC = MODE == PAIRS ? 1 : W;                // accumulators (columns) per thread
+  static constexpr int KP = MODE == FLAT ? kMaxCols : (MODE == PAIRS ? 1 : K);  // columns at most
+  static constexpr int U = MODE == FLAT ? 4 : (W == 2 ? 2 : 1);   // units in flight per thread and vector
+  static_assert(kVecThreads % NG == 0, "a thread's units must share one column group");
+  // units of an n x k block, threads of a CTA that take part, first column of thread t
+  __host__ __device__ static int64_t units(int64_t n, int k) {
+    return MODE == FLAT ? n * k : MODE == PAIRS ? (n + 1) / 2 : n * NG;
   }
-  __device__ static void load(const double* p, int64_t u, int64_t n, int k, double (&v)[W]) {
-    if (MODE == PAIRS) {
+  __host__ __device__ static int threads(int k) { return MODE == FLAT ? kVecThreads / k * k : kVecThreads; }
+  __device__ static int column(int t, int k) { return MODE == FLAT ? t % k : MODE == VGROUPS ? (t % NG) * 4 : 0; }
+  __device__ static int acc(int w) { return MODE == PAIRS ? 0 : w; }  // accumulator of value w
+  __device__ static void load(const double* p, int64_t u, int64_t n, double (&v)[W]) {
+    if constexpr (MODE == FLAT) {
+      v[0] = p[u];
+    } else if constexpr (MODE == PAIRS) {
       if (2 * u + 1 < n) {
         const double2 t = reinterpret_cast<const double2*>(p)[u];
         v[0] = t.x;
@@ -71,7 +81,7 @@ struct Seg {
         v[0] = p[2 * u];
         v[1] = 0.0;
       }
-    } else if (MODE == VROWS || MODE == VGROUPS) {
+    } else {
       // VGROUPS: u * 4 is the offset of group u % NG of row u / NG
 #pragma unroll
       for (int h = 0; h < W / 2; ++h) {
@@ -79,409 +89,494 @@ struct Seg {
         v[2 * h] = t.x;
         v[2 * h + 1] = t.y;
       }
-    } else {
-#pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = w < k ? p[u * k + w] : 0.0;
     }
   }
-  __device__ static void store(double* p, int64_t u, int64_t n, int k, const double (&v)[W]) {
-    if (MODE == PAIRS) {
+  __device__ static void store(double* p, int64_t u, int64_t n, const double (&v)[W]) {
+    if constexpr (MODE == FLAT) {
+      p[u] = v[0];
+    } else if constexpr (MODE == PAIRS) {
       if (2 * u + 1 < n)
         reinterpret_cast<double2*>(p)[u] = make_double2(v[0], v[1]);
       else
         p[2 * u] = v[0];
-    } else if (MODE == VROWS || MODE == VGROUPS) {
-#pragma unroll
-      for (int h = 0; h < W / 2; ++h) reinterpret_cast<double2*>(p + u * W)[h] = make_double2(v[2 * h], v[2 * h + 1]);
     } else {
 #pragma unroll
-      for (int w = 0; w < W; ++w)
-        if (w < k) p[u * k + w] = v[w];
+      for (int h = 0; h < W / 2; ++h) reinterpret_cast<double2*>(p + u * W)[h] = make_double2(v[2 * h], v[2 * h + 1]);
     }
   }
 };
 
+// The walk of one thread: U units per step, all loads of a step before its arithmetic and stores.
+template <typename G>
+struct Walk {
+  int64_t u, stride, units, n;
+  __device__ Walk(int64_t n_, int k) : n(n_) {
+    const int t = G::threads(k);
+    units = (int)threadIdx.x < t ? G::units(n, k) : 0;
+    stride = (int64_t)gridDim.x * t;
+    u = (int64_t)blockIdx.x * t + threadIdx.x;
+  }
+  __device__ bool more() const { return u < units; }
+  __device__ bool has(int j) const { return j == 0 || u + j * stride < units; }  // of a step that more() allows
+  __device__ void next() { u += stride * G::U; }
+  __device__ void load(const double* p, double (&v)[G::U][G::W]) const {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (u + j * stride < units) {
+        G::load(p, u + j * stride, n, v[j]);
+      } else {
+#pragma unroll
+        for (int w = 0; w < G::W; ++w) v[j][w] = 0.0;
+      }
+    }
+  }
+  __device__ void store(double* p, const double (&v)[G::U][G::W]) const {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j)
+      if (has(j)) G::store(p, u + j * stride, n, v[j]);
+  }
+};
+
 // ---------------------------------------------------------------- reductions
-// Per-column sums over a CTA and then over the CTAs, in a fixed order (so a
-// solver's results do not depend on timing).
+// Per-column sums over a CTA and then over the CTAs, in a fixed order (so a solver's results do not
+// depend on timing).  No CTA waits to be the last: each writes its column sums (a partial), and every
+// CTA of the kernel that needs the totals adds all partials again in the same order.  A warp's FP64 add
+// occupies the SM for 16 cycles whatever it adds, so the sums go through shared memory in passes that
+// keep 32 lanes busy; an xor-shuffle tree per warp and column spent as many cycles on the sums as on the
+// vectors' arithmetic (320 against 66 warp adds for 512 threads and four columns).
+struct VecShared {
+  double sums[kVecThreads * 4], part[128];
+};
 
-// Writes this CTA's NS x KP column sums of the threads' accumulators
-// (G::KC per thread: thread t holds the columns of group t % G::NG, or all
-// of them), then returns true in the CTA that finished last (all partials
-// visible to it).  Order: xor-shuffle tree within each warp, then warps in
-// order.
-template <typename G, int NS>
-__device__ bool publish_partials(double (&acc)[NS][G::KC], double* partial, uint32_t* counter, int k) {
-  constexpr int KP = G::KP, KC = G::KC, R = G::NG;  // R lanes of a warp hold distinct column sets
-  __shared__ double sh[kThreads / 32][KP];
-  __shared__ bool last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-#pragma unroll
-    for (int w = 0; w < KC; ++w)
-#pragma unroll
-      for (int off = 16; off >= R; off >>= 1) acc[s][w] += __shfl_xor_sync(0xffffffffu, acc[s][w], off);
-    if (lane < R)
-#pragma unroll
-      for (int w = 0; w < KC; ++w) sh[warp][lane * KC + w] = acc[s][w];
-    __syncthreads();
-    if (threadIdx.x < KP && threadIdx.x < k) {
-      double t = 0.0;
-#pragma unroll
-      for (int v = 0; v < kThreads / 32; ++v) t += sh[v][threadIdx.x];
-      partial[((size_t)blockIdx.x * NS + s) * kMaxCols + threadIdx.x] = t;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  }
+// Thread c < period gets the sum of the values of column c among the N values in sh.sums, value i
+// belonging to column i % period.  (period = KP, a power of two, or in FLAT mode k; N <= 2048.)
+template <typename G>
+__device__ __forceinline__ double column_sum(VecShared& sh, int N, int k) {
+  const int t = threadIdx.x;
   __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-
-// In the last CTA (all threads): the sums of the CTAs' partials, per sum s
-// and column q, into tot[s][q].  Thread t takes column t % KP and adds the
-// partials of CTAs t / KP, t / KP + 256 / KP, ... in order; the threads of a
-// column are then combined by an xor-shuffle tree and the warps in order.
-template <int KP, int NS>
-__device__ void finish_partials(const double* partial, int k, double (&tot)[NS][KP]) {
-  constexpr int SL = kThreads / KP;  // threads per column
-  __shared__ double sh[kThreads / 32][KP];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int q = threadIdx.x % KP;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    double x = 0.0;
-    if (q < k)
-      for (unsigned b = threadIdx.x / KP; b < gridDim.x; b += SL)
-        x += __ldcg(partial + ((size_t)b * NS + s) * kMaxCols + q);
-#pragma unroll
-    for (int off = 16; off >= KP; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-    if (lane < KP) sh[warp][lane] = x;
-    __syncthreads();
-    if (threadIdx.x < KP) {
-      double t = 0.0;
-#pragma unroll
-      for (int v = 0; v < kThreads / 32; ++v) t += sh[v][threadIdx.x];
-      tot[s][threadIdx.x] = t;
+  double x = 0.0;
+  if constexpr (G::KP == kMaxCols && G::KC == 1 && G::W == 1) {  // FLAT
+    const int r1 = 128 / k * k, r2 = 32 / k * k;
+    if (t < r1) {
+      for (int i = t; i < N; i += r1) x += sh.sums[i];
+      sh.part[t] = x;
     }
     __syncthreads();
+    if (t < 32) {
+      x = 0.0;
+      if (t < r2)
+        for (int i = t; i < r1; i += r2) x += sh.part[i];
+      __syncwarp();
+      sh.part[t] = x;
+      __syncwarp();
+      x = 0.0;
+      if (t < k)
+        for (int i = t; i < r2; i += k) x += sh.part[i];
+    }
+  } else {
+    if (t < 128) {
+      x = sh.sums[t];
+      for (int i = t + 128; i < N; i += 128) x += sh.sums[i];
+      sh.part[t] = x;
+    }
+    __syncthreads();
+    if (t < 32) {
+      x = (sh.part[t] + sh.part[t + 32]) + (sh.part[t + 64] + sh.part[t + 96]);
+#pragma unroll
+      for (int off = 16; off >= G::KP; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    }
   }
+  return x;
 }
 
-#define UNIT_LOOP(u, n) \
-  for (int64_t u = (int64_t)blockIdx.x * kThreads + threadIdx.x; u < G::units(n); u += (int64_t)gridDim.x * kThreads)
+// This CTA's column sums of the threads' accumulators, to partial[blockIdx.x * period + c].
+template <typename G>
+__device__ __forceinline__ void write_partial(const double (&acc)[G::KC], int k, double* partial, VecShared& sh) {
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < G::KC; ++w) sh.sums[threadIdx.x * G::KC + w] = acc[w];
+  const int period = G::NG * G::KC == G::KP ? G::KP : k;
+  const double x = column_sum<G>(sh, G::threads(k) * G::KC, k);
+  if ((int)threadIdx.x < period) partial[(size_t)blockIdx.x * period + threadIdx.x] = x;
+}
+
+// Thread c < period gets the total of column c over n_partials partials.
+template <typename G>
+__device__ __forceinline__ double read_partials(const double* partial, unsigned n_partials, int k, VecShared& sh) {
+  const int period = G::NG * G::KC == G::KP ? G::KP : k;
+  const unsigned step = G::threads(k), count = n_partials * period;
+  double x = 0.0;
+  if (threadIdx.x < step) {
+    unsigned i = threadIdx.x;
+    for (; i + 3 * step < count; i += 4 * step) {
+      double v[4];
+#pragma unroll
+      for (unsigned j = 0; j < 4; ++j) v[j] = __ldcg(partial + i + j * step);
+      x += (v[0] + v[1]) + (v[2] + v[3]);
+    }
+    for (; i < count; i += step) x += __ldcg(partial + i);
+  }
+  sh.sums[threadIdx.x] = x;
+  return column_sum<G>(sh, step, k);
+}
 
 // ---------------------------------------------------------------- CG kernels
-// R = B - AX (AX in Q), P = R; rr = R.R, tol2 = rtol^2 B.B, active = rr > tol2.
+// R = B - AX (AX in Q), P = R; column sums of R.R and B.B.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_cg_init(int64_t n, int k, const double* __restrict__ B,
-                                                      const double* __restrict__ Q, double* R, double* P,
-                                                      double* partial, uint32_t* counter, CgScalars* S,
-                                                      double rtol2) {
+__global__ void __launch_bounds__(kVecThreads) k_cg_init(int64_t n, int k, const double* __restrict__ B,
+                                                         const double* __restrict__ Q, double* __restrict__ R,
+                                                         double* __restrict__ P, double* rr_partial,
+                                                         double* bb_partial) {
   using G = Seg<K, MODE>;
-  double acc[2][G::KC];
+  __shared__ VecShared sh;
+  double rr[G::KC], bb[G::KC];
 #pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = acc[1][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double b[G::W], r[G::W];
-    G::load(B, u, n, k, b);
-    G::load(Q, u, n, k, r);
+  for (int q = 0; q < G::KC; ++q) rr[q] = bb[q] = 0.0;
+  for (Walk<G> w(n, k); w.more(); w.next()) {
+    double b[G::U][G::W], r[G::U][G::W];
+    w.load(B, b);
+    w.load(Q, r);
 #pragma unroll
-    for (int w = 0; w < G::W; ++w) {
-      r[w] = b[w] - r[w];
-      acc[0][G::acol(w)] = fma(r[w], r[w], acc[0][G::acol(w)]);
-      acc[1][G::acol(w)] = fma(b[w], b[w], acc[1][G::acol(w)]);
-    }
-    G::store(R, u, n, k, r);
-    G::store(P, u, n, k, r);
-  }
-  if (!publish_partials<G, 2>(acc, partial, counter, k)) return;
-  __shared__ double tot[2][G::KP];
-  finish_partials<G::KP, 2>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    const double rr = tot[0][q], bb = tot[1][q];
-    S->rr[q] = rr;
-    S->tol2[q] = rtol2 * bb;
-    S->active[q] = rr > rtol2 * bb;
-    S->iters[q] = 0;
-    S->breakdown[q] = 0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int na = 0;
-    for (int q = 0; q < k; ++q) na += S->active[q];
-    S->n_active = na;
-    *counter = 0;
-  }
-}
-
-// pq = P.Q; active columns: alpha = rr / pq, or breakdown when pq <= 0.
-template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_cg_alpha(int64_t n, int k, const double* __restrict__ P,
-                                                       const double* __restrict__ Q, double* partial,
-                                                       uint32_t* counter, CgScalars* S) {
-  using G = Seg<K, MODE>;
-  double acc[1][G::KC];
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
 #pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double p[G::W], q2[G::W];
-    G::load(P, u, n, k, p);
-    G::load(Q, u, n, k, q2);
-#pragma unroll
-    for (int w = 0; w < G::W; ++w) acc[0][G::acol(w)] = fma(p[w], q2[w], acc[0][G::acol(w)]);
-  }
-  if (!publish_partials<G, 1>(acc, partial, counter, k)) return;
-  __shared__ double tot[1][G::KP];
-  finish_partials<G::KP, 1>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    const double pq = tot[0][q];
-    if (S->active[q] && !(pq > 0.0)) {
-      S->breakdown[q] = 1;
-      S->active[q] = 0;
-    }
-    S->alpha[q] = S->active[q] ? S->rr[q] / pq : 0.0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *counter = 0;
-}
-
-// Active columns: X += alpha P, R -= alpha Q; rr' = R.R, beta = rr' / rr.
-// (Inactive columns are written back unchanged.)
-template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_cg_update(int64_t n, int k, double* X, double* R,
-                                                        const double* __restrict__ P, const double* __restrict__ Q,
-                                                        double* partial, uint32_t* counter, CgScalars* S) {
-  using G = Seg<K, MODE>;
-  __shared__ double s_alpha[G::KP];
-  __shared__ int s_active[G::KP];
-  if (threadIdx.x < G::KP) {
-    s_alpha[threadIdx.x] = threadIdx.x < k ? S->alpha[threadIdx.x] : 0.0;
-    s_active[threadIdx.x] = threadIdx.x < k ? S->active[threadIdx.x] : 0;
-  }
-  __syncthreads();
-  double acc[1][G::KC];
-#pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double x[G::W], r[G::W], p[G::W], q2[G::W];
-    G::load(X, u, n, k, x);
-    G::load(R, u, n, k, r);
-    G::load(P, u, n, k, p);
-    G::load(Q, u, n, k, q2);
-#pragma unroll
-    for (int w = 0; w < G::W; ++w) {
-      const int c = G::gcol(u, w);
-      if (s_active[c]) {
-        x[w] = fma(s_alpha[c], p[w], x[w]);
-        r[w] = fma(-s_alpha[c], q2[w], r[w]);
+      for (int i = 0; i < G::W; ++i) {
+        r[j][i] = b[j][i] - r[j][i];
+        rr[G::acc(i)] = fma(r[j][i], r[j][i], rr[G::acc(i)]);
+        bb[G::acc(i)] = fma(b[j][i], b[j][i], bb[G::acc(i)]);
       }
-      acc[0][G::acol(w)] = fma(r[w], r[w], acc[0][G::acol(w)]);
     }
-    G::store(X, u, n, k, x);
-    G::store(R, u, n, k, r);
+    w.store(R, r);
+    w.store(P, r);
   }
-  if (!publish_partials<G, 1>(acc, partial, counter, k)) return;
-  __shared__ double tot[1][G::KP];
-  finish_partials<G::KP, 1>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    if (S->active[q]) {
-      const double rr = tot[0][q];
-      S->beta[q] = rr / S->rr[q];
-      S->rr[q] = rr;
-      S->iters[q] += 1;
-      S->next_active[q] = rr > S->tol2[q];
-    } else {
-      S->beta[q] = 0.0;
-      S->next_active[q] = 0;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *counter = 0;
+  write_partial<G>(rr, k, rr_partial, sh);
+  write_partial<G>(bb, k, bb_partial, sh);
 }
 
-// Active columns: P = R + beta P; then the columns that met the tolerance stop.
+// One CTA: the scalars of the start, tol2 = rtol^2 B.B, active = rr > tol2.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_cg_direction(int64_t n, int k, const double* __restrict__ R,
-                                                           double* P, uint32_t* counter, CgScalars* S) {
+__global__ void __launch_bounds__(kVecThreads) k_cg_begin(int k, const double* rr_partial, const double* bb_partial,
+                                                          unsigned n_partials, CgScalars* S, double rtol2) {
   using G = Seg<K, MODE>;
-  __shared__ double s_beta[G::KP];
-  __shared__ int s_active[G::KP];
-  __shared__ bool last;
-  if (threadIdx.x < G::KP) {
-    s_beta[threadIdx.x] = threadIdx.x < k ? S->beta[threadIdx.x] : 0.0;
-    s_active[threadIdx.x] = threadIdx.x < k ? S->active[threadIdx.x] : 0;
+  __shared__ VecShared sh;
+  __shared__ int n_active;
+  const int c = threadIdx.x;
+  if (c == 0) n_active = 0;
+  const double rr = read_partials<G>(rr_partial, n_partials, k, sh);
+  __syncthreads();
+  const double bb = read_partials<G>(bb_partial, n_partials, k, sh);
+  if (c < k) {
+    S->rr[c] = rr;
+    S->tol2[c] = rtol2 * bb;
+    S->active[c] = rr > rtol2 * bb;
+    S->iters[c] = 0;
+    S->breakdown[c] = 0;
+    if (rr > rtol2 * bb) atomicAdd(&n_active, 1);
   }
   __syncthreads();
-  UNIT_LOOP(u, n) {
-    double r[G::W], p[G::W];
-    G::load(R, u, n, k, r);
-    G::load(P, u, n, k, p);
+  if (c == 0) S->n_active = n_active;
+}
+
+// Column sums of P.Q.
+template <int K, int MODE>
+__global__ void __launch_bounds__(kVecThreads, 2) k_cg_dot(int64_t n, int k, const double* __restrict__ P,
+                                                           const double* __restrict__ Q, double* partial) {
+  using G = Seg<K, MODE>;
+  __shared__ VecShared sh;
+  double acc[G::KC];
 #pragma unroll
-    for (int w = 0; w < G::W; ++w)
-      if (s_active[G::gcol(u, w)]) p[w] = fma(s_beta[G::gcol(u, w)], p[w], r[w]);
-    G::store(P, u, n, k, p);
+  for (int q = 0; q < G::KC; ++q) acc[q] = 0.0;
+  for (Walk<G> w(n, k); w.more(); w.next()) {
+    double p[G::U][G::W], q2[G::U][G::W];
+    w.load(P, p);
+    w.load(Q, q2);
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) acc[G::acc(i)] = fma(p[j][i], q2[j][i], acc[G::acc(i)]);
+    }
+  }
+  write_partial<G>(acc, k, partial, sh);
+}
+
+// alpha = R.R / P.Q (breakdown when P.Q <= 0); running columns: R -= alpha Q; column sums of R.R.  (The
+// first step's loads are issued before the scalars are known; so in the kernels below.)
+template <int K, int MODE>
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_cg_update(int64_t n, int k, double* __restrict__ R, const double* __restrict__ Q, const double* pq_partial,
+                double* rr_partial, CgScalars* S) {
+  using G = Seg<K, MODE>;
+  __shared__ VecShared sh;
+  __shared__ double s_alpha[kMaxCols];
+  __shared__ int s_run[kMaxCols];
+  Walk<G> w(n, k);
+  double r[G::U][G::W], q2[G::U][G::W];
+  w.load(R, r);
+  w.load(Q, q2);
+  const double pq = read_partials<G>(pq_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) {
+    const int active = S->active[c], run = active && pq > 0.0;
+    const double rr = S->rr[c];
+    s_run[c] = run;
+    s_alpha[c] = run ? rr / pq : 0.0;
+    if (blockIdx.x == 0) {
+      if (active && !run) S->breakdown[c] = 1;
+      S->running[c] = run;
+      S->alpha[c] = s_alpha[c];
+      S->rr_old[c] = rr;
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  double alpha[G::KC], acc[G::KC];
+  bool run[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
+#pragma unroll
+  for (int q = 0; q < G::KC; ++q) {
+    alpha[q] = s_alpha[c0 + q];
+    run[q] = s_run[c0 + q];
+    acc[q] = 0.0;
+  }
+  while (w.more()) {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) {
+        const int q = G::acc(i);
+        const double x = fma(-alpha[q], q2[j][i], r[j][i]);  // (a select: a branch issued both sides' multiply-adds)
+        r[j][i] = run[q] ? x : r[j][i];
+        acc[q] = fma(r[j][i], r[j][i], acc[q]);
+      }
+    }
+    w.store(R, r);
+    w.next();
+    w.load(R, r);
+    w.load(Q, q2);
+  }
+  write_partial<G>(acc, k, rr_partial, sh);
+}
+
+// beta = R.R(new) / R.R(old); running columns: X += alpha P, P = R + beta P; then the columns that met
+// the tolerance stop.  (X is updated here, where P is read anyway.)
+template <int K, int MODE>
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_cg_direction(int64_t n, int k, double* __restrict__ X, const double* __restrict__ R, double* __restrict__ P,
+                   const double* rr_partial, CgScalars* S) {
+  using G = Seg<K, MODE>;
+  __shared__ VecShared sh;
+  __shared__ double s_alpha[kMaxCols], s_beta[kMaxCols];
+  __shared__ int s_run[kMaxCols], s_next[kMaxCols];
+  Walk<G> w(n, k);
+  double x[G::U][G::W], r[G::U][G::W], p[G::U][G::W];
+  w.load(X, x);
+  w.load(R, r);
+  w.load(P, p);
+  const double rr = read_partials<G>(rr_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) {
+    const int run = S->running[c];
+    s_run[c] = run;
+    s_alpha[c] = S->alpha[c];
+    s_beta[c] = run ? rr / S->rr_old[c] : 0.0;
+    s_next[c] = run && rr > S->tol2[c];
+    if (blockIdx.x == 0) {
+      if (run) {
+        S->rr[c] = rr;
+        S->iters[c] += 1;
+      }
+      S->active[c] = s_next[c];
+    }
   }
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  int na = 0;
-  for (int q = 0; q < k; ++q) {
-    S->active[q] = S->active[q] && S->next_active[q];
-    na += S->active[q];
+  if (blockIdx.x == 0 && c == 0) {
+    int na = 0;
+    for (int q = 0; q < k; ++q) na += s_next[q];
+    S->n_active = na;
   }
-  S->n_active = na;
-  *counter = 0;
+  double alpha[G::KC], beta[G::KC];
+  bool run[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
+#pragma unroll
+  for (int q = 0; q < G::KC; ++q) {
+    alpha[q] = s_alpha[c0 + q];
+    beta[q] = s_beta[c0 + q];
+    run[q] = s_run[c0 + q];
+  }
+  while (w.more()) {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) {
+        const int q = G::acc(i);
+        const double xn = fma(alpha[q], p[j][i], x[j][i]), pn = fma(beta[q], p[j][i], r[j][i]);
+        x[j][i] = run[q] ? xn : x[j][i];
+        p[j][i] = run[q] ? pn : p[j][i];
+      }
+    }
+    w.store(X, x);
+    w.store(P, p);
+    w.next();
+    w.load(X, x);
+    w.load(R, r);
+    w.load(P, p);
+  }
 }
 
 // ---------------------------------------------------------------- Lanczos kernels
-// |V0| per column; live = |V0| > 0; inv_b = 1 / |V0| (consumed by k_lz_scale).
+// Column sums of V0.V0.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_lz_norm(int64_t n, int k, const double* __restrict__ V0,
-                                                      double* partial, uint32_t* counter, LzScalars* S) {
+__global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, const double* __restrict__ V0,
+                                                            double* partial) {
   using G = Seg<K, MODE>;
-  double acc[1][G::KC];
+  __shared__ VecShared sh;
+  double acc[G::KC];
 #pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double v[G::W];
-    G::load(V0, u, n, k, v);
+  for (int q = 0; q < G::KC; ++q) acc[q] = 0.0;
+  for (Walk<G> w(n, k); w.more(); w.next()) {
+    double v[G::U][G::W];
+    w.load(V0, v);
 #pragma unroll
-    for (int w = 0; w < G::W; ++w) acc[0][G::acol(w)] = fma(v[w], v[w], acc[0][G::acol(w)]);
-  }
-  if (!publish_partials<G, 1>(acc, partial, counter, k)) return;
-  __shared__ double tot[1][G::KP];
-  finish_partials<G::KP, 1>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    const double b = sqrt(tot[0][q]);
-    S->live[q] = b > 0.0;
-    S->b_prev[q] = b;
-    S->inv_b[q] = b > 0.0 ? 1.0 / b : 0.0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *counter = 0;
-}
-
-// dst = live ? src * (1 / beta) : 0 (one FP64 division per column, in the
-// reducing CTA, instead of one per entry); zero_out (if given) = 0.
-template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_lz_scale(int64_t n, int k, const double* __restrict__ src,
-                                                       double* dst, double* zero_out, const LzScalars* S) {
-  using G = Seg<K, MODE>;
-  __shared__ double s_b[G::KP];
-  __shared__ int s_live[G::KP];
-  if (threadIdx.x < G::KP) {
-    s_b[threadIdx.x] = threadIdx.x < k ? S->inv_b[threadIdx.x] : 0.0;
-    s_live[threadIdx.x] = threadIdx.x < k ? S->live[threadIdx.x] : 0;
-  }
-  __syncthreads();
-  UNIT_LOOP(u, n) {
-    double v[G::W];
-    G::load(src, u, n, k, v);
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
 #pragma unroll
-    for (int w = 0; w < G::W; ++w) v[w] = s_live[G::gcol(u, w)] ? v[w] * s_b[G::gcol(u, w)] : 0.0;
-    G::store(dst, u, n, k, v);
-    if (zero_out) {
-#pragma unroll
-      for (int w = 0; w < G::W; ++w) v[w] = 0.0;
-      G::store(zero_out, u, n, k, v);
+      for (int i = 0; i < G::W; ++i) acc[G::acc(i)] = fma(v[j][i], v[j][i], acc[G::acc(i)]);
     }
   }
+  write_partial<G>(acc, k, partial, sh);
 }
 
-// W = W - b_prev v_prev; alpha = W.v (live columns), stored to alpha_out.
+// W = W - b_prev v_prev; column sums of W.v.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_lz_alpha(int64_t n, int k, double* W, const double* __restrict__ v,
-                                                       const double* __restrict__ v_prev, double* partial,
-                                                       uint32_t* counter, LzScalars* S, double* alpha_out) {
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_lz_alpha(int64_t n, int k, double* __restrict__ W, const double* __restrict__ v,
+               const double* __restrict__ v_prev, double* partial, LzScalars* S) {
   using G = Seg<K, MODE>;
-  __shared__ double s_b[G::KP];
-  if (threadIdx.x < G::KP) s_b[threadIdx.x] = threadIdx.x < k ? S->b_prev[threadIdx.x] : 0.0;
-  __syncthreads();
-  double acc[1][G::KC];
+  __shared__ VecShared sh;
+  if (blockIdx.x == 0 && (int)threadIdx.x < k) S->live[threadIdx.x] = S->live_next[threadIdx.x];
+  double b[G::KC], acc[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
 #pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double w_[G::W], vv[G::W], vp[G::W];
-    G::load(W, u, n, k, w_);
-    G::load(v, u, n, k, vv);
-    G::load(v_prev, u, n, k, vp);
+  for (int q = 0; q < G::KC; ++q) {
+    b[q] = S->b_prev[c0 + q];
+    acc[q] = 0.0;
+  }
+  for (Walk<G> w(n, k); w.more(); w.next()) {
+    double x[G::U][G::W], vv[G::U][G::W], vp[G::U][G::W];
+    w.load(W, x);
+    w.load(v, vv);
+    w.load(v_prev, vp);
 #pragma unroll
-    for (int w = 0; w < G::W; ++w) {
-      w_[w] = fma(-s_b[G::gcol(u, w)], vp[w], w_[w]);
-      acc[0][G::acol(w)] = fma(w_[w], vv[w], acc[0][G::acol(w)]);
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) {
+        const int q = G::acc(i);
+        x[j][i] = fma(-b[q], vp[j][i], x[j][i]);
+        acc[q] = fma(x[j][i], vv[j][i], acc[q]);
+      }
     }
-    G::store(W, u, n, k, w_);
+    w.store(W, x);
   }
-  if (!publish_partials<G, 1>(acc, partial, counter, k)) return;
-  __shared__ double tot[1][G::KP];
-  finish_partials<G::KP, 1>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    const double a = S->live[q] ? tot[0][q] : 0.0;
-    S->alpha[q] = a;
-    alpha_out[q] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *counter = 0;
+  write_partial<G>(acc, k, partial, sh);
 }
 
-// W = W - alpha v; beta = |W| (live columns), stored to beta_out; a column
-// whose beta is 0 stops.
+// alpha = W.v (live columns), stored to alpha_out; W = W - alpha v; column sums of W.W.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kThreads) k_lz_beta(int64_t n, int k, double* W, const double* __restrict__ v,
-                                                      double* partial, uint32_t* counter, LzScalars* S,
-                                                      double* beta_out) {
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_lz_beta(int64_t n, int k, double* __restrict__ W, const double* __restrict__ v, const double* a_partial,
+              double* b_partial, const LzScalars* S, double* alpha_out) {
   using G = Seg<K, MODE>;
-  __shared__ double s_a[G::KP];
-  if (threadIdx.x < G::KP) s_a[threadIdx.x] = threadIdx.x < k ? S->alpha[threadIdx.x] : 0.0;
+  __shared__ VecShared sh;
+  __shared__ double s_a[kMaxCols];
+  Walk<G> w(n, k);
+  double x[G::U][G::W], vv[G::U][G::W];
+  w.load(W, x);
+  w.load(v, vv);
+  const double wv = read_partials<G>(a_partial, gridDim.x, k, sh);
+  if ((int)threadIdx.x < k) {
+    s_a[threadIdx.x] = S->live_next[threadIdx.x] ? wv : 0.0;
+    if (blockIdx.x == 0) alpha_out[threadIdx.x] = s_a[threadIdx.x];
+  }
   __syncthreads();
-  double acc[1][G::KC];
+  double a[G::KC], acc[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
 #pragma unroll
-  for (int q = 0; q < G::KC; ++q) acc[0][q] = 0.0;
-  UNIT_LOOP(u, n) {
-    double w_[G::W], vv[G::W];
-    G::load(W, u, n, k, w_);
-    G::load(v, u, n, k, vv);
+  for (int q = 0; q < G::KC; ++q) {
+    a[q] = s_a[c0 + q];
+    acc[q] = 0.0;
+  }
+  while (w.more()) {
 #pragma unroll
-    for (int w = 0; w < G::W; ++w) {
-      w_[w] = fma(-s_a[G::gcol(u, w)], vv[w], w_[w]);
-      acc[0][G::acol(w)] = fma(w_[w], w_[w], acc[0][G::acol(w)]);
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) {
+        const int q = G::acc(i);
+        x[j][i] = fma(-a[q], vv[j][i], x[j][i]);
+        acc[q] = fma(x[j][i], x[j][i], acc[q]);
+      }
     }
-    G::store(W, u, n, k, w_);
+    w.store(W, x);
+    w.next();
+    w.load(W, x);
+    w.load(v, vv);
   }
-  if (!publish_partials<G, 1>(acc, partial, counter, k)) return;
-  __shared__ double tot[1][G::KP];
-  finish_partials<G::KP, 1>(partial, k, tot);
-  if (threadIdx.x < k) {
-    const int q = threadIdx.x;
-    const double b = S->live[q] ? sqrt(tot[0][q]) : 0.0;
-    beta_out[q] = b;
-    S->live[q] = S->live[q] && b > 0.0;
-    S->b_prev[q] = S->live[q] ? b : 0.0;
-    S->inv_b[q] = S->live[q] ? 1.0 / b : 0.0;
+  write_partial<G>(acc, k, b_partial, sh);
+}
+
+// beta = |W| (live columns), stored to beta_out; v_next = W / beta (one FP64 division per column
+// instead of one per entry); a column whose beta is 0 stops.  FIRST (W = V0): every column is live
+// before, and the previous vector's coefficient is 0.
+template <int K, int MODE, bool FIRST>
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_lz_scale(int64_t n, int k, const double* __restrict__ W, double* __restrict__ v_next, const double* b_partial,
+               LzScalars* S, double* beta_out) {
+  using G = Seg<K, MODE>;
+  __shared__ VecShared sh;
+  __shared__ double s_inv[kMaxCols];
+  __shared__ int s_live[kMaxCols];
+  Walk<G> w(n, k);
+  double x[G::U][G::W];
+  w.load(W, x);
+  const double ww = read_partials<G>(b_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) {
+    const double b = FIRST || S->live[c] ? sqrt(ww) : 0.0;
+    const bool live = b > 0.0;
+    s_live[c] = live;
+    s_inv[c] = live ? 1.0 / b : 0.0;
+    if (blockIdx.x == 0) {
+      if (!FIRST) beta_out[c] = b;
+      S->live_next[c] = live;
+      S->b_prev[c] = !FIRST && live ? b : 0.0;
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) *counter = 0;
+  double inv[G::KC];
+  bool live[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
+#pragma unroll
+  for (int q = 0; q < G::KC; ++q) {
+    inv[q] = s_inv[c0 + q];
+    live[q] = s_live[c0 + q];
+  }
+  while (w.more()) {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) x[j][i] = live[G::acc(i)] ? x[j][i] * inv[G::acc(i)] : 0.0;
+    }
+    w.store(v_next, x);
+    w.next();
+    w.load(W, x);
+  }
 }
-#undef UNIT_LOOP
 
 // ---------------------------------------------------------------- dispatch
-// k = 1 -> pairs; k = 2, 4 -> vector rows; k = 8, 16 -> 4-column groups;
-// other k -> scalar rows.
 template <template <int, int> class F, typename... Args>
 static cudaError_t by_k(int k, Args... args) {
   switch (k) {
@@ -490,49 +585,39 @@ static cudaError_t by_k(int k, Args... args) {
     case 4: return F<4, VROWS>::run(args...);
     case 8: return F<8, VGROUPS>::run(args...);
     case 16: return F<16, VGROUPS>::run(args...);
-    default: break;
+    default: return F<1, FLAT>::run(args...);
   }
-  if (k <= 4) return F<4, ROWS>::run(args...);
-  if (k <= 8) return F<8, ROWS>::run(args...);
-  return F<16, ROWS>::run(args...);
 }
 
-#define SOLVER_LAUNCHER(NAME, KERNEL)                                \
+#define SOLVER_LAUNCHER(NAME, ...)                                   \
   template <int K, int MODE>                                         \
   struct NAME {                                                      \
     template <typename... A>                                         \
     static cudaError_t run(unsigned grid, cudaStream_t s, A... a) { \
-      KERNEL<K, MODE><<<grid, kThreads, 0, s>>>(a...);               \
+      __VA_ARGS__<<<grid, kVecThreads, 0, s>>>(a...);                \
       return cudaGetLastError();                                     \
     }                                                                \
   };
-SOLVER_LAUNCHER(LCgInit, k_cg_init)
-SOLVER_LAUNCHER(LCgAlpha, k_cg_alpha)
-SOLVER_LAUNCHER(LCgUpdate, k_cg_update)
-SOLVER_LAUNCHER(LCgDirection, k_cg_direction)
-SOLVER_LAUNCHER(LLzNorm, k_lz_norm)
-SOLVER_LAUNCHER(LLzScale, k_lz_scale)
-SOLVER_LAUNCHER(LLzAlpha, k_lz_alpha)
-SOLVER_LAUNCHER(LLzBeta, k_lz_beta)
+SOLVER_LAUNCHER(LCgInit, k_cg_init<K, MODE>)
+SOLVER_LAUNCHER(LCgBegin, k_cg_begin<K, MODE>)
+SOLVER_LAUNCHER(LCgDot, k_cg_dot<K, MODE>)
+SOLVER_LAUNCHER(LCgUpdate, k_cg_update<K, MODE>)
+SOLVER_LAUNCHER(LCgDirection, k_cg_direction<K, MODE>)
+SOLVER_LAUNCHER(LLzNorm, k_lz_norm<K, MODE>)
+SOLVER_LAUNCHER(LLzFirst, k_lz_scale<K, MODE, true>)
+SOLVER_LAUNCHER(LLzAlpha, k_lz_alpha<K, MODE>)
+SOLVER_LAUNCHER(LLzBeta, k_lz_beta<K, MODE>)
+SOLVER_LAUNCHER(LLzScale, k_lz_scale<K, MODE, false>)
 #undef SOLVER_LAUNCHER
 
-// Resident CTAs per SM of each vector kernel (the CG kernels come first,
-// then the Lanczos ones, four each).
-enum { KI_CG_INIT = 0, KI_CG_ALPHA, KI_CG_UPDATE, KI_CG_DIRECTION, KI_LZ_NORM, KI_LZ_SCALE, KI_LZ_ALPHA,
-       KI_LZ_BETA, KI_COUNT };
-
+// CTAs of the vector kernels on an n x k block: enough for its units, at most `most`.
 template <int K, int MODE>
-struct LOccupancy {
-  static cudaError_t run(int* o) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 0, k_cg_init<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 1, k_cg_alpha<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 2, k_cg_update<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 3, k_cg_direction<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 4, k_lz_norm<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 5, k_lz_scale<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 6, k_lz_alpha<K, MODE>, kThreads, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(o + 7, k_lz_beta<K, MODE>, kThreads, 0);
-    return e;
+struct LGrid {
+  static cudaError_t run(int64_t n, int k, int64_t most, unsigned* grid) {
+    using G = Seg<K, MODE>;
+    const int64_t per_cta = G::threads(k);
+    *grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((G::units(n, k) + per_cta - 1) / per_cta, most));
+    return cudaSuccess;
   }
 };
 
@@ -544,10 +629,9 @@ struct spmv_solver {
   spmv_handle A = nullptr;
   int device = 0, k = 0;
   int64_t n = 0;
-  unsigned grid[KI_COUNT] = {};    // one-wave grid of each vector kernel
+  unsigned grid = 1;               // CTAs of the vector kernels (one wave at most)
   double *buf[3] = {nullptr, nullptr, nullptr};  // CG: R, P, Q; Lanczos: v_prev, v, W
-  double* partial = nullptr;
-  uint32_t* counter = nullptr;
+  double *partial = nullptr, *partial2 = nullptr;  // column sums per CTA (two, one read while the other is written)
   CgScalars* cg = nullptr;
   LzScalars* lz = nullptr;
   double* lz_out = nullptr;        // alpha[m][16], beta[m][16] on the device
@@ -566,7 +650,7 @@ static void solver_free(spmv_solver* s) {
   if (s->graph) cudaGraphExecDestroy(s->graph);
   for (double* b : s->buf) if (b) cudaFree(b);
   if (s->partial) cudaFree(s->partial);
-  if (s->counter) cudaFree(s->counter);
+  if (s->partial2) cudaFree(s->partial2);
   if (s->cg) cudaFree(s->cg);
   if (s->lz) cudaFree(s->lz);
   if (s->lz_out) cudaFree(s->lz_out);
@@ -588,18 +672,17 @@ struct SolverDeviceGuard {
   }
 };
 
-// One CG iteration on stream s: Q = A P, then alpha, the X/R update and the new direction.
+// One CG iteration on stream s: Q = A P, then P.Q, the R update, and X with the new direction.
 spmv_status cg_iteration(spmv_solver* S, double* X, cudaStream_t s) {
   double *R = S->buf[0], *P = S->buf[1], *Q = S->buf[2];
   spmv_status st = spmv_apply_block(S->A, P, S->k, S->k, Q, S->k, s);
   if (st != SPMV_OK) return st;
-  cudaError_t e = by_k<LCgAlpha>(S->k, S->grid[KI_CG_ALPHA], s, S->n, S->k, (const double*)P, (const double*)Q,
-                                 S->partial, S->counter, S->cg);
+  cudaError_t e = by_k<LCgDot>(S->k, S->grid, s, S->n, S->k, (const double*)P, (const double*)Q, S->partial);
   if (e == cudaSuccess)
-    e = by_k<LCgUpdate>(S->k, S->grid[KI_CG_UPDATE], s, S->n, S->k, X, R, (const double*)P, (const double*)Q,
-                        S->partial, S->counter, S->cg);
+    e = by_k<LCgUpdate>(S->k, S->grid, s, S->n, S->k, R, (const double*)Q, (const double*)S->partial, S->partial2,
+                        S->cg);
   if (e == cudaSuccess)
-    e = by_k<LCgDirection>(S->k, S->grid[KI_CG_DIRECTION], s, S->n, S->k, (const double*)R, P, S->counter, S->cg);
+    e = by_k<LCgDirection>(S->k, S->grid, s, S->n, S->k, X, (const double*)R, P, (const double*)S->partial2, S->cg);
   return e == cudaSuccess ? SPMV_OK : cuda_fail(e, "CG kernel launch");
 }
 }  // namespace
@@ -623,27 +706,12 @@ spmv_status spmv_solver_create(spmv_handle A, int32_t k, spmv_solver_handle* out
   SolverDeviceGuard g(S->device);
   int sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S->device);
-  // The kernels of one method (CG: 4, Lanczos: 4) share the one-wave grid of the
-  // heaviest of them (measured: 1-2 % faster iterations at k >= 4 than a grid per
-  // kernel, and 2 % faster at k = 1 than one grid for all 8 kernels).
-  int per_sm[KI_COUNT] = {};
-  if (e == cudaSuccess) e = by_k<LOccupancy>(k, per_sm);
-  const int64_t want = (S->n + kThreads - 1) / kThreads;
-  unsigned max_grid = 1;
-  for (int m0 = 0; m0 < KI_COUNT; m0 += 4) {
-    int r = kSolverCtasPerSm;
-    for (int i = m0; i < m0 + 4; ++i) r = per_sm[i] < r ? per_sm[i] : r;
-    r = r < 1 ? 1 : r;
-    const int64_t cap = (int64_t)(sms > 0 ? sms : 1) * r;
-    const unsigned g = (unsigned)(want < 1 ? 1 : (want < cap ? want : cap));
-    for (int i = m0; i < m0 + 4; ++i) S->grid[i] = g;
-    max_grid = g > max_grid ? g : max_grid;
-  }
+  if (e == cudaSuccess)
+    e = by_k<LGrid>(k, S->n, k, (int64_t)(sms > 0 ? sms : 1) * kVecCtasPerSm, &S->grid);
   const size_t vec = sizeof(double) * (size_t)(S->n > 0 ? S->n : 1) * (size_t)k;
   for (int b = 0; b < 3 && e == cudaSuccess; ++b) e = cudaMalloc(&S->buf[b], vec);
-  if (e == cudaSuccess) e = cudaMalloc(&S->partial, sizeof(double) * max_grid * 2 * kMaxCols);
-  if (e == cudaSuccess) e = cudaMalloc(&S->counter, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(S->counter, 0, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&S->partial, sizeof(double) * S->grid * kMaxCols);
+  if (e == cudaSuccess) e = cudaMalloc(&S->partial2, sizeof(double) * S->grid * kMaxCols);
   if (e == cudaSuccess) e = cudaMalloc(&S->cg, sizeof(CgScalars));
   if (e == cudaSuccess) e = cudaMemset(S->cg, 0, sizeof(CgScalars));
   if (e == cudaSuccess) e = cudaMalloc(&S->lz, sizeof(LzScalars));
@@ -685,8 +753,11 @@ spmv_status spmv_cg_solve(spmv_solver_handle S, const double* B_dev, double* X_d
     // R = B - A X0, P = R, scalars
     spmv_status st = spmv_apply_block(S->A, X_dev, S->k, S->k, S->buf[2], S->k, s);
     if (st != SPMV_OK) return st;
-    cudaError_t e = by_k<LCgInit>(S->k, S->grid[KI_CG_INIT], s, S->n, S->k, B_dev, (const double*)S->buf[2],
-                                  S->buf[0], S->buf[1], S->partial, S->counter, S->cg, rtol * rtol);
+    cudaError_t e = by_k<LCgInit>(S->k, S->grid, s, S->n, S->k, B_dev, (const double*)S->buf[2], S->buf[0], S->buf[1],
+                                  S->partial, S->partial2);
+    if (e == cudaSuccess)
+      e = by_k<LCgBegin>(S->k, 1u, s, S->k, (const double*)S->partial, (const double*)S->partial2, S->grid, S->cg,
+                         rtol * rtol);
     if (e != cudaSuccess) return cuda_fail(e, "CG init launch");
     const int steps = check_every < max_iter ? check_every : (max_iter > 0 ? max_iter : 1);
     const uint64_t gen = plan_generation(S->A);
@@ -777,23 +848,22 @@ spmv_status spmv_lanczos(spmv_solver_handle S, const double* V0_dev, int32_t m, 
   double* a_out = S->lz_out;
   double* b_out = S->lz_out + (size_t)m * kMaxCols;
   double *v_prev = S->buf[0], *v = S->buf[1], *W = S->buf[2];
-  cudaError_t e = by_k<LLzNorm>(k, S->grid[KI_LZ_NORM], s, S->n, k, V0_dev, S->partial, S->counter, S->lz);
+  cudaError_t e = by_k<LLzNorm>(k, S->grid, s, S->n, k, V0_dev, S->partial);
   if (e == cudaSuccess)
-    e = by_k<LLzScale>(k, S->grid[KI_LZ_SCALE], s, S->n, k, V0_dev, v, v_prev, (const LzScalars*)S->lz);
-  if (e == cudaSuccess) e = cudaMemsetAsync(S->lz->b_prev, 0, sizeof(double) * kMaxCols, s);
+    e = by_k<LLzFirst>(k, S->grid, s, S->n, k, V0_dev, v, (const double*)S->partial, S->lz, (double*)nullptr);
+  if (e == cudaSuccess) e = cudaMemsetAsync(v_prev, 0, sizeof(double) * (size_t)S->n * (size_t)k, s);
   if (e != cudaSuccess) return cuda_fail(e, "Lanczos start");
   for (int j = 0; j < m; ++j) {
     spmv_status st = spmv_apply_block(S->A, v, k, k, W, k, s);
     if (st != SPMV_OK) return st;
-    e = by_k<LLzAlpha>(k, S->grid[KI_LZ_ALPHA], s, S->n, k, W, (const double*)v, (const double*)v_prev, S->partial,
-                       S->counter, S->lz, a_out + (size_t)j * kMaxCols);
+    e = by_k<LLzAlpha>(k, S->grid, s, S->n, k, W, (const double*)v, (const double*)v_prev, S->partial, S->lz);
     if (e == cudaSuccess)
-      e = by_k<LLzBeta>(k, S->grid[KI_LZ_BETA], s, S->n, k, W, (const double*)v, S->partial, S->counter, S->lz,
-                        b_out + (size_t)j * kMaxCols);
+      e = by_k<LLzBeta>(k, S->grid, s, S->n, k, W, (const double*)v, (const double*)S->partial, S->partial2,
+                        (const LzScalars*)S->lz, a_out + (size_t)j * kMaxCols);
     // v_{j+1} = W / beta_j into the buffer of v_{j-1}, then rotate
     if (e == cudaSuccess)
-      e = by_k<LLzScale>(k, S->grid[KI_LZ_SCALE], s, S->n, k, (const double*)W, v_prev, (double*)nullptr,
-                         (const LzScalars*)S->lz);
+      e = by_k<LLzScale>(k, S->grid, s, S->n, k, (const double*)W, v_prev, (const double*)S->partial2, S->lz,
+                         b_out + (size_t)j * kMaxCols);
     if (e != cudaSuccess) return cuda_fail(e, "Lanczos kernel launch");
     double* t = v_prev;
     v_prev = v;
