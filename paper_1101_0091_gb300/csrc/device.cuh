@@ -96,6 +96,15 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// Programmatic dependent launch (launch_dependent, internal.h): grid_dependents lets the next kernel of
+// the stream be launched as soon as every CTA of this one has got here, so that its CTAs take the slots
+// that this kernel's last ones leave; grid_wait holds a kernel launched that way until the work before
+// it is complete and visible.  Before grid_wait a kernel reads its plan's own arrays only, and what
+// earlier work may have written (B, the solvers' vectors and scalars) is read with plain loads: a
+// read-only load (ld.global.nc, __ldg, const __restrict__) could be moved above the wait.
+__device__ __forceinline__ void grid_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ double to_f64(double v) { return v; }
 __device__ __forceinline__ double to_f64(float v) { return (double)v; }
 __device__ __forceinline__ double to_f64(f32n v) { return widen_f32n(v.v); }
@@ -143,15 +152,15 @@ inline int cols_per_lane(int k, const double* B, int64_t ldb, const double* C, i
   return !a16 || k % 2 ? 1 : (k % 4 ? 2 : 4);
 }
 
-// W consecutive columns of a block row: 16-byte accesses for W = 2, 4.
+// W consecutive columns of a block row: 16-byte accesses for W = 2, 4.  (Plain loads: see grid_wait.)
 template <int W>
-__device__ __forceinline__ void load_cols(const double* __restrict__ b, double (&g)[W]) {
+__device__ __forceinline__ void load_cols(const double* b, double (&g)[W]) {
   if constexpr (W == 1) {
-    g[0] = __ldg(b);
+    g[0] = *b;
   } else {
 #pragma unroll
     for (int q = 0; q < W; q += 2) {
-      const double2 x = __ldg(reinterpret_cast<const double2*>(b + q));
+      const double2 x = *reinterpret_cast<const double2*>(b + q);
       g[q] = x.x;
       g[q + 1] = x.y;
     }

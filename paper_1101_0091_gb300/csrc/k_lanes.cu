@@ -14,6 +14,7 @@
 // B row.  Each column's sum is formed in the same order whatever W is, so the bits
 // are the same.
 #include "device.cuh"
+#include "internal.h"
 
 namespace spmv {
 
@@ -128,14 +129,16 @@ __device__ __forceinline__ void add_tail(int r, const VT* v, const double (*x)[W
 template <typename VT, bool UNIT>  // UNIT: ldb = 1 (its multiplication and two registers saved)
 __global__ void __launch_bounds__(kThreads, 8)
     k_crs_row(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-              const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+              const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
               int64_t ldc, int prefetch) {
+  grid_dependents();
   if (threadIdx.x == 0 && prefetch > 0)
     prefetch_rows(((int64_t)blockIdx.x + prefetch) * kThreads, kThreads, n_rows, row_ptr, col, val);
   const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (g >= n_rows) return;
   int j = __ldg(row_ptr + g);
   const int re = __ldg(row_ptr + g + 1);
+  grid_wait();
   double acc[1] = {0.0};
   for (; j + 4 <= re; j += 4) {
     const VT* vj = val + j;
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, 8)
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       v[u] = to_f64(ldg(vj + u));
-      x[u] = __ldg(UNIT ? B + ldg(cj + u) : B + (int64_t)ldg(cj + u) * ldb);
+      x[u] = *(UNIT ? B + ldg(cj + u) : B + (int64_t)ldg(cj + u) * ldb);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) acc[0] = fma(v[u], x[u], acc[0]);
@@ -155,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     v[u] = x[u][0] = 0.0;
     if (j + u < re) {
       v[u] = to_f64(ldg(val + j + u));
-      x[u][0] = __ldg(UNIT ? B + ldg(col + j + u) : B + (int64_t)ldg(col + j + u) * ldb);
+      x[u][0] = *(UNIT ? B + ldg(col + j + u) : B + (int64_t)ldg(col + j + u) * ldb);
     }
   }
   add_tail(re - j, v, x, acc);
@@ -166,8 +169,9 @@ __global__ void __launch_bounds__(kThreads, 8)
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_crs_cols(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-               const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc, int G, int prefetch) {
+  grid_dependents();
   const int rpc = kThreads / G;  // rows per CTA
   if (threadIdx.x == 0 && prefetch > 0)
     prefetch_rows(((int64_t)blockIdx.x + prefetch) * rpc, rpc, n_rows, row_ptr, col, val);
@@ -176,6 +180,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   if (r >= rpc || g >= n_rows) return;
   const int c0 = ((int)threadIdx.x - r * G) * W;  // first column of this lane
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
+  grid_wait();
   double acc[W];
 #pragma unroll
   for (int q = 0; q < W; ++q) acc[q] = 0.0;
@@ -195,8 +200,8 @@ static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int
                                const double* B, int64_t ldb, double* C, int64_t ldc, int k, int pf, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (n_rows + rpc - 1) / rpc;
-  k_crs_cols<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, row_ptr, col, val, B, ldb, C, ldc, G, pf);
-  return cudaGetLastError();
+  return launch_dependent(k_crs_cols<VT, W>, (unsigned)grid, kThreads, s, n_rows, row_ptr, col, val, B, ldb, C, ldc, G,
+                          pf);
 }
 
 // out[i] = (a, b)[i + phase], i < 4, phase < 4: four consecutive entries that straddle two aligned groups.
@@ -227,8 +232,9 @@ __device__ __forceinline__ void realign(const T (&a)[4], const T (&b)[4], int ph
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 4 ? 3 : 5))
     k_crs_wide(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-               const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc) {
+  grid_dependents();
   const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (g >= n_rows) return;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
@@ -245,6 +251,7 @@ __global__ void __launch_bounds__(kThreads, (W == 4 ? 3 : 5))
     ldg4(val + at, va);
     ldg4(col + at, ca);
   }
+  grid_wait();
   for (int n = re - rs; n > 0; n -= 4) {
     at += 4;
     if (at < re) {
@@ -283,8 +290,8 @@ template <typename VT, int W>
 static cudaError_t launch_wide(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                                cudaStream_t s) {
   const int64_t grid = (A.n_rows + kThreads - 1) / kThreads;
-  k_crs_wide<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc);
-  return cudaGetLastError();
+  return launch_dependent(k_crs_wide<VT, W>, (unsigned)grid, kThreads, s, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
+                          ldc);
 }
 
 // One row on NT threads (a warp or the CTA; thread t of them): EP entry lanes, a power of two, times
@@ -294,12 +301,13 @@ static cudaError_t launch_wide(const CsrDev& A, const VT* val, const double* B, 
 template <typename VT, int NT>
 __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* __restrict__ row_ptr,
                                          const int32_t* __restrict__ col, const VT* __restrict__ val,
-                                         const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+                                         const double* B, int64_t ldb, double* C,
                                          int64_t ldc, double* sh) {
   const int rs = __ldg(row_ptr + row), re = __ldg(row_ptr + row + 1);
   const int ep = 1 << (31 - __clz(NT / k));
   const int e = t / k, c = t - e * k;
   double acc = 0.0;
+  grid_wait();
   if (e < ep) {
     constexpr int U = 4;  // entries in flight per lane
     for (int j = rs + e; j < re; j += U * ep) {
@@ -308,7 +316,7 @@ __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* _
       for (int u = 0; u < U; ++u) {
         const int jj = j + u * ep < re ? j + u * ep : j;
         v[u] = to_f64(ldcs(val + jj));
-        g[u] = __ldg(B + (int64_t)ldcs(col + jj) * ldb + c);
+        g[u] = B[(int64_t)ldcs(col + jj) * ldb + c];
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
@@ -333,9 +341,10 @@ __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* _
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 5))
     k_crs_long(LongRows lr, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-               const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc, int G, int prefetch) {
   __shared__ double sh[kThreads];
+  grid_dependents();
   constexpr int WARPS = kThreads / 32;
   const int tid = (int)threadIdx.x;
   int64_t blk = blockIdx.x;
@@ -360,6 +369,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 5))
   if (r >= rpc || g >= n_rows) return;
   const int c0 = (tid - r * G) * W;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
+  grid_wait();
   if (re - rs > kShortRow) return;
   double acc[W];
 #pragma unroll
@@ -398,8 +408,8 @@ static cudaError_t launch_long(const LongRows& lr, int64_t n_rows, const int32_t
                                int pf, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G, warps = kThreads / 32;
   const int64_t grid = lr.n_cta + (lr.n_warp + warps - 1) / warps + (n_rows + rpc - 1) / rpc;
-  k_crs_long<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(lr, n_rows, row_ptr, col, val, B, ldb, C, ldc, G, pf);
-  return cudaGetLastError();
+  return launch_dependent(k_crs_long<VT, W>, (unsigned)grid, kThreads, s, lr, n_rows, row_ptr, col, val, B, ldb, C, ldc,
+                          G, pf);
 }
 
 template <typename VT, int L, int K>
@@ -429,9 +439,8 @@ static cudaError_t lanes_k(int64_t n, const int32_t* rows, const int32_t* rp, co
   if constexpr (L == 1) {
     if (k == 1 && !rows) {
       const int64_t grid = (n + kThreads - 1) / kThreads;
-      (ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>)<<<(unsigned)grid, kThreads, 0, s>>>(
-          n, rp, col, val, B, ldb, C, ldc, pf);
-      return cudaGetLastError();
+      return launch_dependent(ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>, (unsigned)grid, kThreads, s, n, rp,
+                              col, val, B, ldb, C, ldc, pf);
     }
   }
   if (k <= 1) return launch_lanes_t<VT, L, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);

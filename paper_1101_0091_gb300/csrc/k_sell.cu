@@ -14,6 +14,7 @@
 // read one contiguous piece of its B row; a row's slots are still summed in
 // order, so every W gives the same bits.
 #include "device.cuh"
+#include "internal.h"
 
 namespace spmv {
 
@@ -36,8 +37,9 @@ template <typename VT>
 __global__ void __launch_bounds__(kThreads)
     k_sell(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm,
            const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
-           const int32_t* __restrict__ col, const VT* __restrict__ val, const double* __restrict__ B,
-           int64_t ldb, double* __restrict__ C, int64_t ldc, int prefetch) {
+           const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B,
+           int64_t ldb, double* C, int64_t ldc, int prefetch) {
+  grid_dependents();
   constexpr int CPC = kThreads / kSellC;  // chunks per CTA
   // bring the slots of the CTA `prefetch` positions ahead into L2
   if (threadIdx.x == 0 && prefetch > 0)
@@ -48,6 +50,7 @@ __global__ void __launch_bounds__(kThreads)
   const int t = threadIdx.x & 31;
   const int len = __ldg(chunk_len + c);
   const int64_t base = __ldg(chunk_ptr + c) + t;
+  grid_wait();
   double acc = 0.0;
   // batches of NB slots: all gathers of a batch are issued before its FMAs (len is the warp's, so
   // the last slots take a branch, not masked multiply-adds)
@@ -59,14 +62,14 @@ __global__ void __launch_bounds__(kThreads)
     for (int u = 0; u < NB; ++u) {
       const int64_t slot = base + (int64_t)(j + u) * kSellC;
       v[u] = to_f64(ldcs(val + slot));
-      g[u] = __ldg(B + (int64_t)ldcs(col + slot) * ldb);
+      g[u] = B[(int64_t)ldcs(col + slot) * ldb];
     }
 #pragma unroll
     for (int u = 0; u < NB; ++u) acc = fma(v[u], g[u], acc);
   }
   for (; j < len; ++j) {
     const int64_t slot = base + (int64_t)j * kSellC;
-    acc = fma(to_f64(ldcs(val + slot)), __ldg(B + (int64_t)ldcs(col + slot) * ldb), acc);
+    acc = fma(to_f64(ldcs(val + slot)), B[(int64_t)ldcs(col + slot) * ldb], acc);
   }
   if (r >= n_rows) return;
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
@@ -77,8 +80,9 @@ template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm,
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
-                const int32_t* __restrict__ col, const VT* __restrict__ val, const double* __restrict__ B,
-                int64_t ldb, double* __restrict__ C, int64_t ldc, int G, int prefetch) {
+                const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B,
+                int64_t ldb, double* C, int64_t ldc, int G, int prefetch) {
+  grid_dependents();
   const int rpc = kThreads / G;  // sorted rows per CTA
   if (threadIdx.x == 0 && prefetch > 0) {
     // the chunks that start in the rows of the CTA `prefetch` positions ahead
@@ -93,6 +97,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   const int c0 = ((int)threadIdx.x - rl * G) * W;  // first column of this lane
   const int len = __ldg(chunk_len + c);
   const int64_t base = __ldg(chunk_ptr + c) + (r & (kSellC - 1));
+  grid_wait();
   double acc[W];
 #pragma unroll
   for (int q = 0; q < W; ++q) acc[q] = 0.0;
@@ -113,9 +118,8 @@ static cudaError_t launch_cols(const SellDev& S, const VT* val, const double* B,
                                int k, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (S.n_rows + rpc - 1) / rpc;
-  k_sell_cols<VT, W><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len,
-                                                         S.col, val, B, ldb, C, ldc, G, S.prefetch);
-  return cudaGetLastError();
+  return launch_dependent(k_sell_cols<VT, W>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.chunk_ptr,
+                          S.chunk_len, S.col, val, B, ldb, C, ldc, G, S.prefetch);
 }
 
 template <typename VT>
@@ -130,9 +134,8 @@ static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int6
     }
   }
   const int64_t grid = (S.n_chunks * kSellC + kThreads - 1) / kThreads;
-  k_sell<VT><<<(unsigned)grid, kThreads, 0, s>>>(S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len, S.col, val,
-                                                 B, ldb, C, ldc, S.prefetch);
-  return cudaGetLastError();
+  return launch_dependent(k_sell<VT>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len,
+                          S.col, val, B, ldb, C, ldc, S.prefetch);
 }
 
 cudaError_t launch_sell(const SellDev& S, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc, int k,

@@ -223,11 +223,13 @@ __device__ __forceinline__ double read_partials(const double* partial, unsigned 
 // ---------------------------------------------------------------- CG kernels
 // R = B - AX (AX in Q), P = R; column sums of R.R and B.B.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kVecThreads) k_cg_init(int64_t n, int k, const double* __restrict__ B,
-                                                         const double* __restrict__ Q, double* __restrict__ R,
-                                                         double* __restrict__ P, double* rr_partial,
+__global__ void __launch_bounds__(kVecThreads) k_cg_init(int64_t n, int k, const double* B,
+                                                         const double* Q, double* R,
+                                                         double* P, double* rr_partial,
                                                          double* bb_partial) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   double rr[G::KC], bb[G::KC];
 #pragma unroll
@@ -258,6 +260,8 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads) k_cg_begin(int k, const double* rr_partial, const double* bb_partial,
                                                           unsigned n_partials, CgScalars* S, double rtol2) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   __shared__ int n_active;
   const int c = threadIdx.x;
@@ -279,9 +283,11 @@ __global__ void __launch_bounds__(kVecThreads) k_cg_begin(int k, const double* r
 
 // Column sums of P.Q.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kVecThreads, 2) k_cg_dot(int64_t n, int k, const double* __restrict__ P,
-                                                           const double* __restrict__ Q, double* partial) {
+__global__ void __launch_bounds__(kVecThreads, 2) k_cg_dot(int64_t n, int k, const double* P,
+                                                           const double* Q, double* partial) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   double acc[G::KC];
 #pragma unroll
@@ -304,9 +310,11 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_cg_dot(int64_t n, int k, con
 // first step's loads are issued before the scalars are known; so in the kernels below.)
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_cg_update(int64_t n, int k, double* __restrict__ R, const double* __restrict__ Q, const double* pq_partial,
+    k_cg_update(int64_t n, int k, double* R, const double* Q, const double* pq_partial,
                 double* rr_partial, CgScalars* S) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   __shared__ double s_alpha[kMaxCols];
   __shared__ int s_run[kMaxCols];
@@ -362,9 +370,11 @@ __global__ void __launch_bounds__(kVecThreads, 2)
 // the tolerance stop.  (X is updated here, where P is read anyway.)
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_cg_direction(int64_t n, int k, double* __restrict__ X, const double* __restrict__ R, double* __restrict__ P,
+    k_cg_direction(int64_t n, int k, double* X, const double* R, double* P,
                    const double* rr_partial, CgScalars* S) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   __shared__ double s_alpha[kMaxCols], s_beta[kMaxCols];
   __shared__ int s_run[kMaxCols], s_next[kMaxCols];
@@ -428,9 +438,11 @@ __global__ void __launch_bounds__(kVecThreads, 2)
 // ---------------------------------------------------------------- Lanczos kernels
 // Column sums of V0.V0.
 template <int K, int MODE>
-__global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, const double* __restrict__ V0,
+__global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, const double* V0,
                                                             double* partial) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   double acc[G::KC];
 #pragma unroll
@@ -451,9 +463,11 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, co
 // W = W - b_prev v_prev; column sums of W.v.
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_alpha(int64_t n, int k, double* __restrict__ W, const double* __restrict__ v,
-               const double* __restrict__ v_prev, double* partial, LzScalars* S) {
+    k_lz_alpha(int64_t n, int k, double* W, const double* v,
+               const double* v_prev, double* partial, LzScalars* S) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   if (blockIdx.x == 0 && (int)threadIdx.x < k) S->live[threadIdx.x] = S->live_next[threadIdx.x];
   double b[G::KC], acc[G::KC];
@@ -486,9 +500,11 @@ __global__ void __launch_bounds__(kVecThreads, 2)
 // alpha = W.v (live columns), stored to alpha_out; W = W - alpha v; column sums of W.W.
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_beta(int64_t n, int k, double* __restrict__ W, const double* __restrict__ v, const double* a_partial,
+    k_lz_beta(int64_t n, int k, double* W, const double* v, const double* a_partial,
               double* b_partial, const LzScalars* S, double* alpha_out) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   __shared__ double s_a[kMaxCols];
   Walk<G> w(n, k);
@@ -532,9 +548,11 @@ __global__ void __launch_bounds__(kVecThreads, 2)
 // before, and the previous vector's coefficient is 0.
 template <int K, int MODE, bool FIRST>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_scale(int64_t n, int k, const double* __restrict__ W, double* __restrict__ v_next, const double* b_partial,
+    k_lz_scale(int64_t n, int k, const double* W, double* v_next, const double* b_partial,
                LzScalars* S, double* beta_out) {
   using G = Seg<K, MODE>;
+  grid_dependents();
+  grid_wait();
   __shared__ VecShared sh;
   __shared__ double s_inv[kMaxCols];
   __shared__ int s_live[kMaxCols];
@@ -594,8 +612,7 @@ static cudaError_t by_k(int k, Args... args) {
   struct NAME {                                                      \
     template <typename... A>                                         \
     static cudaError_t run(unsigned grid, cudaStream_t s, A... a) { \
-      __VA_ARGS__<<<grid, kVecThreads, 0, s>>>(a...);                \
-      return cudaGetLastError();                                     \
+      return launch_dependent(__VA_ARGS__, grid, kVecThreads, s, a...); \
     }                                                                \
   };
 SOLVER_LAUNCHER(LCgInit, k_cg_init<K, MODE>)
