@@ -95,7 +95,7 @@ struct spmv_plan {
   double scattered = 0.0;
   double fill256 = 1.0;
   bool auto_sell = false;
-  LongRows long_rows;   // built on AUTO's first resolution to CRS_L1 on a matrix with long rows
+  LongRows long_rows;   // what AUTO's CRS_L1 splits off (behind row_ptr in its allocation)
   HostCsr host;
   DevArena arena;
   CsrDev A;            // the whole matrix
@@ -212,11 +212,44 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
   return SPMV_OK;
 }
 
+// The rows of more than kShortRow entries, those of more than kWarpRow first (*n_cta of them); none when
+// no row exceeds kAutoLongestRow or when they are more than kAutoLongShare of the rows.
+static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, int* n_cta) {
+  int32_t longest = 0;
+  int64_t n_long = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    const int32_t len = rp[i + 1] - rp[i];
+    longest = std::max(longest, len);
+    n_long += len > kShortRow;
+  }
+  std::vector<int32_t> list;
+  *n_cta = 0;
+  if (longest <= kAutoLongestRow || n_long > kAutoLongShare * n) return list;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int64_t i = 0; i < n; ++i) {
+      const int32_t len = rp[i + 1] - rp[i];
+      if (len > kShortRow && (len > kWarpRow) == (pass == 0)) list.push_back((int32_t)i);
+    }
+    if (pass == 0) *n_cta = (int)list.size();
+  }
+  return list;
+}
+
+// long_rows (may be NULL) receives the list of list_long_rows, uploaded behind row_ptr.
 static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n_cols, const int32_t* rp,
-                              const int32_t* col, const double* val, int64_t nnz) {
+                              const int32_t* col, const double* val, int64_t nnz, LongRows* long_rows) {
   int32_t *drp, *dcol;
   double* dval;
-  SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, 0));
+  int n_cta = 0;
+  std::vector<int32_t> list;
+  if (long_rows) list = list_long_rows(rp, n_rows, &n_cta);
+  SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, (int64_t)list.size()));
+  if (!list.empty()) {
+    SPMV_CUDA(cudaMemcpy(drp + n_rows + 1, list.data(), sizeof(int32_t) * list.size(), cudaMemcpyHostToDevice));
+    long_rows->rows = drp + n_rows + 1;
+    long_rows->n_cta = n_cta;
+    long_rows->n_warp = (int)list.size() - n_cta;
+  }
   SPMV_CUDA(upload(p->arena, &dcol, col, nnz, pad_to(nnz, 4)));
   SPMV_CUDA(upload(p->arena, &dval, val, nnz, pad_to(nnz, 4)));
   M->n_rows = n_rows;
@@ -239,13 +272,13 @@ static spmv_status build_split_dev(spmv_plan* p, int64_t h) {
   build_split(p->host, h, &p->split_host);
   const SplitHost& S = p->split_host;
   spmv_status st = upload_csr(p, &p->local, p->host.n_rows, p->host.n_cols, S.loc_row_ptr.data(),
-                              S.loc_col.data(), S.loc_val.data(), (int64_t)S.loc_col.size());
+                              S.loc_col.data(), S.loc_val.data(), (int64_t)S.loc_col.size(), nullptr);
   if (st != SPMV_OK) return st;
   st = build_blocks(p, &p->local, S.loc_row_ptr.data());
   if (st != SPMV_OK) return st;
   CsrDev hc;
   st = upload_csr(p, &hc, (int64_t)S.halo_rows.size(), p->host.n_cols, S.halo_row_ptr.data(), S.halo_col.data(),
-                  S.halo_val.data(), (int64_t)S.halo_col.size());
+                  S.halo_val.data(), (int64_t)S.halo_col.size(), nullptr);
   if (st != SPMV_OK) return st;
   int32_t* rows;
   SPMV_CUDA(upload(p->arena, &rows, S.halo_rows.data(), (int64_t)S.halo_rows.size(), 0));
@@ -292,35 +325,6 @@ static spmv_status build_sym_dev(spmv_plan* p) {
   return SPMV_OK;
 }
 
-// The rows of more than kShortRow entries; none when no row exceeds kAutoLongestRow or when they are
-// more than kAutoLongShare of the rows.
-static spmv_status build_long_rows(spmv_plan* p) {
-  if (p->long_rows.rows) return SPMV_OK;
-  const int32_t* rp = p->host.row_ptr.data();
-  const int64_t n = p->host.n_rows;
-  int32_t longest = 0;
-  int64_t n_long = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    longest = std::max(longest, rp[i + 1] - rp[i]);
-    n_long += rp[i + 1] - rp[i] > kShortRow;
-  }
-  if (longest <= kAutoLongestRow || n_long > kAutoLongShare * n) return SPMV_OK;
-  std::vector<int32_t> list, warp_rows;
-  for (int64_t i = 0; i < n; ++i) {
-    const int32_t len = rp[i + 1] - rp[i];
-    if (len > kShortRow) (len > kWarpRow ? list : warp_rows).push_back((int32_t)i);
-  }
-  LongRows lr;
-  lr.n_cta = (int)list.size();
-  lr.n_warp = (int)warp_rows.size();
-  list.insert(list.end(), warp_rows.begin(), warp_rows.end());
-  int32_t* d;
-  SPMV_CUDA(upload(p->arena, &d, list.data(), (int64_t)list.size(), 0));
-  lr.rows = d;
-  p->long_rows = lr;
-  return SPMV_OK;
-}
-
 static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
   const bool is_auto = variant == SPMV_VARIANT_AUTO;
   if (variant == SPMV_VARIANT_AUTO) {
@@ -342,13 +346,7 @@ static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
     spmv_status st = build_sym_dev(p);
     if (st != SPMV_OK) return st;
   }
-  LongRows lr;
-  if (is_auto && variant == SPMV_CRS_L1) {
-    spmv_status st = build_long_rows(p);
-    if (st != SPMV_OK) return st;
-    lr = p->long_rows;
-  }
-  p->A.long_rows = lr;
+  p->A.long_rows = is_auto ? p->long_rows : LongRows{};
   p->variant = variant;
   ++p->generation;
   return SPMV_OK;
@@ -434,7 +432,7 @@ spmv_status spmv_create(spmv_handle* out, int64_t n_rows, int64_t n_cols, int64_
     return st;
   };
   spmv_status st = upload_csr(p.get(), &p->A, n_rows, n_cols, p->host.row_ptr.data(), p->host.col.data(),
-                              p->host.val.data(), nnz);
+                              p->host.val.data(), nnz, &p->long_rows);
   if (st != SPMV_OK) return cleanup(st);
   int* status;
   e = upload(p->arena, &status, (const int*)nullptr, 0, 4);
