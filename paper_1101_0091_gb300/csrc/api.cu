@@ -195,6 +195,7 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
   p->sell.slots = S.slots;
   p->sell.sigma = sigma;
   p->sell.perm = perm;
+  p->sell.row_ptr = p->A.row_ptr;
   p->sell.chunk_ptr = cptr;
   p->sell.chunk_len = clen;
   p->sell.col = col;
@@ -212,43 +213,73 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
   return SPMV_OK;
 }
 
-// The rows of more than kShortRow entries, those of more than kWarpRow first (*n_cta of them); none when
-// no row exceeds kAutoLongestRow or when they are more than kAutoLongShare of the rows.
-static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, int* n_cta) {
+// What the choice of a CRS_L1 kernel needs of the row lengths, in one pass.
+struct RowStats {
   int32_t longest = 0;
-  int64_t n_long = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    const int32_t len = rp[i + 1] - rp[i];
-    longest = std::max(longest, len);
-    n_long += len > kShortRow;
-  }
-  std::vector<int32_t> list;
-  *n_cta = 0;
-  if (longest <= kAutoLongestRow || n_long > kAutoLongShare * n) return list;
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int64_t i = 0; i < n; ++i) {
+  int64_t n_long = 0;    // rows of more than kShortRow entries
+  int64_t slots = 0;     // 32 x the longest row of every 32 consecutive rows
+};
+static RowStats row_stats(const int32_t* rp, int64_t n) {
+  RowStats s;
+  for (int64_t r0 = 0; r0 < n; r0 += 32) {
+    const int64_t r1 = std::min(r0 + 32, n);
+    int32_t most = 0;
+    for (int64_t i = r0; i < r1; ++i) {
       const int32_t len = rp[i + 1] - rp[i];
-      if (len > kShortRow && (len > kWarpRow) == (pass == 0)) list.push_back((int32_t)i);
+      most = std::max(most, len);
+      s.n_long += len > kShortRow;
     }
-    if (pass == 0) *n_cta = (int)list.size();
+    s.longest = std::max(s.longest, most);
+    s.slots += 32 * (int64_t)most;
   }
+  return s;
+}
+
+// Columns of a block per lane: the more of them, the fewer times a row's entries are read, but the more
+// rows a warp holds and waits for the longest of.  By the share of a warp's slots that hold entries
+// (1,000,000 rows; four / two / one columns): 1.00 (3D Poisson, k = 16) 184.6 / 186.3 / 190.5 us; 0.72
+// (lengths 4 .. 9, k = 8) 147.0 / 142.3 / 175.8; 0.52 (mean 6, k = 8) 163.9 / 150.2 / 167.6; 0.15
+// (power-law up to 40, k = 4) 118.3 / 85.2 / 66.4.
+static int lane_cols(const RowStats& s, int64_t nnz) {
+  return nnz >= 0.95 * s.slots ? 4 : nnz >= 0.3 * s.slots ? 2 : 1;
+}
+
+// The rows of more than kShortRow entries, longest first (ties by row); none when no row exceeds
+// kAutoLongestRow or when they are more than kAutoLongShare of the rows.
+static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s) {
+  std::vector<int32_t> list;
+  if (s.longest <= kAutoLongestRow || s.n_long > kAutoLongShare * n) return list;
+  list.reserve((size_t)s.n_long);
+  for (int64_t i = 0; i < n; ++i)
+    if (rp[i + 1] - rp[i] > kShortRow) list.push_back((int32_t)i);
+  std::stable_sort(list.begin(), list.end(),
+                   [rp](int32_t a, int32_t b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
   return list;
 }
 
-// long_rows (may be NULL) receives the list of list_long_rows, uploaded behind row_ptr.
+// long_rows (NULL for the parts of a split, which run one vector) receives the list of list_long_rows,
+// uploaded behind row_ptr.
 static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n_cols, const int32_t* rp,
                               const int32_t* col, const double* val, int64_t nnz, LongRows* long_rows) {
   int32_t *drp, *dcol;
   double* dval;
-  int n_cta = 0;
   std::vector<int32_t> list;
-  if (long_rows) list = list_long_rows(rp, n_rows, &n_cta);
+  if (long_rows) {
+    const RowStats stats = row_stats(rp, n_rows);
+    M->lane_cols = lane_cols(stats, nnz);
+    list = list_long_rows(rp, n_rows, stats);
+  }
   SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, (int64_t)list.size()));
   if (!list.empty()) {
     SPMV_CUDA(cudaMemcpy(drp + n_rows + 1, list.data(), sizeof(int32_t) * list.size(), cudaMemcpyHostToDevice));
     long_rows->rows = drp + n_rows + 1;
-    long_rows->n_cta = n_cta;
-    long_rows->n_warp = (int)list.size() - n_cta;
+    long_rows->n = (int)list.size();
+    for (int k = 1; k <= kMaxK; ++k) {
+      const int32_t warp = list.size() >= kManyLongRows ? kWarpRow : kShortRow + kWarpRow / k;
+      long_rows->n_cta[k] = (int)(std::partition_point(list.begin(), list.end(), [&](int32_t r) {
+                                    return rp[r + 1] - rp[r] > warp;
+                                  }) - list.begin());
+    }
   }
   SPMV_CUDA(upload(p->arena, &dcol, col, nnz, pad_to(nnz, 4)));
   SPMV_CUDA(upload(p->arena, &dval, val, nnz, pad_to(nnz, 4)));

@@ -140,23 +140,40 @@ __device__ __forceinline__ void ldg4(const int32_t* p, int32_t (&x)[4]) {
   x[0] = t.x, x[1] = t.y, x[2] = t.z, x[3] = t.w;
 }
 
-// Columns per lane of the column-split kernels (k_crs_cols, k_sell_cols) for k right-hand sides: 4 or
-// 2 when k divides by it and every row of B and C starts on 16 bytes (16-byte accesses), else 1 (odd k,
-// odd leading dimensions, blocks 8 bytes off).  These products are bound by the FP64 pipe (one warp
-// FMA occupies an SM for 16 cycles), so a lane per column costs nothing that the pipe does not hide,
-// while a masked kernel of 4, 8 or 16 columns on one lane issued the masked FMAs as well.  Measured,
-// masked -> lanes: k = 3 on a 131 x 127 x 129 Poisson matrix 107.9 -> 86.3 us (FP64 floor 71); k = 6,
-// ld = 8 on a 600,011-row eigenproblem matrix 173.1 -> 111.4 us (floor 79); k = 16, ld = 17 up to 8 x.
-inline int cols_per_lane(int k, const double* B, int64_t ldb, const double* C, int64_t ldc) {
-  const bool a16 = ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0;
-  return !a16 || k % 2 ? 1 : (k % 4 ? 2 : 4);
+// Whether every row of the blocks B and C starts on 16 bytes.
+inline bool rows_on_16_bytes(const double* B, int64_t ldb, const double* C, int64_t ldc) {
+  return ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0;
 }
 
-// W consecutive columns of a block row: 16-byte accesses for W = 2, 4.  (Plain loads: see grid_wait.)
+// Columns per lane of the column-split kernels (k_crs_cols, k_sell_cols) for k right-hand sides over
+// n_rows rows: up to `even` (4 or 2; 16-byte accesses) where k divides by it and the rows start on 16
+// bytes (a16), 3, 5 or 7 in 8-byte accesses where k divides by one of those and `odd` allows it, else 1.
+// These products are bound by the FP64 pipe (a warp's FMA occupies an SM for 16 cycles), so a lane per
+// column costs little that the pipe does not hide; a masked kernel of 4, 8 or 16 columns on one lane
+// issued the masked FMAs as well (k = 3 on a 131 x 127 x 129 Poisson matrix: 107.9 us masked, 79.7 with
+// one column per lane, FP64 floor 71).  Several columns per lane read the row's entries fewer times
+// (128^3 Poisson, k = 3 / 7 / 15, one -> several: 78.5 -> 76.1, 178.7 -> 170.5, 374.1 -> 362.3 us;
+// 600,011-row eigenproblem matrix in SELL, k = 6 / 9: 114.7 -> 94.4, 173.9 -> 140.9 us) as long as the
+// threads still fill the GPU: at 60,000 rows, k = 4, four / two / one columns took 23.8 / 16.7 / 14.1 us, k = 5
+// five / one 30.7 / 13.5 us, hence kMinColThreads (the GPU holds 311,296 threads).
+constexpr int64_t kMinColThreads = 400000;
+inline int cols_per_lane(int k, bool a16, int64_t n_rows, int even, bool odd) {
+  const int even_widths[] = {4, 2}, odd_widths[] = {7, 5, 3};
+  for (int w : even_widths)
+    if (a16 && w <= even && k % w == 0 && n_rows * (k / w) >= kMinColThreads) return w;
+  if (odd && !(a16 && k % 2 == 0))
+    for (int w : odd_widths)
+      if (k % w == 0 && n_rows * (k / w) >= kMinColThreads) return w;
+  return 1;
+}
+
+// W consecutive columns of a block row: 16-byte accesses for W = 2, 4, else 8-byte ones.  (Plain loads:
+// see grid_wait.)
 template <int W>
 __device__ __forceinline__ void load_cols(const double* b, double (&g)[W]) {
-  if constexpr (W == 1) {
-    g[0] = *b;
+  if constexpr (W % 2 == 1) {
+#pragma unroll
+    for (int q = 0; q < W; ++q) g[q] = b[q];
   } else {
 #pragma unroll
     for (int q = 0; q < W; q += 2) {
@@ -168,8 +185,9 @@ __device__ __forceinline__ void load_cols(const double* b, double (&g)[W]) {
 }
 template <int W>
 __device__ __forceinline__ void store_cols(double* c, const double (&a)[W]) {
-  if constexpr (W == 1) {
-    c[0] = a[0];
+  if constexpr (W % 2 == 1) {
+#pragma unroll
+    for (int q = 0; q < W; ++q) c[q] = a[q];
   } else {
 #pragma unroll
     for (int q = 0; q < W; q += 2) reinterpret_cast<double2*>(c)[q / 2] = make_double2(a[q], a[q + 1]);

@@ -7,12 +7,13 @@
 // scalar CRS kernel.  The same kernel with a row list and accumulate = 1 is the
 // halo pass of the local/halo split: C[rows[t]] += (halo row t) * B.
 //
-// CRS_L1 on a block of k >= 2 columns runs k_crs_cols instead: the row's entries
-// still go to one lane each in order, but the k columns are split over G = k / W
-// lanes (cols_per_lane: W = 4 or 2 with 16-byte gathers and stores, W = 1 for odd
-// or unaligned blocks), and the G lanes of a row read one contiguous piece of its
-// B row.  Each column's sum is formed in the same order whatever W is, so the bits
-// are the same.
+// CRS_L1 as a plan's kernel is a family of its own (crs_l1): one vector on short rows
+// (k_crs_row) or on rows of eight and more entries on average (k_crs_wide), blocks of
+// k >= 2 columns with a row's columns split over k / W lanes (k_crs_cols), and, when
+// AUTO asks for it, a few long rows on a warp or a CTA each (k_crs_long).  Except for
+// those long rows a row's entries go to one lane in order, each column's sum is
+// formed in the same order whatever the block's width and alignment are, and the
+// bits are the same.
 #include "device.cuh"
 #include "internal.h"
 
@@ -331,85 +332,73 @@ __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* _
   if (e == 0) C[(int64_t)row * ldc + c] = acc;
 }
 
-// CRS_L1 as AUTO runs it on matrices with long rows: the listed long rows first, each on a CTA or a
-// warp, then the others as in k_crs_cols.  What bounded these products was the longest row, walked by
-// one thread with one or eight gathers in flight: a 200,000-row matrix with power-law lengths up to 2000
-// took 212.9 us at k = 1 and takes 14.4 now (k = 4, 32 entries and more per row and lane: 86 -> 32 us at
-// lengths up to 256); what is left is three dependent loads per wave and, back to back, the host's
-// launch.  A warp covers up to 512 entries in 16 steps of which four are in flight; longer rows take
-// a CTA, and both come first so that the short rows fill their tail.
-template <typename VT, int W>
-__global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 5))
-    k_crs_long(LongRows lr, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+// CRS_L1 as AUTO runs it on matrices with long rows: the listed long rows first (longest first), each on
+// a CTA or a warp, then the others with a lane per row and column.  What bounded these products was the
+// longest row, walked by one thread with one or eight gathers in flight: a 200,000-row matrix with
+// power-law lengths up to 2000 took 212.9 us at k = 1 and takes 13.1 now; what is left is three dependent
+// loads per wave and, back to back, the host's launch.  One column per lane for every k: a warp that
+// covers fewer of these uneven rows waits less for its longest (1,000,000 rows, lengths up to 500, k = 4 / 8,
+// four columns per lane 121.9 / 171.5 us, one 69.6 / 112.6).
+template <typename VT>
+__global__ void __launch_bounds__(kThreads, 8)
+    k_crs_long(const int32_t* __restrict__ long_rows, int n_long, int n_cta, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
-               int64_t ldc, int G, int prefetch) {
+               int64_t ldc, int k, int prefetch) {
   __shared__ double sh[kThreads];
   grid_dependents();
   constexpr int WARPS = kThreads / 32;
   const int tid = (int)threadIdx.x;
   int64_t blk = blockIdx.x;
-  if (blk < lr.n_cta) {
-    long_row<VT, kThreads>(__ldg(lr.rows + blk), tid, G * W, row_ptr, col, val, B, ldb, C, ldc, sh);
+  if (blk < n_cta) {
+    long_row<VT, kThreads>(__ldg(long_rows + blk), tid, k, row_ptr, col, val, B, ldb, C, ldc, sh);
     return;
   }
-  blk -= lr.n_cta;
-  const int warp_ctas = (lr.n_warp + WARPS - 1) / WARPS;
+  blk -= n_cta;
+  const int warp_ctas = (n_long - n_cta + WARPS - 1) / WARPS;
   if (blk < warp_ctas) {
-    const int i = (int)blk * WARPS + tid / 32;
-    if (i < lr.n_warp)
-      long_row<VT, 32>(__ldg(lr.rows + lr.n_cta + i), tid % 32, G * W, row_ptr, col, val, B, ldb, C, ldc,
+    const int i = n_cta + (int)blk * WARPS + tid / 32;
+    if (i < n_long)
+      long_row<VT, 32>(__ldg(long_rows + i), tid % 32, k, row_ptr, col, val, B, ldb, C, ldc,
                        sh + (tid & ~31));
     return;
   }
   blk -= warp_ctas;
-  const int rpc = kThreads / G;
+  const int rpc = kThreads / k;
   if (tid == 0 && prefetch > 0) prefetch_rows((blk + prefetch) * rpc, rpc, n_rows, row_ptr, col, val);
-  const int r = tid / G;
+  const int r = tid / k;
   const int64_t g = blk * rpc + r;
   if (r >= rpc || g >= n_rows) return;
-  const int c0 = (tid - r * G) * W;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   grid_wait();
   if (re - rs > kShortRow) return;
-  double acc[W];
-#pragma unroll
-  for (int q = 0; q < W; ++q) acc[q] = 0.0;
-  const double* Bc = B + c0;
-  // NB entries in flight, then one by one: these products are bound by the FP64 pipe on large
-  // matrices, and a batch padded with masked multiply-adds issues them (3,000,000 rows of 5 entries,
-  // k = 3: 127.5 us padded, 94.6 us so)
-  constexpr int NB = W == 4 ? 2 : 4;
+  const double* Bc = B + (tid - r * k);
+  double acc = 0.0;
+  // four entries in flight, then one by one: large matrices are bound by the FP64 pipe, and a batch
+  // padded with masked multiply-adds issues them (3,000,000 rows of 5 entries, k = 3: 127.5 us padded,
+  // 94.6 us so)
   int j = rs;
-  for (; j + NB <= re; j += NB) {
-    double v[NB], gv[NB][W];
+  for (; j + 4 <= re; j += 4) {
+    double v[4], x[4];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
+    for (int u = 0; u < 4; ++u) {
       v[u] = to_f64(ldg(val + j + u));
-      load_cols(Bc + (int64_t)ldg(col + j + u) * ldb, gv[u]);
+      x[u] = Bc[(int64_t)ldg(col + j + u) * ldb];
     }
 #pragma unroll
-    for (int u = 0; u < NB; ++u)
-#pragma unroll
-      for (int q = 0; q < W; ++q) acc[q] = fma(v[u], gv[u][q], acc[q]);
+    for (int u = 0; u < 4; ++u) acc = fma(v[u], x[u], acc);
   }
-  for (; j < re; ++j) {
-    const double v = to_f64(ldg(val + j));
-    double gv[W];
-    load_cols(Bc + (int64_t)ldg(col + j) * ldb, gv);
-#pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = fma(v, gv[q], acc[q]);
-  }
-  store_cols(C + g * ldc + c0, acc);
+  for (; j < re; ++j) acc = fma(to_f64(ldg(val + j)), Bc[(int64_t)ldg(col + j) * ldb], acc);
+  C[g * ldc + (tid - r * k)] = acc;
 }
 
-template <typename VT, int W>
-static cudaError_t launch_long(const LongRows& lr, int64_t n_rows, const int32_t* row_ptr, const int32_t* col,
-                               const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
-                               int pf, cudaStream_t s) {
-  const int G = k / W, rpc = kThreads / G, warps = kThreads / 32;
-  const int64_t grid = lr.n_cta + (lr.n_warp + warps - 1) / warps + (n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_crs_long<VT, W>, (unsigned)grid, kThreads, s, lr, n_rows, row_ptr, col, val, B, ldb, C, ldc,
-                          G, pf);
+template <typename VT>
+static cudaError_t launch_long(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
+                               int k, cudaStream_t s) {
+  const LongRows& lr = A.long_rows;
+  const int rpc = kThreads / k, warps = kThreads / 32, n_cta = lr.n_cta[k];
+  const int64_t grid = n_cta + (lr.n - n_cta + warps - 1) / warps + (A.n_rows + rpc - 1) / rpc;
+  return launch_dependent(k_crs_long<VT>, (unsigned)grid, kThreads, s, lr.rows, lr.n, n_cta, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
+                          ldc, k, A.prefetch);
 }
 
 template <typename VT, int L, int K>
@@ -436,21 +425,9 @@ static cudaError_t lanes_k(int64_t n, const int32_t* rows, const int32_t* rp, co
                            const double* B, int64_t ldb, double* C, int64_t ldc, int k, bool acc,
                            int pf, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  if constexpr (L == 1) {
-    if (k == 1 && !rows) {
-      const int64_t grid = (n + kThreads - 1) / kThreads;
-      return launch_dependent(ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>, (unsigned)grid, kThreads, s, n, rp,
-                              col, val, B, ldb, C, ldc, pf);
-    }
-  }
   if (k <= 1) return launch_lanes_t<VT, L, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  if constexpr (L == 1) {  // k >= 2 never comes with a row list (the halo pass has k = 1)
-    switch (cols_per_lane(k, B, ldb, C, ldc)) {
-      case 4: return launch_cols<VT, 4>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
-      case 2: return launch_cols<VT, 2>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
-      default: return launch_cols<VT, 1>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
-    }
-  } else {
+  if constexpr (L == 1) return cudaErrorInvalidValue;  // the halo pass only, k = 1
+  else {
     if (k <= 2) return launch_lanes_t<VT, L, 2>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
     if (k <= 4) return launch_lanes_t<VT, L, 4>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
     if (k <= 8) return launch_lanes_t<VT, L, 8>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
@@ -473,23 +450,40 @@ static cudaError_t lanes_dispatch(int lanes, int64_t n, const int32_t* rows, con
   }
 }
 
+// CRS_L1: the kernel for the plan's rows and the block's width and alignment.
+template <typename VT>
+static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
+                          cudaStream_t s) {
+  const int64_t n = A.n_rows;
+  if (n == 0) return cudaSuccess;
+  const int32_t *rp = A.row_ptr, *col = A.col;
+  const int pf = A.prefetch;
+  const bool a16 = rows_on_16_bytes(B, ldb, C, ldc);
+  if (A.long_rows.n > 0) return launch_long(A, val, B, ldb, C, ldc, k, s);
+  if (k == 1) {
+    if (A.nnz >= kWideRow * n) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
+    return launch_dependent(ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>,
+                            (unsigned)((n + kThreads - 1) / kThreads), kThreads, s, n, rp, col, val, B, ldb, C, ldc, pf);
+  }
+  const bool long_average = A.nnz >= kWideRowCols * n;
+  if (long_average && a16 && k == 2) return launch_wide<VT, 2>(A, val, B, ldb, C, ldc, s);
+  if (long_average && a16 && k == 4) return launch_wide<VT, 4>(A, val, B, ldb, C, ldc, s);
+  // (rows of 16 and more entries: one column per lane rather than 3, 5 or 7; the lanes of a row share its
+  // uncoalesced entries.  27-point stencil on 60^3, k = 3 / 5, one / several: 32.5 / 34.8, 51.4 / 54.9 us)
+  switch (cols_per_lane(k, a16, n, A.lane_cols, A.lane_cols > 1 && !long_average)) {
+    case 7: return launch_cols<VT, 7>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    case 5: return launch_cols<VT, 5>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    case 4: return launch_cols<VT, 4>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    case 3: return launch_cols<VT, 3>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    case 2: return launch_cols<VT, 2>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    default: return launch_cols<VT, 1>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+  }
+}
+
 template <typename VT>
 static cudaError_t crs_dispatch(const CsrDev& A, int lanes, const VT* val, const double* B, int64_t ldb, double* C,
                                 int64_t ldc, int k, cudaStream_t s) {
-  const LongRows& lr = A.long_rows;
-  if (lanes == 1 && lr.n_cta + lr.n_warp > 0) {
-    switch (cols_per_lane(k, B, ldb, C, ldc)) {
-      case 4: return launch_long<VT, 4>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
-      case 2: return launch_long<VT, 2>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
-      default: return launch_long<VT, 1>(lr, A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc, k, A.prefetch, s);
-    }
-  }
-  if (lanes == 1 && A.nnz >= kWideRow * A.n_rows && A.n_rows > 0) {
-    const int w = cols_per_lane(k, B, ldb, C, ldc);
-    if (k == 1) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
-    if (w == k && A.nnz >= kWideRowCols * A.n_rows)
-      return k == 2 ? launch_wide<VT, 2>(A, val, B, ldb, C, ldc, s) : launch_wide<VT, 4>(A, val, B, ldb, C, ldc, s);
-  }
+  if (lanes == 1) return crs_l1(A, val, B, ldb, C, ldc, k, s);
   return lanes_dispatch<VT>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, val, B, ldb, C, ldc, k, false, A.prefetch, s);
 }
 

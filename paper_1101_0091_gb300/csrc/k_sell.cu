@@ -12,7 +12,13 @@
 // A block of k >= 2 columns runs k_sell_cols: each sorted row is shared by
 // G = k / W lanes with W columns each (cols_per_lane), and the G lanes of a row
 // read one contiguous piece of its B row; a row's slots are still summed in
-// order, so every W gives the same bits.
+// order, so every W gives the same bits.  Here a lane stops at its row's own
+// length (from the CRS row_ptr): a warp's rows are fewer than a chunk's, and the
+// padding that they leave out is FP64 work, which bounds these products (600,011-row
+// eigenproblem matrix, k = 6: 106.3 -> 96.7 us, FP64 floor 79).  One vector is bound by
+// the SMs' requests to L2 on scattered matrices (2,000,003 rows: 95.7 us, request
+// floor 73); there the two dependent loads in front of each row cost more than
+// its padding (99.9 us).
 #include "device.cuh"
 #include "internal.h"
 
@@ -78,7 +84,7 @@ __global__ void __launch_bounds__(kThreads)
 // k columns of a sorted row on G = k / W lanes, W columns each (as k_crs_cols).
 template <typename VT, int W>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
-    k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm,
+    k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm, const int32_t* __restrict__ row_ptr,
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
                 const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B,
                 int64_t ldb, double* C, int64_t ldc, int G, int prefetch) {
@@ -95,22 +101,24 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   if (rl >= rpc || r >= n_rows) return;
   const int64_t c = r >> 5;
   const int c0 = ((int)threadIdx.x - rl * G) * W;  // first column of this lane
-  const int len = __ldg(chunk_len + c);
+  const int row = __ldg(perm + r);
+  const int len = __ldg(row_ptr + row + 1) - __ldg(row_ptr + row);
   const int64_t base = __ldg(chunk_ptr + c) + (r & (kSellC - 1));
   grid_wait();
   double acc[W];
 #pragma unroll
   for (int q = 0; q < W; ++q) acc[q] = 0.0;
   const double* Bc = B + c0;
+  const VT* vp = val + base;
+  const int32_t* cp = col + base;
   for (int j = 0; j < len; ++j) {
-    const int64_t slot = base + (int64_t)j * kSellC;
-    const double v = to_f64(ldcs(val + slot));
+    const double v = to_f64(ldcs(vp + j * kSellC));
     double g[W];
-    load_cols(Bc + (int64_t)ldcs(col + slot) * ldb, g);
+    load_cols(Bc + (int64_t)ldcs(cp + j * kSellC) * ldb, g);
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
   }
-  store_cols(C + (int64_t)__ldg(perm + r) * ldc + c0, acc);
+  store_cols(C + (int64_t)row * ldc + c0, acc);
 }
 
 template <typename VT, int W>
@@ -118,7 +126,7 @@ static cudaError_t launch_cols(const SellDev& S, const VT* val, const double* B,
                                int k, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (S.n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_sell_cols<VT, W>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.chunk_ptr,
+  return launch_dependent(k_sell_cols<VT, W>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.row_ptr, S.chunk_ptr,
                           S.chunk_len, S.col, val, B, ldb, C, ldc, G, S.prefetch);
 }
 
@@ -127,8 +135,12 @@ static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int6
                           int k, cudaStream_t s) {
   if (S.n_chunks == 0) return cudaSuccess;
   if (k > 1) {
-    switch (cols_per_lane(k, B, ldb, C, ldc)) {
-      case 4: return launch_cols<VT, 4>(S, val, B, ldb, C, ldc, k, s);
+    // two columns per lane at most: 600,011-row eigenproblem matrix, k = 4 / 8 / 16, four -> two columns 71.6 ->
+    // 66.2, 126.5 -> 120.4, 232.1 -> 227.8 us (fewer rows per warp: less is added for the chunk's padding)
+    switch (cols_per_lane(k, rows_on_16_bytes(B, ldb, C, ldc), S.n_rows, 2, true)) {
+      case 7: return launch_cols<VT, 7>(S, val, B, ldb, C, ldc, k, s);
+      case 5: return launch_cols<VT, 5>(S, val, B, ldb, C, ldc, k, s);
+      case 3: return launch_cols<VT, 3>(S, val, B, ldb, C, ldc, k, s);
       case 2: return launch_cols<VT, 2>(S, val, B, ldb, C, ldc, k, s);
       default: return launch_cols<VT, 1>(S, val, B, ldb, C, ldc, k, s);
     }

@@ -20,13 +20,19 @@ constexpr int kWarpRowsPerBlock = kThreads / 32;
 constexpr int kSellC = 32;           // SELL chunk height
 constexpr uint32_t kBlockWarpFlag = 0x80000000u;  // high bit of a row-block entry: warp-per-row block
 
-// Rows of more than kShortRow entries, for the kernel that gives them a warp or a CTA each: those of
-// more than kWarpRow entries first (n_cta of them), then the others (n_warp).
+// Rows of more than kShortRow entries, longest first, for the kernel that gives them a warp or a CTA
+// each: n_cta[k] of the n rows take a CTA.  With k right-hand sides a warp has 32 / k lanes per column,
+// so while they are few a row takes a CTA from more than kShortRow + kWarpRow / k entries on (200,000
+// power-law rows of up to 500 entries, 3,100 long ones, k = 8 / 16: 27.4 -> 23.1, 47.1 -> 32.1 us against a
+// warp up to 512 entries); kManyLongRows keep the GPU busy by themselves, and warps waste less on their sums
+// (40,000 rows of 200 entries, k = 4: 207.7 us on CTAs, 92 on warps).
 constexpr int kShortRow = 32;
 constexpr int kWarpRow = 512;
+constexpr size_t kManyLongRows = 4096;
+constexpr int kMaxK = 16;
 struct LongRows {
   const int32_t* rows = nullptr;
-  int n_cta = 0, n_warp = 0;
+  int n = 0, n_cta[kMaxK + 1] = {};
 };
 
 // CRS_L1 reads the rows in aligned groups of four entries from this many entries per row on average
@@ -46,6 +52,7 @@ struct CsrDev {
   int tile = 0;                     // nonzero capacity of a CRS_STAGED tile
   int prefetch = 0;                 // CTAs ahead whose val/col slices are prefetched into L2 (0 = off)
   bool val32_special = false;       // val32 holds a subnormal, infinite or NaN float
+  int lane_cols = 4;                // most columns of a block that a lane of CRS_L1 takes (see upload_csr)
   LongRows long_rows;               // listed (n_cta + n_warp > 0) when AUTO splits the long rows off CRS_L1
 };
 
@@ -53,6 +60,7 @@ struct SellDev {
   int64_t n_rows = 0, n_chunks = 0, slots = 0;
   int sigma = 0;
   const int32_t* perm = nullptr;
+  const int32_t* row_ptr = nullptr;  // of the CRS matrix (row lengths)
   const int64_t* chunk_ptr = nullptr;
   const int32_t* chunk_len = nullptr;
   const int32_t* col = nullptr;

@@ -41,3 +41,35 @@ def test_every_column_equals_the_vector_product(lib, k, vname, fp32):
                 assert np.array_equal(y[:, :k], want), (ldb, ldc, off)
                 assert np.all(y[:, k:] == 7.0)
         assert_close(want, A, B, f32val=fp32)
+
+
+def big(n, lo, hi, seed):
+    """n rows of lo .. hi entries (columns may repeat)."""
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(lo, hi + 1, n)
+    rp = np.zeros(n + 1, np.int32)
+    rp[1:] = np.cumsum(lens)
+    return gen.CSR(n, 5000, rp, rng.integers(0, 5000, rp[-1]).astype(np.int32), rng.uniform(-1, 1, rp[-1]))
+
+
+@pytest.mark.parametrize("vname,fp32", [("SPMV_CRS_L1", False), ("SPMV_CRS_L1", True), ("SPMV_SELL", False)])
+@pytest.mark.parametrize("lo,hi", [(3, 3), (0, 5), (17, 17)])
+def test_several_columns_per_lane_equal_the_vector_product(lib, lo, hi, vname, fp32):
+    """Enough rows for two to seven columns per lane: even rows (up to four), uneven ones (two), longer
+    ones (no 3, 5, 7 in CRS_L1), in aligned and unaligned blocks."""
+    A = big(400_013 if hi < 16 else 60_001, lo, hi, seed=hi)
+    with lib.Plan.from_csr(A, variant=getattr(lib, vname), sell_sigma=64, val_fp32=fp32) as p:
+        B = gen.rhs_block(A.n_cols, 16, seed=1)
+        want = np.empty((A.n_rows, 16))
+        for c in range(16):
+            y = block(A.n_rows, 1, 0)
+            p.apply(dev(B[:, c]), y)
+            want[:, c] = host(y)[:, 0]
+        for k in (2, 3, 4, 5, 6, 7, 8, 9, 10, 14, 15, 16):
+            for ld, off in ((k, 0), (k + 1, 0), (k, 1)):
+                Bd, C = block(A.n_cols, ld, off), block(A.n_rows, ld, off)
+                Bd[:, :k] = dev(B[:, :k])
+                p.apply_block(Bd, C, k)
+                y = host(C)
+                assert np.array_equal(y[:, :k], want[:, :k]), (k, ld, off)
+                assert np.all(y[:, k:] == 7.0)
