@@ -216,8 +216,8 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
 // What the choice of a CRS_L1 kernel needs of the row lengths, in one pass.
 struct RowStats {
   int32_t longest = 0;
-  int64_t n_long = 0;    // rows of more than kShortRow entries
-  int64_t slots = 0;     // 32 x the longest row of every 32 consecutive rows
+  int64_t n_over = 0, n_long = 0;  // rows of more than kShortRow and of more than kShortRowWide entries
+  int64_t slots = 0;               // 32 x the longest row of every 32 consecutive rows
 };
 static RowStats row_stats(const int32_t* rp, int64_t n) {
   RowStats s;
@@ -227,7 +227,8 @@ static RowStats row_stats(const int32_t* rp, int64_t n) {
     for (int64_t i = r0; i < r1; ++i) {
       const int32_t len = rp[i + 1] - rp[i];
       most = std::max(most, len);
-      s.n_long += len > kShortRow;
+      s.n_over += len > kShortRow;
+      s.n_long += len > kShortRowWide;
     }
     s.longest = std::max(s.longest, most);
     s.slots += 32 * (int64_t)most;
@@ -244,14 +245,15 @@ static int lane_cols(const RowStats& s, int64_t nnz) {
   return nnz >= 0.95 * s.slots ? 4 : nnz >= 0.3 * s.slots ? 2 : 1;
 }
 
-// The rows of more than kShortRow entries, longest first (ties by row); none when no row exceeds
-// kAutoLongestRow or when they are more than kAutoLongShare of the rows.
-static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s) {
+// The long rows (LongRows), longest first (ties by row); none when no row exceeds kAutoLongestRow or when
+// more than kAutoLongShare of the rows are long.
+static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s, int* short_row) {
   std::vector<int32_t> list;
-  if (s.longest <= kAutoLongestRow || s.n_long > kAutoLongShare * n) return list;
-  list.reserve((size_t)s.n_long);
+  const double most = kAutoLongShare * (double)n;
+  if (s.longest <= kAutoLongestRow || s.n_long > most) return list;
+  *short_row = s.n_over <= most ? kShortRow : kShortRowWide;
   for (int64_t i = 0; i < n; ++i)
-    if (rp[i + 1] - rp[i] > kShortRow) list.push_back((int32_t)i);
+    if (rp[i + 1] - rp[i] > *short_row) list.push_back((int32_t)i);
   std::stable_sort(list.begin(), list.end(),
                    [rp](int32_t a, int32_t b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
   return list;
@@ -267,7 +269,7 @@ static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n
   if (long_rows) {
     const RowStats stats = row_stats(rp, n_rows);
     M->lane_cols = lane_cols(stats, nnz);
-    list = list_long_rows(rp, n_rows, stats);
+    list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
   }
   SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, (int64_t)list.size()));
   if (!list.empty()) {
@@ -275,7 +277,7 @@ static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n
     long_rows->rows = drp + n_rows + 1;
     long_rows->n = (int)list.size();
     for (int k = 1; k <= kMaxK; ++k) {
-      const int32_t warp = list.size() >= kManyLongRows ? kWarpRow : kShortRow + kWarpRow / k;
+      const int32_t warp = list.size() >= kManyLongRows ? kWarpRow : kCtaRow + kWarpRow / k;
       long_rows->n_cta[k] = (int)(std::partition_point(list.begin(), list.end(), [&](int32_t r) {
                                     return rp[r + 1] - rp[r] > warp;
                                   }) - list.begin());

@@ -90,9 +90,9 @@ constexpr int kDefaultPrefetch = 456;
 // that format stores at least kAutoSellFill nonzeros per slot.
 constexpr double kAutoScattered = 0.3;
 constexpr double kAutoSellFill = 0.85;
-// AUTO's CRS_L1 gives the rows of more than kShortRow entries a warp or a CTA each when the longest
-// row exceeds kAutoLongestRow and they are at most kAutoLongShare of the rows; an explicit CRS_L1 keeps
-// every row on one thread.  Both sides, one thread per row -> long rows split: power-law lengths, 200,000
+// AUTO's CRS_L1 gives the long rows (LongRows, layout.h) a warp or a CTA each when the longest row
+// exceeds kAutoLongestRow and they are at most kAutoLongShare of the rows; an explicit CRS_L1 keeps
+// every row on one thread.  Both sides (rows of more than 32 entries split), one thread per row -> long rows split: power-law lengths, 200,000
 // rows, longest row 40 / 64 / 96 / 256 at k = 1: 14.5 -> 14.0 / 16.6 -> 12.6 / 20.7 -> 14.3 /
 // 39.0 -> 14.4 us (2,000,000 rows: 69.7 -> 69.0 / 82.8 -> 73.4 / 95.7 -> 74.3 / 135.6 -> 77.6).  300,000
 // banded rows of which a share has 96 entries, the others 7: share 0.1 / 0.25 / 0.5 / 1 at k = 1 57.7 ->

@@ -335,15 +335,15 @@ __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* _
 // CRS_L1 as AUTO runs it on matrices with long rows: the listed long rows first (longest first), each on
 // a CTA or a warp, then the others with a lane per row and column.  What bounded these products was the
 // longest row, walked by one thread with one or eight gathers in flight: a 200,000-row matrix with
-// power-law lengths up to 2000 took 212.9 us at k = 1 and takes 13.1 now; what is left is three dependent
-// loads per wave and, back to back, the host's launch.  One column per lane for every k: a warp that
+// power-law lengths up to 2000 took 212.9 us at k = 1 and takes 10.2 now; what is left is the dependent loads
+// of a lane's rounds and, back to back, the host's launch.  One column per lane for every k: a warp that
 // covers fewer of these uneven rows waits less for its longest (1,000,000 rows, lengths up to 500, k = 4 / 8,
 // four columns per lane 121.9 / 171.5 us, one 69.6 / 112.6).
 template <typename VT>
 __global__ void __launch_bounds__(kThreads, 8)
     k_crs_long(const int32_t* __restrict__ long_rows, int n_long, int n_cta, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
-               int64_t ldc, int k, int prefetch) {
+               int64_t ldc, int k, int short_row, int prefetch) {
   __shared__ double sh[kThreads];
   grid_dependents();
   constexpr int WARPS = kThreads / 32;
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 8)
   if (r >= rpc || g >= n_rows) return;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   grid_wait();
-  if (re - rs > kShortRow) return;
+  if (re - rs > short_row) return;
   const double* Bc = B + (tid - r * k);
   double acc = 0.0;
   // four entries in flight, then one by one: large matrices are bound by the FP64 pipe, and a batch
@@ -398,7 +398,7 @@ static cudaError_t launch_long(const CsrDev& A, const VT* val, const double* B, 
   const int rpc = kThreads / k, warps = kThreads / 32, n_cta = lr.n_cta[k];
   const int64_t grid = n_cta + (lr.n - n_cta + warps - 1) / warps + (A.n_rows + rpc - 1) / rpc;
   return launch_dependent(k_crs_long<VT>, (unsigned)grid, kThreads, s, lr.rows, lr.n, n_cta, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
-                          ldc, k, A.prefetch);
+                          ldc, k, lr.short_row, A.prefetch);
 }
 
 template <typename VT, int L, int K>

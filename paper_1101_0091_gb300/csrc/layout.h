@@ -20,19 +20,24 @@ constexpr int kWarpRowsPerBlock = kThreads / 32;
 constexpr int kSellC = 32;           // SELL chunk height
 constexpr uint32_t kBlockWarpFlag = 0x80000000u;  // high bit of a row-block entry: warp-per-row block
 
-// Rows of more than kShortRow entries, longest first, for the kernel that gives them a warp or a CTA
-// each: n_cta[k] of the n rows take a CTA.  With k right-hand sides a warp has 32 / k lanes per column,
-// so while they are few a row takes a CTA from more than kShortRow + kWarpRow / k entries on (200,000
-// power-law rows of up to 500 entries, 3,100 long ones, k = 8 / 16: 27.4 -> 23.1, 47.1 -> 32.1 us against a
-// warp up to 512 entries); kManyLongRows keep the GPU busy by themselves, and warps waste less on their sums
-// (40,000 rows of 200 entries, k = 4: 207.7 us on CTAs, 92 on warps).
-constexpr int kShortRow = 32;
+// Rows of more than short_row entries, longest first, for the kernel that gives them a warp or a CTA
+// each: n_cta[k] of the n rows take a CTA.  The other rows take a lane (per column), four entries a round
+// of dependent loads, so short_row is kShortRow, or kShortRowWide where more than kAutoLongShare of the
+// rows exceed that (power-law rows of up to 2000 entries, 200,000 / 1,000,000 of them, k = 1, short_row 32 /
+// 16 / 12 / 8: 13.2 / 11.2 / 10.3 / 10.9 and 43.2 / 40.0 / 40.0 / 45.8 us).  With k right-hand sides a warp
+// has 32 / k lanes per column, so while they are few a row takes a CTA from more than kCtaRow +
+// kWarpRow / k entries on (200,000 power-law rows of up to 500 entries, k = 8 / 16: 27.4 -> 23.1, 47.1 ->
+// 32.1 us against a warp up to 512 entries); kManyLongRows keep the GPU busy by themselves, and warps waste
+// less on their sums (40,000 rows of 200 entries, k = 4: 207.7 us on CTAs, 92 on warps).
+constexpr int kShortRow = 12;
+constexpr int kShortRowWide = 32;
+constexpr int kCtaRow = 32;
 constexpr int kWarpRow = 512;
-constexpr size_t kManyLongRows = 4096;
+constexpr size_t kManyLongRows = 16384;
 constexpr int kMaxK = 16;
 struct LongRows {
   const int32_t* rows = nullptr;
-  int n = 0, n_cta[kMaxK + 1] = {};
+  int n = 0, short_row = 0, n_cta[kMaxK + 1] = {};
 };
 
 // CRS_L1 reads the rows in aligned groups of four entries from this many entries per row on average

@@ -81,3 +81,33 @@ def test_infinities_stay_in_their_rows(lib):
             yi = run(p, Bi)
             assert np.array_equal(yi[~hit], y[~hit]) and not np.isfinite(yi[hit]).any()
     assert hit.any() and oracle.spmv(A, B[:, 0].copy()).shape == (A.n_rows,)
+
+
+def quick(lens, n_cols, seed):
+    """Rows of the given lengths, random columns (repeats allowed)."""
+    rng = np.random.default_rng(seed)
+    rp = np.zeros(len(lens) + 1, np.int32)
+    rp[1:] = np.cumsum(lens)
+    return gen.CSR(len(lens), n_cols, rp, rng.integers(0, n_cols, rp[-1]).astype(np.int32),
+                   rng.uniform(-1, 1, rp[-1]))
+
+
+@pytest.mark.parametrize("k", [1, 3, 8, 16])
+def test_classes_of_rows(lib, k):
+    """Where a lane's rows end (12 entries, or 32 when a quarter of the rows exceed 12), where a warp's end
+    for this k, and more than 16,384 long rows (warps up to 512 entries)."""
+    rng = np.random.default_rng(k)
+    few = rng.integers(0, 13, 3000)
+    few[::60] = rng.choice([11, 12, 13, 14, 32 + 512 // k, 33 + 512 // k, 700], 50)
+    half = np.where(rng.random(3000) < 0.5, rng.integers(13, 33, 3000), 3)
+    half[::200] = [33, 34, 60, 64, 100, 500, 544, 545, 600, 1000, 31, 32, 33, 70, 90]
+    many = np.full(80_000, 2)
+    many[::4] = rng.integers(13, 60, 20_000)
+    many[1] = 900
+    for lens in (few, half, many):
+        A = quick(lens, 4000, seed=k)
+        B = gen.rhs_block(A.n_cols, k, seed=k)
+        B = B[:, 0].copy() if k == 1 else B
+        with lib.Plan.from_csr(A) as p:
+            assert p.info().variant == lib.SPMV_CRS_L1
+            assert_close(run(p, B), A, B)
