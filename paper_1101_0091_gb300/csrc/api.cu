@@ -249,9 +249,10 @@ static int lane_cols(const RowStats& s, int64_t nnz) {
 // more than kAutoLongShare of the rows are long.
 static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s, int* short_row) {
   std::vector<int32_t> list;
-  const double most = kAutoLongShare * (double)n;
+  const int64_t few = std::max<int64_t>(kManyLongRows, (int64_t)(kAutoOverShare * (double)n));
+  const int64_t most = (int64_t)(kAutoLongShare * (double)n);
   if (s.longest <= kAutoLongestRow || s.n_long > most) return list;
-  *short_row = s.n_over <= most ? kShortRow : kShortRowWide;
+  *short_row = s.n_over <= std::min(few, most) ? kShortRow : kShortRowWide;
   for (int64_t i = 0; i < n; ++i)
     if (rp[i + 1] - rp[i] > *short_row) list.push_back((int32_t)i);
   std::stable_sort(list.begin(), list.end(),

@@ -92,14 +92,18 @@ constexpr double kAutoScattered = 0.3;
 constexpr double kAutoSellFill = 0.85;
 // AUTO's CRS_L1 gives the long rows (LongRows, layout.h) a warp or a CTA each when the longest row
 // exceeds kAutoLongestRow and they are at most kAutoLongShare of the rows; an explicit CRS_L1 keeps
-// every row on one thread.  Both sides (rows of more than 32 entries split), one thread per row -> long rows split: power-law lengths, 200,000
-// rows, longest row 40 / 64 / 96 / 256 at k = 1: 14.5 -> 14.0 / 16.6 -> 12.6 / 20.7 -> 14.3 /
-// 39.0 -> 14.4 us (2,000,000 rows: 69.7 -> 69.0 / 82.8 -> 73.4 / 95.7 -> 74.3 / 135.6 -> 77.6).  300,000
-// banded rows of which a share has 96 entries, the others 7: share 0.1 / 0.25 / 0.5 / 1 at k = 1 57.7 ->
-// 25.1 / 65.7 -> 49.6 / 70.3 -> 88.9 / 95.4 -> 164.4 us, at k = 4 204.8 -> 48.0 / 209.8 -> 94.7 / 212.0 ->
-// 168.5 / 209.1 -> 302.7 us.
-constexpr int kAutoLongestRow = 48;
+// every row on one lane.  Both sides, one lane per row -> long rows split: power-law lengths, 200,000
+// rows, longest row 20 / 32 / 48 / 96 / 256 at k = 1: 10.9 -> 8.5 / 12.9 -> 8.9 / 15.5 -> 9.2 / 20.3 -> 9.6 /
+// 32.5 -> 9.8 us (2,000,000 rows: 48.8 -> 49.4 / 59.3 -> 56.6 / 69.8 -> 60.3 / 89.4 -> 63.8 / 125.4 -> 66.4);
+// 2,000,000 rows of Poisson(6) lengths (longest 20) 49.4 -> 54.6.  300,000 banded rows of which a share has
+// 96 entries, the others 7: share 0.1 / 0.25 / 0.5 / 1 at k = 1 57.7 -> 25.1 / 65.7 -> 49.6 / 70.3 -> 88.9 /
+// 95.4 -> 164.4 us.
+constexpr int kAutoLongestRow = 28;
 constexpr double kAutoLongShare = 0.25;
+// They are the rows of more than kShortRow entries while those are few (kManyLongRows of them, or this
+// share), else those of more than kShortRowWide: 2,000,000 rows of 5 of which 5 % have 24 entries took 101.1
+// us with these on warps, 77.5 on lanes.
+constexpr double kAutoOverShare = 0.03;
 
 // Share of a row sample's entries gathered at scattered addresses by consecutive rows (see host.cpp).
 double scattered_fraction(const int32_t* row_ptr, const int32_t* col, int64_t n_rows);

@@ -22,8 +22,8 @@ constexpr uint32_t kBlockWarpFlag = 0x80000000u;  // high bit of a row-block ent
 
 // Rows of more than short_row entries, longest first, for the kernel that gives them a warp or a CTA
 // each: n_cta[k] of the n rows take a CTA.  The other rows take a lane (per column), four entries a round
-// of dependent loads, so short_row is kShortRow, or kShortRowWide where more than kAutoLongShare of the
-// rows exceed that (power-law rows of up to 2000 entries, 200,000 / 1,000,000 of them, k = 1, short_row 32 /
+// of dependent loads, so short_row is kShortRow, or kShortRowWide where too many rows exceed that
+// (kAutoOverShare, internal.h; power-law rows of up to 2000 entries, 200,000 / 1,000,000 of them, k = 1, short_row 32 /
 // 16 / 12 / 8: 13.2 / 11.2 / 10.3 / 10.9 and 43.2 / 40.0 / 40.0 / 45.8 us).  With k right-hand sides a warp
 // has 32 / k lanes per column, so while they are few a row takes a CTA from more than kCtaRow +
 // kWarpRow / k entries on (200,000 power-law rows of up to 500 entries, k = 8 / 16: 27.4 -> 23.1, 47.1 ->
