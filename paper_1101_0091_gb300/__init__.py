@@ -114,8 +114,7 @@ def sym_build(A) -> dict:
 
 def _stream_handle(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _b.current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

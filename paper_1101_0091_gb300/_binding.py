@@ -87,6 +87,8 @@ def lib_path() -> str:
 def load():
     """Load the built library (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = lib_path()
@@ -100,6 +102,25 @@ def load():
                 fn.restype = res
             _lib = lib
     return _lib
+
+
+_raw_stream = _get_device = None
+
+
+def current_stream() -> int:
+    """Handle of PyTorch's current stream on its current device.  torch.cuda.current_stream() builds a
+    Stream object on every call (2.9 of the 7.2 us of one small product); the raw getter behind it takes
+    0.2 us.  PyTorch's CUDA state is initialised on the first call."""
+    global _raw_stream, _get_device
+    if _raw_stream is None:
+        import torch
+        s = torch.cuda.current_stream().cuda_stream
+        getters = (getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None))
+        if None in getters:
+            return s
+        _get_device = getters[1]
+        _raw_stream = getters[0]
+    return _raw_stream(_get_device())
 
 
 def _check(st: int):

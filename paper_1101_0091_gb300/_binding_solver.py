@@ -6,7 +6,7 @@ import ctypes
 
 import numpy as np
 
-from ._binding import _check, _i32, _vp, load
+from ._binding import _check, _i32, _vp, current_stream, load
 
 
 class spmv_cg_summary(ctypes.Structure):
@@ -59,8 +59,7 @@ def spmv_lanczos(h, V0_dev: int, m: int, alpha_host: int, beta_host: int, stream
 
 def _stream(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return current_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
