@@ -604,7 +604,7 @@ spmv_status spmv_apply_split(spmv_handle h, double* B_dev, const double* B_halo_
   cudaError_t e = run_variant(h, h->local, lv, B_dev, 1, C_dev, 1, 1, ms);
   if (e != cudaSuccess) return cuda_fail(e, "local kernel launch");
   if (nhalo > 0 && cs != ms) SPMV_CUDA(cudaStreamWaitEvent(ms, h->ev_copy, 0));
-  e = launch_halo(h->halo, f32, B_dev, 1, C_dev, 1, 1, ms);
+  e = launch_halo(h->halo, f32, B_dev, C_dev, ms);
   if (e != cudaSuccess) return cuda_fail(e, "halo kernel launch");
   return SPMV_OK;
 }

@@ -139,8 +139,7 @@ cudaError_t launch_crs_lanes(const CsrDev& A, bool fp32, int lanes, const double
                              double* C, int64_t ldc, int k, cudaStream_t s);
 cudaError_t launch_sell(const SellDev& S, bool fp32, const double* B, int64_t ldb, double* C,
                         int64_t ldc, int k, cudaStream_t s);
-cudaError_t launch_halo(const HaloDev& H, bool fp32, const double* B, int64_t ldb, double* C,
-                        int64_t ldc, int k, cudaStream_t s);
+cudaError_t launch_halo(const HaloDev& H, bool fp32, const double* B, double* C, cudaStream_t s);
 // Zeroes C[:, 0:k] on the stream, then runs the symmetric kernel.
 cudaError_t launch_sym(const SymDev& S, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc,
                        int k, cudaStream_t s);

@@ -1,13 +1,11 @@
 // CRS_L{1,2,4,8,16,32}: L lanes per row, loads straight from HBM (Sec. 1.2 loop).
 //
-// A group of L consecutive lanes owns one row; lane t of the group takes
-// entries rs + t, rs + t + L, ... (for L >= 8 a group's loads of val/col_idx
-// coalesce), gathers B with read-only loads and keeps FP64 partial sums, which
-// an xor-shuffle tree of log2(L) steps adds at the end.  L = 1 is the classic
-// scalar CRS kernel.  The same kernel with a row list and accumulate = 1 is the
-// halo pass of the local/halo split: C[rows[t]] += (halo row t) * B.
+// L >= 2 (k_crs_lanes): a group of L consecutive lanes owns one row; lane t of the
+// group takes entries rs + t, rs + t + L, ... (for L >= 8 a group's loads of
+// val/col_idx coalesce), gathers B with read-only loads and keeps FP64 partial sums,
+// which an xor-shuffle tree of log2(L) steps adds at the end.
 //
-// CRS_L1 as a plan's kernel is a family of its own (crs_l1): one vector on short rows
+// CRS_L1 is a family of its own (crs_l1): one vector on short rows
 // (k_crs_row) or on rows of eight and more entries on average (k_crs_wide), blocks of
 // k >= 2 columns with a row's columns split over k / W lanes (k_crs_cols), and, when
 // AUTO asks for it, a few long rows on a warp or a CTA each (k_crs_long).  Except for
@@ -40,9 +38,9 @@ __device__ __forceinline__ void prefetch_rows(int64_t f0, int64_t rows, int64_t 
 // entry's K values are gathered with K / 2 16-byte loads instead of K 8-byte ones.
 template <typename VT, int L, int K, bool VEC>
 __global__ void __launch_bounds__(kThreads, (K == 1 ? 8 : 1))
-    k_crs_lanes(int64_t n_rows, const int32_t* __restrict__ rows, const int32_t* __restrict__ row_ptr,
-                const int32_t* __restrict__ col, const VT* __restrict__ val, const double* __restrict__ B,
-                int64_t ldb, double* __restrict__ C, int64_t ldc, int k, int accumulate, int prefetch) {
+    k_crs_lanes(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                const VT* __restrict__ val, const double* __restrict__ B, int64_t ldb, double* __restrict__ C,
+                int64_t ldc, int k, int prefetch) {
   constexpr int RPC = kThreads / L;  // rows per CTA
   // bring the val/col slices of the CTA `prefetch` positions ahead into L2
   if (threadIdx.x == 0 && prefetch > 0)
@@ -59,10 +57,9 @@ __global__ void __launch_bounds__(kThreads, (K == 1 ? 8 : 1))
 #pragma unroll
   for (int q = 0; q < K; ++q) acc[q] = 0.0;
   // batches of NB entries per lane: all gathers of a batch are issued before its FMAs
-  constexpr int NB1 = sizeof(VT) == 8 ? 8 : 4;  // single-lane batch (FP32 storage: widening needs registers)
   // (K >= 4: one entry per batch; its K gathers already keep the FP64 pipe fed, and two entries
   // measured 9 % slower at K = 4)
-  constexpr int NB = K >= 4 ? 1 : (L >= 4 ? 1 : (L == 2 ? 4 / K : NB1 / K > 0 ? NB1 / K : 1));
+  constexpr int NB = K < 4 && L == 2 ? 4 / K : 1;
   for (int j = rs + t; j < re; j += NB * L) {
     double v[NB];
     const double* b[NB];
@@ -94,17 +91,13 @@ __global__ void __launch_bounds__(kThreads, (K == 1 ? 8 : 1))
       for (int q = 0; q < K; ++q)
         if (j + u * L < re && q < k) acc[q] = fma(v[u], gv[u][q], acc[q]);
   }
-  if (L > 1) {
 #pragma unroll
-    for (int q = 0; q < K; ++q) acc[q] = warp_sum_xor(acc[q], L);
-  }
+  for (int q = 0; q < K; ++q) acc[q] = warp_sum_xor(acc[q], L);
   if (!active) return;
-  const int64_t row = rows ? (int64_t)__ldg(rows + g) : g;
-  double* out = C + row * ldc;
+  double* out = C + g * ldc;
 #pragma unroll
-  for (int q = 0; q < K; ++q) {
-    if (q < k && (L == 1 || t == q % L)) out[q] = accumulate ? out[q] + acc[q] : acc[q];
-  }
+  for (int q = 0; q < K; ++q)
+    if (q < k && t == q % L) out[q] = acc[q];
 }
 
 // The last 0..3 entries of a row (r of them, gathers x): no multiply-add is issued that no lane of the
@@ -164,6 +157,23 @@ __global__ void __launch_bounds__(kThreads, 8)
   }
   add_tail(re - j, v, x, acc);
   C[g * ldc] = acc[0];
+}
+
+// The halo pass of the local/halo split: C[rows[t]] += (halo row t) * B, as k_crs_row.
+template <typename VT>
+__global__ void __launch_bounds__(kThreads, 8)
+    k_crs_halo(int64_t n_rows, const int32_t* __restrict__ rows, const int32_t* __restrict__ row_ptr,
+               const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B, double* C) {
+  grid_dependents();
+  const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (g >= n_rows) return;
+  const int64_t row = __ldg(rows + g);
+  const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
+  grid_wait();
+  const double c = C[row];
+  double acc = 0.0;
+  for (int j = rs; j < re; ++j) acc = fma(to_f64(ldg(val + j)), B[ldg(col + j)], acc);
+  C[row] = c + acc;
 }
 
 // k columns of a row on G = k / W lanes, W columns each (W = 4 or 2 with 16-byte accesses, else 1).
@@ -402,52 +412,29 @@ static cudaError_t launch_long(const CsrDev& A, const VT* val, const double* B, 
 }
 
 template <typename VT, int L, int K>
-static cudaError_t launch_lanes_t(int64_t n_rows, const int32_t* rows, const int32_t* row_ptr,
-                                  const int32_t* col, const VT* val, const double* B, int64_t ldb, double* C,
-                                  int64_t ldc, int k, bool acc, int pf, cudaStream_t s) {
+static cudaError_t launch_lanes_t(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C,
+                                  int64_t ldc, int k, cudaStream_t s) {
   const int64_t rows_per_cta = kThreads / L;
-  const int64_t grid = (n_rows + rows_per_cta - 1) / rows_per_cta;
-  if constexpr (L > 1 && K >= 2) {
-    // several lanes per row on a full block with 16-byte aligned B rows: 16-byte gathers
-    if (k == K && ldb % 2 == 0 && (((uintptr_t)B) & 15) == 0) {
-      k_crs_lanes<VT, L, K, true><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, rows, row_ptr, col, val, B, ldb, C,
-                                                                        ldc, k, acc ? 1 : 0, pf);
-      return cudaGetLastError();
-    }
-  }
-  k_crs_lanes<VT, L, K, false><<<(unsigned)grid, kThreads, 0, s>>>(n_rows, rows, row_ptr, col, val, B, ldb, C,
-                                                                     ldc, k, acc ? 1 : 0, pf);
+  const int64_t grid = (A.n_rows + rows_per_cta - 1) / rows_per_cta;
+  // a full block with 16-byte aligned B rows: 16-byte gathers
+  if (K >= 2 && k == K && ldb % 2 == 0 && (((uintptr_t)B) & 15) == 0)
+    k_crs_lanes<VT, L, K, (K >= 2)><<<(unsigned)grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
+                                                                          ldc, k, A.prefetch);
+  else
+    k_crs_lanes<VT, L, K, false><<<(unsigned)grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, B, ldb, C, ldc,
+                                                                       k, A.prefetch);
   return cudaGetLastError();
 }
 
 template <typename VT, int L>
-static cudaError_t lanes_k(int64_t n, const int32_t* rows, const int32_t* rp, const int32_t* col, const VT* val,
-                           const double* B, int64_t ldb, double* C, int64_t ldc, int k, bool acc,
-                           int pf, cudaStream_t s) {
-  if (n == 0) return cudaSuccess;
-  if (k <= 1) return launch_lanes_t<VT, L, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  if constexpr (L == 1) return cudaErrorInvalidValue;  // the halo pass only, k = 1
-  else {
-    if (k <= 2) return launch_lanes_t<VT, L, 2>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    if (k <= 4) return launch_lanes_t<VT, L, 4>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    if (k <= 8) return launch_lanes_t<VT, L, 8>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    return launch_lanes_t<VT, L, 16>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-  }
-}
-
-template <typename VT>
-static cudaError_t lanes_dispatch(int lanes, int64_t n, const int32_t* rows, const int32_t* rp,
-                                  const int32_t* col, const VT* val, const double* B, int64_t ldb, double* C,
-                                  int64_t ldc, int k, bool acc, int pf, cudaStream_t s) {
-  switch (lanes) {
-    case 1: return lanes_k<VT, 1>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    case 2: return lanes_k<VT, 2>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    case 4: return lanes_k<VT, 4>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    case 8: return lanes_k<VT, 8>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    case 16: return lanes_k<VT, 16>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    case 32: return lanes_k<VT, 32>(n, rows, rp, col, val, B, ldb, C, ldc, k, acc, pf, s);
-    default: return cudaErrorInvalidValue;
-  }
+static cudaError_t lanes_k(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
+                           cudaStream_t s) {
+  if (A.n_rows == 0) return cudaSuccess;
+  if (k <= 1) return launch_lanes_t<VT, L, 1>(A, val, B, ldb, C, ldc, k, s);
+  if (k <= 2) return launch_lanes_t<VT, L, 2>(A, val, B, ldb, C, ldc, k, s);
+  if (k <= 4) return launch_lanes_t<VT, L, 4>(A, val, B, ldb, C, ldc, k, s);
+  if (k <= 8) return launch_lanes_t<VT, L, 8>(A, val, B, ldb, C, ldc, k, s);
+  return launch_lanes_t<VT, L, 16>(A, val, B, ldb, C, ldc, k, s);
 }
 
 // CRS_L1: the kernel for the plan's rows and the block's width and alignment.
@@ -483,8 +470,15 @@ static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64
 template <typename VT>
 static cudaError_t crs_dispatch(const CsrDev& A, int lanes, const VT* val, const double* B, int64_t ldb, double* C,
                                 int64_t ldc, int k, cudaStream_t s) {
-  if (lanes == 1) return crs_l1(A, val, B, ldb, C, ldc, k, s);
-  return lanes_dispatch<VT>(lanes, A.n_rows, nullptr, A.row_ptr, A.col, val, B, ldb, C, ldc, k, false, A.prefetch, s);
+  switch (lanes) {
+    case 1: return crs_l1(A, val, B, ldb, C, ldc, k, s);
+    case 2: return lanes_k<VT, 2>(A, val, B, ldb, C, ldc, k, s);
+    case 4: return lanes_k<VT, 4>(A, val, B, ldb, C, ldc, k, s);
+    case 8: return lanes_k<VT, 8>(A, val, B, ldb, C, ldc, k, s);
+    case 16: return lanes_k<VT, 16>(A, val, B, ldb, C, ldc, k, s);
+    case 32: return lanes_k<VT, 32>(A, val, B, ldb, C, ldc, k, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_crs_lanes(const CsrDev& A, bool fp32, int lanes, const double* B, int64_t ldb, double* C,
@@ -494,14 +488,17 @@ cudaError_t launch_crs_lanes(const CsrDev& A, bool fp32, int lanes, const double
   return crs_dispatch<double>(A, lanes, A.val, B, ldb, C, ldc, k, s);
 }
 
-cudaError_t launch_halo(const HaloDev& H, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc, int k,
-                        cudaStream_t s) {
-  if (fp32 && H.val32_special)
-    return lanes_dispatch<float>(1, H.n_rows, H.rows, H.row_ptr, H.col, H.val32, B, ldb, C, ldc, k, true, 0, s);
-  if (fp32)
-    return lanes_dispatch<f32n>(1, H.n_rows, H.rows, H.row_ptr, H.col, reinterpret_cast<const f32n*>(H.val32), B,
-                                ldb, C, ldc, k, true, 0, s);
-  return lanes_dispatch<double>(1, H.n_rows, H.rows, H.row_ptr, H.col, H.val, B, ldb, C, ldc, k, true, 0, s);
+template <typename VT>
+static cudaError_t launch_halo_v(const HaloDev& H, const VT* val, const double* B, double* C, cudaStream_t s) {
+  if (H.n_rows == 0) return cudaSuccess;
+  return launch_dependent(k_crs_halo<VT>, (unsigned)((H.n_rows + kThreads - 1) / kThreads), kThreads, s, H.n_rows,
+                          H.rows, H.row_ptr, H.col, val, B, C);
+}
+
+cudaError_t launch_halo(const HaloDev& H, bool fp32, const double* B, double* C, cudaStream_t s) {
+  if (fp32 && H.val32_special) return launch_halo_v<float>(H, H.val32, B, C, s);
+  if (fp32) return launch_halo_v<f32n>(H, reinterpret_cast<const f32n*>(H.val32), B, C, s);
+  return launch_halo_v<double>(H, H.val, B, C, s);
 }
 
 }  // namespace spmv

@@ -67,3 +67,27 @@ def test_chains_equal_synchronised_chains(lib, name):
             g.replay()
             torch.cuda.synchronize()
             assert np.array_equal(host(x), chain(p, x0, 40, False, True))
+
+
+def test_split_chain_equals_the_synchronised_one(lib):
+    """The halo pass and the next local pass start behind one another the same way."""
+    import torch
+    A = gen.poisson3d_var(40)
+    h = A.n_cols - A.n_cols // 10
+    x0 = gen.uniform(A.n_cols, seed=3)
+    halo = torch.from_numpy(x0[h:].copy()).pin_memory()
+    copy = torch.cuda.Stream()
+    with lib.Plan.from_csr(A, halo_begin=h) as p:
+        got = []
+        for sync in (True, False, False):
+            B, C = dev(x0.copy()), torch.zeros(A.n_rows, dtype=torch.float64, device="cuda")
+            for _ in range(20):
+                p.apply_split(B, halo, C, copy_stream=copy)
+                if sync:
+                    torch.cuda.synchronize()
+                torch.mul(C[:h], 1.0 / 32, out=B[:h])
+                p.apply_split(B, halo, C, copy_stream=copy)
+                if sync:
+                    torch.cuda.synchronize()
+            got.append(host(C))
+        assert np.isfinite(got[0]).all() and all(np.array_equal(g, got[0]) for g in got)
