@@ -28,8 +28,8 @@ constexpr int kMaxCols = 16;
 
 // Per-column scalars.  Every CTA of a kernel reads them and CTA 0 writes, so no kernel writes a field
 // that it reads: k_cg_direction writes rr, active, iters and n_active, k_cg_update the others, with
-// copies (rr_old) or working sets (running) of what k_cg_direction needs; in the Lanczos kernels
-// k_lz_scale writes live_next and b_prev, k_lz_alpha live.
+// copies (rr_old) or working sets (running) of what k_cg_direction needs; k_lz_alpha writes inv and
+// live, k_lz_beta their copies.
 struct CgScalars {
   double rr[kMaxCols], rr_old[kMaxCols], tol2[kMaxCols], alpha[kMaxCols];
   int active[kMaxCols], running[kMaxCols], iters[kMaxCols], breakdown[kMaxCols];
@@ -37,8 +37,8 @@ struct CgScalars {
 };
 
 struct LzScalars {
-  double b_prev[kMaxCols];
-  int live[kMaxCols], live_next[kMaxCols];
+  double inv[kMaxCols], inv_old[kMaxCols];
+  int live[kMaxCols], live_old[kMaxCols];
 };
 
 // ---------------------------------------------------------------- block walking
@@ -460,61 +460,92 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, co
   write_partial<G>(acc, k, partial, sh);
 }
 
-// W = W - b_prev v_prev; column sums of W.v.
+// The Lanczos vectors stay unscaled: u_j = |u_j| v_j, where |u_j| = beta_{j-1} and inv_j = 1 / |u_j| (0 for
+// a column that has stopped).  W (= A u_j) becomes A v_j - beta_{j-1} v_{j-1} = inv_j W - (beta_{j-1}
+// inv_{j-1}) u_{j-1}; column sums of W.u_j.  The pass that divided W by its norm is gone (k = 4, 500,009 rows:
+// 92.2 -> 89.2 us a step; seven vector
+// passes instead of nine).  beta_{j-1} comes from the partials of u_j.u_j; it is stored to
+// beta_out unless that is NULL (j = 1: |V0|, every column live before).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_alpha(int64_t n, int k, double* W, const double* v,
-               const double* v_prev, double* partial, LzScalars* S) {
+    k_lz_alpha(int64_t n, int k, double* W, const double* u, const double* u_prev, const double* uu_partial,
+               double* wu_partial, LzScalars* S, double* beta_out) {
   using G = Seg<K, MODE>;
   grid_dependents();
   grid_wait();
   __shared__ VecShared sh;
-  if (blockIdx.x == 0 && (int)threadIdx.x < k) S->live[threadIdx.x] = S->live_next[threadIdx.x];
-  double b[G::KC], acc[G::KC];
+  __shared__ double s_inv[kMaxCols], s_prev[kMaxCols];
+  Walk<G> w(n, k);
+  double x[G::U][G::W], uj[G::U][G::W], up[G::U][G::W];
+  w.load(W, x);
+  w.load(u, uj);
+  const double uu = read_partials<G>(uu_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) {
+    const bool first = beta_out == nullptr;
+    const double b = first || S->live_old[c] ? sqrt(uu) : 0.0;
+    const bool live = b > 0.0;
+    s_inv[c] = live ? 1.0 / b : 0.0;
+    s_prev[c] = !first && live ? b * S->inv_old[c] : 0.0;
+    if (blockIdx.x == 0) {
+      if (!first) beta_out[c] = b;
+      S->live[c] = live;
+      S->inv[c] = s_inv[c];
+    }
+  }
+  __syncthreads();
+  double inv[G::KC], prev[G::KC], acc[G::KC];
   const int c0 = G::column(threadIdx.x, k);
 #pragma unroll
   for (int q = 0; q < G::KC; ++q) {
-    b[q] = S->b_prev[c0 + q];
+    inv[q] = s_inv[c0 + q];
+    prev[q] = s_prev[c0 + q];
     acc[q] = 0.0;
   }
-  for (Walk<G> w(n, k); w.more(); w.next()) {
-    double x[G::U][G::W], vv[G::U][G::W], vp[G::U][G::W];
-    w.load(W, x);
-    w.load(v, vv);
-    w.load(v_prev, vp);
+  while (w.more()) {
+    w.load(u_prev, up);
 #pragma unroll
     for (int j = 0; j < G::U; ++j) {
       if (!w.has(j)) break;
 #pragma unroll
       for (int i = 0; i < G::W; ++i) {
         const int q = G::acc(i);
-        x[j][i] = fma(-b[q], vp[j][i], x[j][i]);
-        acc[q] = fma(x[j][i], vv[j][i], acc[q]);
+        x[j][i] = fma(-prev[q], up[j][i], inv[q] * x[j][i]);
+        acc[q] = fma(x[j][i], uj[j][i], acc[q]);
       }
     }
     w.store(W, x);
+    w.next();
+    w.load(W, x);
+    w.load(u, uj);
   }
-  write_partial<G>(acc, k, partial, sh);
+  write_partial<G>(acc, k, wu_partial, sh);
 }
 
-// alpha = W.v (live columns), stored to alpha_out; W = W - alpha v; column sums of W.W.
+// alpha_j = W.v_j (live columns), stored to alpha_out; W = W - alpha_j v_j = u_{j+1}; column sums of W.W.
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_beta(int64_t n, int k, double* W, const double* v, const double* a_partial,
-              double* b_partial, const LzScalars* S, double* alpha_out) {
+    k_lz_beta(int64_t n, int k, double* W, const double* u, const double* wu_partial, double* uu_partial,
+              LzScalars* S, double* alpha_out) {
   using G = Seg<K, MODE>;
   grid_dependents();
   grid_wait();
   __shared__ VecShared sh;
   __shared__ double s_a[kMaxCols];
   Walk<G> w(n, k);
-  double x[G::U][G::W], vv[G::U][G::W];
+  double x[G::U][G::W], uj[G::U][G::W];
   w.load(W, x);
-  w.load(v, vv);
-  const double wv = read_partials<G>(a_partial, gridDim.x, k, sh);
-  if ((int)threadIdx.x < k) {
-    s_a[threadIdx.x] = S->live_next[threadIdx.x] ? wv : 0.0;
-    if (blockIdx.x == 0) alpha_out[threadIdx.x] = s_a[threadIdx.x];
+  w.load(u, uj);
+  const double wu = read_partials<G>(wu_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) {
+    const double inv = S->inv[c], alpha = S->live[c] ? wu * inv : 0.0;
+    s_a[c] = alpha * inv;
+    if (blockIdx.x == 0) {
+      alpha_out[c] = alpha;
+      S->inv_old[c] = inv;
+      S->live_old[c] = S->live[c];
+    }
   }
   __syncthreads();
   double a[G::KC], acc[G::KC];
@@ -531,67 +562,28 @@ __global__ void __launch_bounds__(kVecThreads, 2)
 #pragma unroll
       for (int i = 0; i < G::W; ++i) {
         const int q = G::acc(i);
-        x[j][i] = fma(-a[q], vv[j][i], x[j][i]);
+        x[j][i] = fma(-a[q], uj[j][i], x[j][i]);
         acc[q] = fma(x[j][i], x[j][i], acc[q]);
       }
     }
     w.store(W, x);
     w.next();
     w.load(W, x);
-    w.load(v, vv);
+    w.load(u, uj);
   }
-  write_partial<G>(acc, k, b_partial, sh);
+  write_partial<G>(acc, k, uu_partial, sh);
 }
 
-// beta = |W| (live columns), stored to beta_out; v_next = W / beta (one FP64 division per column
-// instead of one per entry); a column whose beta is 0 stops.  FIRST (W = V0): every column is live
-// before, and the previous vector's coefficient is 0.
-template <int K, int MODE, bool FIRST>
-__global__ void __launch_bounds__(kVecThreads, 2)
-    k_lz_scale(int64_t n, int k, const double* W, double* v_next, const double* b_partial,
-               LzScalars* S, double* beta_out) {
+// One CTA: the last beta.
+template <int K, int MODE>
+__global__ void __launch_bounds__(kVecThreads) k_lz_end(int k, const double* uu_partial, unsigned n_partials,
+                                                        const LzScalars* S, double* beta_out) {
   using G = Seg<K, MODE>;
   grid_dependents();
   grid_wait();
   __shared__ VecShared sh;
-  __shared__ double s_inv[kMaxCols];
-  __shared__ int s_live[kMaxCols];
-  Walk<G> w(n, k);
-  double x[G::U][G::W];
-  w.load(W, x);
-  const double ww = read_partials<G>(b_partial, gridDim.x, k, sh);
-  const int c = threadIdx.x;
-  if (c < k) {
-    const double b = FIRST || S->live[c] ? sqrt(ww) : 0.0;
-    const bool live = b > 0.0;
-    s_live[c] = live;
-    s_inv[c] = live ? 1.0 / b : 0.0;
-    if (blockIdx.x == 0) {
-      if (!FIRST) beta_out[c] = b;
-      S->live_next[c] = live;
-      S->b_prev[c] = !FIRST && live ? b : 0.0;
-    }
-  }
-  __syncthreads();
-  double inv[G::KC];
-  bool live[G::KC];
-  const int c0 = G::column(threadIdx.x, k);
-#pragma unroll
-  for (int q = 0; q < G::KC; ++q) {
-    inv[q] = s_inv[c0 + q];
-    live[q] = s_live[c0 + q];
-  }
-  while (w.more()) {
-#pragma unroll
-    for (int j = 0; j < G::U; ++j) {
-      if (!w.has(j)) break;
-#pragma unroll
-      for (int i = 0; i < G::W; ++i) x[j][i] = live[G::acc(i)] ? x[j][i] * inv[G::acc(i)] : 0.0;
-    }
-    w.store(v_next, x);
-    w.next();
-    w.load(W, x);
-  }
+  const double uu = read_partials<G>(uu_partial, n_partials, k, sh);
+  if ((int)threadIdx.x < k) beta_out[threadIdx.x] = S->live_old[threadIdx.x] ? sqrt(uu) : 0.0;
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -621,10 +613,9 @@ SOLVER_LAUNCHER(LCgDot, k_cg_dot<K, MODE>)
 SOLVER_LAUNCHER(LCgUpdate, k_cg_update<K, MODE>)
 SOLVER_LAUNCHER(LCgDirection, k_cg_direction<K, MODE>)
 SOLVER_LAUNCHER(LLzNorm, k_lz_norm<K, MODE>)
-SOLVER_LAUNCHER(LLzFirst, k_lz_scale<K, MODE, true>)
 SOLVER_LAUNCHER(LLzAlpha, k_lz_alpha<K, MODE>)
 SOLVER_LAUNCHER(LLzBeta, k_lz_beta<K, MODE>)
-SOLVER_LAUNCHER(LLzScale, k_lz_scale<K, MODE, false>)
+SOLVER_LAUNCHER(LLzEnd, k_lz_end<K, MODE>)
 #undef SOLVER_LAUNCHER
 
 // CTAs of the vector kernels on an n x k block: enough for its units, at most `most`.
@@ -647,7 +638,7 @@ struct spmv_solver {
   int device = 0, k = 0;
   int64_t n = 0;
   unsigned grid = 1;               // CTAs of the vector kernels (one wave at most)
-  double *buf[3] = {nullptr, nullptr, nullptr};  // CG: R, P, Q; Lanczos: v_prev, v, W
+  double *buf[3] = {nullptr, nullptr, nullptr};  // CG: R, P, Q; Lanczos: u_{j-1}, u_j, W in turn
   double *partial = nullptr, *partial2 = nullptr;  // column sums per CTA (two, one read while the other is written)
   CgScalars* cg = nullptr;
   LzScalars* lz = nullptr;
@@ -864,28 +855,27 @@ spmv_status spmv_lanczos(spmv_solver_handle S, const double* V0_dev, int32_t m, 
   }
   double* a_out = S->lz_out;
   double* b_out = S->lz_out + (size_t)m * kMaxCols;
-  double *v_prev = S->buf[0], *v = S->buf[1], *W = S->buf[2];
+  // u_1 = V0; u_{j+1} is the W of step j, which takes the buffers in turn (buffer 0 is u_0 = 0)
+  const double *u_prev = S->buf[0], *u = V0_dev;
   cudaError_t e = by_k<LLzNorm>(k, S->grid, s, S->n, k, V0_dev, S->partial);
-  if (e == cudaSuccess)
-    e = by_k<LLzFirst>(k, S->grid, s, S->n, k, V0_dev, v, (const double*)S->partial, S->lz, (double*)nullptr);
-  if (e == cudaSuccess) e = cudaMemsetAsync(v_prev, 0, sizeof(double) * (size_t)S->n * (size_t)k, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(S->buf[0], 0, sizeof(double) * (size_t)S->n * (size_t)k, s);
   if (e != cudaSuccess) return cuda_fail(e, "Lanczos start");
   for (int j = 0; j < m; ++j) {
-    spmv_status st = spmv_apply_block(S->A, v, k, k, W, k, s);
+    double* W = S->buf[(j + 1) % 3];
+    spmv_status st = spmv_apply_block(S->A, u, k, k, W, k, s);
     if (st != SPMV_OK) return st;
-    e = by_k<LLzAlpha>(k, S->grid, s, S->n, k, W, (const double*)v, (const double*)v_prev, S->partial, S->lz);
+    e = by_k<LLzAlpha>(k, S->grid, s, S->n, k, W, u, u_prev, (const double*)S->partial, S->partial2, S->lz,
+                       j ? b_out + (size_t)(j - 1) * kMaxCols : (double*)nullptr);
     if (e == cudaSuccess)
-      e = by_k<LLzBeta>(k, S->grid, s, S->n, k, W, (const double*)v, (const double*)S->partial, S->partial2,
-                        (const LzScalars*)S->lz, a_out + (size_t)j * kMaxCols);
-    // v_{j+1} = W / beta_j into the buffer of v_{j-1}, then rotate
-    if (e == cudaSuccess)
-      e = by_k<LLzScale>(k, S->grid, s, S->n, k, (const double*)W, v_prev, (const double*)S->partial2, S->lz,
-                         b_out + (size_t)j * kMaxCols);
+      e = by_k<LLzBeta>(k, S->grid, s, S->n, k, W, u, (const double*)S->partial2, S->partial, S->lz,
+                        a_out + (size_t)j * kMaxCols);
     if (e != cudaSuccess) return cuda_fail(e, "Lanczos kernel launch");
-    double* t = v_prev;
-    v_prev = v;
-    v = t;
+    u_prev = u;
+    u = W;
   }
+  e = by_k<LLzEnd>(k, 1u, s, k, (const double*)S->partial, S->grid, (const LzScalars*)S->lz,
+                   b_out + (size_t)(m - 1) * kMaxCols);
+  if (e != cudaSuccess) return cuda_fail(e, "Lanczos kernel launch");
   std::vector<double> tmp((size_t)2 * m * kMaxCols);
   SPMV_CUDA(cudaMemcpyAsync(tmp.data(), S->lz_out, sizeof(double) * tmp.size(), cudaMemcpyDeviceToHost, s));
   SPMV_CUDA(cudaStreamSynchronize(s));
