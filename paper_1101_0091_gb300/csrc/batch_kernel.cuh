@@ -69,7 +69,8 @@ __device__ __forceinline__ void gather_row(const double* __restrict__ b, int k, 
   }
 }
 
-template <int L, int K, bool VEC>
+// NB entries per lane have their gathers issued before their FMAs.
+template <int L, int K, bool VEC, int NB = (L == 1 && K <= 2 ? 4 / K : 1)>
 __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, const int2* __restrict__ rowlist,
                                            const BatchItem& item, int k, int lane) {
   const BatchMat& M = *Mp;  // fields are read where used, not held across the item
@@ -94,7 +95,6 @@ __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, cons
     double acc[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) acc[q] = 0.0;
-    constexpr int NB = (L == 1 && K <= 2) ? 4 / K : 1;  // gathers issued before their FMAs
     for (int j = rs + t; j < re; j += NB * L) {
       double v[NB];
       const double* b[NB];
@@ -136,6 +136,35 @@ __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, cons
           if (q < k && (L == 1 || t == q % L)) st_c(out + q, acc[q]);
       }
     }
+  }
+}
+
+// A round is a dependent pair of loads, a round trip to L2 or DRAM.  Long rows of
+// the same length class (mode 2, some 32 entries per lane) at K = 2 take four
+// entries a round, which costs no occupancy (512 members, k = 2: 355 -> 337 us; 32
+// members 46.7 -> 41.6).  Items of unsorted rows keep to one: slots past the end of
+// a short row still occupy the FP64 pipe (512 members on 8 lanes per row: 2.77 -> 4.05
+// ms).  So does K = 4, where two a round lengthen the launch (499 -> 507 us), and K = 1
+// (293 -> 301).
+template <int K, bool VEC>
+__device__ __forceinline__ void batch_row_item(const BatchMat* __restrict__ Mp, const int2* __restrict__ rowlist,
+                                               const BatchItem& item, int k, int lane) {
+  if (K == 2 && item.mode == 2) {
+    switch (item.lanes) {
+      case 2: batch_rows<2, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
+      case 4: batch_rows<4, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
+      case 8: batch_rows<8, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
+      case 16: batch_rows<16, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
+      case 32: batch_rows<32, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
+    }
+  }
+  switch (item.lanes) {
+    case 1: batch_rows<1, K, VEC>(Mp, rowlist, item, k, lane); break;
+    case 2: batch_rows<2, K, VEC>(Mp, rowlist, item, k, lane); break;
+    case 4: batch_rows<4, K, VEC>(Mp, rowlist, item, k, lane); break;
+    case 8: batch_rows<8, K, VEC>(Mp, rowlist, item, k, lane); break;
+    case 16: batch_rows<16, K, VEC>(Mp, rowlist, item, k, lane); break;
+    default: batch_rows<32, K, VEC>(Mp, rowlist, item, k, lane); break;
   }
 }
 
@@ -299,14 +328,7 @@ __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
   int it = dynamic ? next_item(0, nw, 1, counter, lane) : wid;
   while (it < n_items) {
     const BatchItem item = items[it];
-    switch (item.lanes) {
-      case 1: batch_rows<1, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      case 2: batch_rows<2, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      case 4: batch_rows<4, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      case 8: batch_rows<8, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      case 16: batch_rows<16, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      default: batch_rows<32, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-    }
+    batch_row_item<K, VEC>(mats + item.mat, rowlist, item, k, lane);
     it = next_item(it, nw, dynamic, counter, lane);
   }
 }
@@ -325,18 +347,10 @@ __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
   int it = dynamic ? next_item(0, nw, 1, counter, lane) : wid;
   while (it < n_items) {
     const BatchItem item = items[it];
-    if (item.mode == 3) {
+    if (item.mode == 3)
       batch_chunks<K, VEC>(mats + item.mat, sell, item, k, lane);
-    } else {
-      switch (item.lanes) {
-        case 1: batch_rows<1, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-        case 2: batch_rows<2, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-        case 4: batch_rows<4, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-        case 8: batch_rows<8, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-        case 16: batch_rows<16, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-        default: batch_rows<32, K, VEC>(mats + item.mat, rowlist, item, k, lane); break;
-      }
-    }
+    else
+      batch_row_item<K, VEC>(mats + item.mat, rowlist, item, k, lane);
     it = next_item(it, nw, dynamic, counter, lane);
   }
 }
