@@ -121,9 +121,10 @@ __device__ __forceinline__ float ldcs(const float* p) { return __ldcs(p); }
 __device__ __forceinline__ f32n ldcs(const f32n* p) { return f32n{__ldcs(reinterpret_cast<const float*>(p))}; }
 __device__ __forceinline__ int32_t ldcs(const int32_t* p) { return __ldcs(p); }
 
-// Four consecutive entries from a 16-byte (col, float) or 32-byte (double) aligned address.
+// Four consecutive entries from a 16-byte (col, float) or 32-byte (double) aligned address.  The doubles
+// are a whole sector, which nothing reads again: they take no line of L1.
 __device__ __forceinline__ void ldg4(const double* p, double (&x)[4]) {
-  asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];"
                : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3])
                : "l"(p));
 }

@@ -235,18 +235,24 @@ __device__ __forceinline__ void realign(const T (&a)[4], const T (&b)[4], int ph
 // kernel's.  One entry at a time, the 32 lanes of a load touch 32 lines of which each gives 8 or 4
 // bytes, and at 27 entries a row L1 loses most of them before their next use: 569 MB came from DRAM for
 // 330 MB of matrix.  Now every sector is used by the load that fetches it.  On a 27-point stencil of
-// 999,900 rows 131.0 -> 78.5 us (HBM floor 50, FP64 floor 42): the gathers' latency at 40 warps
-// per SM bounds it (FP64 pipe 60 %, DRAM 54 % busy).  Staging a warp's 32 rows in shared memory instead
-// (one bulk copy) took 75 us, but 248 against 93 us at 32 entries a row, where the lanes meet in one
-// bank, and rows of 60 entries left 8 warps on an SM.  An L2 prefetch of the CTAs ahead slows it
-// (77.7 -> 100 us), and so does a second group in flight (48 -> 59 registers: 79.2 us).
+// 999,900 rows 131.0 -> 71.2 us (HBM floor 50, FP64 floor 42): the gathers' latency at 40 warps
+// per SM bounds it, and what L1 keeps for them.  So the doubles take no line there (76.5 -> 74.4 us; the
+// column groups of half a sector must: 110 us without) and CTAs are of 64 threads, whose slots are
+// refilled sooner (128: 72.6, 64: 71.2).  20 million entries in rows of 8 / 16 / 32 / 64, doubles, against 256
+// threads and all in L1: 52.8 -> 49.7, 54.0 -> 49.3, 62.8 -> 52.5, 61.8 -> 51.8 us.  Staging a warp's 32 rows in
+// shared memory instead (one bulk copy) took 75 us, but 248 against 93 us at 32 entries a row, where the
+// lanes meet in one bank, and rows of 60 entries left 8 warps on an SM.  An L2 prefetch of the CTAs
+// ahead slows it (152 ahead 79, 456 100 us), and so do a second group or its columns in flight (79 and
+// 81 us), columns in groups of eight (72 registers: 74.5 us) and more warps with spilled registers (75 us).
+constexpr int kWideThreads = 64;
+
 template <typename VT, int W>
-__global__ void __launch_bounds__(kThreads, (W == 4 ? 3 : 5))
+__global__ void __launch_bounds__(kWideThreads, (W == 4 ? 12 : 20))
     k_crs_wide(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc) {
   grid_dependents();
-  const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int64_t g = (int64_t)blockIdx.x * kWideThreads + threadIdx.x;
   if (g >= n_rows) return;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   double acc[W];
@@ -300,8 +306,8 @@ __global__ void __launch_bounds__(kThreads, (W == 4 ? 3 : 5))
 template <typename VT, int W>
 static cudaError_t launch_wide(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                                cudaStream_t s) {
-  const int64_t grid = (A.n_rows + kThreads - 1) / kThreads;
-  return launch_dependent(k_crs_wide<VT, W>, (unsigned)grid, kThreads, s, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
+  const int64_t grid = (A.n_rows + kWideThreads - 1) / kWideThreads;
+  return launch_dependent(k_crs_wide<VT, W>, (unsigned)grid, kWideThreads, s, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
                           ldc);
 }
 
