@@ -221,11 +221,11 @@ struct spmv_batch_plan {
     cudaStream_t in = nullptr, out = nullptr;
     cudaEvent_t in_done[2] = {nullptr, nullptr}, kern_done[2] = {nullptr, nullptr}, out_done[2] = {nullptr, nullptr};
     std::vector<int64_t> b_off, c_off;  // member offsets (doubles) inside a set
-    bool vec = false;
+    int vec = 1;
     int64_t step = 0;
   } pipe;
   bool io_set = false;
-  bool vec = false;  // 16-byte loads/stores of right-hand-side rows
+  int vec = 1;  // doubles per access of the right-hand-side rows
   // length-sorted SELL copy of the sorted-policy members (rebuilt when the policies change)
   std::vector<int32_t> sell_policies;
   SortedSell sell_host;
@@ -285,7 +285,7 @@ static void free_graph(spmv_batch_plan* b) {
 
 // Graph of one batched product over member table `mats`: counter reset +
 // persistent kernel (the rows-only variant when the list holds no sorted chunks).
-static spmv_status capture_graph(spmv_batch_plan* b, BatchMat* mats, bool vec, cudaGraph_t* graph,
+static spmv_status capture_graph(spmv_batch_plan* b, BatchMat* mats, int vec, cudaGraph_t* graph,
                                  cudaGraphExec_t* exec) {
   int grid = b->num_sms * b->cfg.ctas_per_sm;
   int dynamic = b->cfg.schedule ? 1 : 0;
@@ -412,7 +412,7 @@ static spmv_status pipe_setup(spmv_batch_plan* b) {
       SPMV_CUDA(cudaMemcpy(q.mats[s], t.data(), sizeof(BatchMat) * n, cudaMemcpyHostToDevice));
     }
     // every member's block starts at a multiple of k doubles from a 256-byte aligned base
-    q.vec = b->k % 2 == 0;
+    q.vec = batch_access(4, b->k, q.B[0], b->k, q.C[0], b->k);
   }
   for (int s = 0; s < 2; ++s)
     if (!q.exec[s]) {
@@ -521,15 +521,14 @@ spmv_status spmv_batch_set_io(spmv_batch_handle b, const double* const* B_ptrs, 
   }
   // a replay enqueued earlier (on any stream) may still read the table: wait for it
   SPMV_CUDA(cudaEventSynchronize(b->ev_last));
-  bool vec = (b->k % 2 == 0);
+  int vec = 4;
   for (size_t m = 0; m < b->h_mats.size(); ++m) {
     const int64_t lb = ldb ? ldb[m] : b->k, lc = ldc ? ldc[m] : b->k;
     b->h_mats[m].B = B_ptrs[m];
     b->h_mats[m].C = C_ptrs[m];
     b->h_mats[m].ldb = lb;
     b->h_mats[m].ldc = lc;
-    vec = vec && (lb % 2 == 0) && (lc % 2 == 0) && ((uintptr_t)B_ptrs[m] % 16 == 0) &&
-          ((uintptr_t)C_ptrs[m] % 16 == 0);
+    vec = batch_access(vec, b->k, B_ptrs[m], lb, C_ptrs[m], lc);
   }
   SPMV_CUDA(cudaMemcpy(b->d_mats, b->h_mats.data(), sizeof(BatchMat) * b->h_mats.size(), cudaMemcpyHostToDevice));
   if (vec != b->vec || !b->exec) {

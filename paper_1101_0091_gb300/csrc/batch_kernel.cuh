@@ -47,30 +47,51 @@ struct BatchSell {
 __device__ __forceinline__ void st_c(double* p, double x) { __stcs(p, x); }
 __device__ __forceinline__ void st_c(double2* p, double2 x) { __stcs(p, x); }
 
-// 16-byte loads of two consecutive right-hand-side values when B rows are
-// 16-byte aligned (VEC), else single 8-byte loads.
-template <int K, bool VEC>
+__device__ __forceinline__ void st_c4(double* p, const double* x) {
+  asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(x[0]), "d"(x[1]), "d"(x[2]), "d"(x[3])
+               : "memory");
+}
+
+// A row of k values in accesses of VEC doubles (1, 2, 4).  VEC > 1: every member's B and C rows start on VEC
+// doubles and k is a multiple of VEC.  One lane gathers a whole row, so the accesses are what L1 serves
+// one by one (0.73 of its rate at k = 4 in 16 bytes): 512 members, k = 4, 16 -> 32 bytes 491 -> 475 us, 96 members,
+// k = 8 235 -> 229 us.  Rows are stored in 32 bytes from K = 16 on (96 members, k = 16: 444 -> 392 us); a row of one
+// sector gains nothing (475 -> 479), one of two is mixed (96 members 229 -> 225, 16 members 88 -> 92).
+template <int K, int VEC>
 __device__ __forceinline__ void gather_row(const double* __restrict__ b, int k, double (&g)[K]) {
-  if (VEC && K >= 2) {
 #pragma unroll
-    for (int q = 0; q + 1 < K; q += 2) {
-      if (q < k) {
-        const double2 t = __ldg(reinterpret_cast<const double2*>(b + q));
-        g[q] = t.x;
-        g[q + 1] = t.y;
-      } else {
-        g[q] = 0.0;
-        g[q + 1] = 0.0;
-      }
+  for (int q = 0; q < K; q += VEC) {
+    if (q >= k) {
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) g[q + u] = 0.0;
+    } else if constexpr (VEC == 4) {
+      asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+          : "=d"(g[q]), "=d"(g[q + 1]), "=d"(g[q + 2]), "=d"(g[q + 3])
+          : "l"(b + q));
+    } else if constexpr (VEC == 2) {
+      const double2 t = __ldg(reinterpret_cast<const double2*>(b + q));
+      g[q] = t.x;
+      g[q + 1] = t.y;
+    } else {
+      g[q] = __ldg(b + q);
     }
-  } else {
+  }
+}
+
+template <int K, int VEC>
+__device__ __forceinline__ void store_row(double* out, int k, const double (&acc)[K]) {
+  constexpr int SV = VEC == 4 && K < 16 ? 2 : VEC;  // doubles per store
 #pragma unroll
-    for (int q = 0; q < K; ++q) g[q] = (q < k) ? __ldg(b + q) : 0.0;
+  for (int q = 0; q < K; q += SV) {
+    if (q >= k) break;
+    if constexpr (SV == 4) st_c4(out + q, acc + q);
+    if constexpr (SV == 2) st_c(reinterpret_cast<double2*>(out + q), make_double2(acc[q], acc[q + 1]));
+    if constexpr (SV == 1) st_c(out + q, acc[q]);
   }
 }
 
 // NB entries per lane have their gathers issued before their FMAs.
-template <int L, int K, bool VEC, int NB = (L == 1 && K <= 2 ? 4 / K : 1)>
+template <int L, int K, int VEC, int NB = (L == 1 && K <= 2 ? 4 / K : 1)>
 __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, const int2* __restrict__ rowlist,
                                            const BatchItem& item, int k, int lane) {
   const BatchMat& M = *Mp;  // fields are read where used, not held across the item
@@ -126,14 +147,12 @@ __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, cons
     }
     if (active) {
       double* out = M.C + (int64_t)r * M.ldc;
-      if (VEC && L == 1 && K >= 2) {
-#pragma unroll
-        for (int q = 0; q + 1 < K; q += 2)
-          if (q < k) st_c(reinterpret_cast<double2*>(out + q), make_double2(acc[q], acc[q + 1]));
+      if constexpr (L == 1) {
+        store_row<K, VEC>(out, k, acc);
       } else {
 #pragma unroll
         for (int q = 0; q < K; ++q)
-          if (q < k && (L == 1 || t == q % L)) st_c(out + q, acc[q]);
+          if (q < k && t == q % L) st_c(out + q, acc[q]);
       }
     }
   }
@@ -146,7 +165,7 @@ __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, cons
 // a short row still occupy the FP64 pipe (512 members on 8 lanes per row: 2.77 -> 4.05
 // ms).  So does K = 4, where two a round lengthen the launch (499 -> 507 us), and K = 1
 // (293 -> 301).
-template <int K, bool VEC>
+template <int K, int VEC>
 __device__ __forceinline__ void batch_row_item(const BatchMat* __restrict__ Mp, const int2* __restrict__ rowlist,
                                                const BatchItem& item, int k, int lane) {
   if (K == 2 && item.mode == 2) {
@@ -171,7 +190,7 @@ __device__ __forceinline__ void batch_row_item(const BatchMat* __restrict__ Mp, 
 // Chunks whose rows all have exactly LEN entries, CH chunks per step; returns
 // the first chunk left for the generic loop.  Same FMA order per row as the
 // generic loop.
-template <int LEN, int CH, int K, bool VEC>
+template <int LEN, int CH, int K, int VEC>
 __device__ __forceinline__ int chunks_fixed(const BatchMat* __restrict__ Mp, const double* __restrict__ B,
                                             int64_t ldb, const BatchSell& S, const BatchItem& item, int k,
                                             int lane) {
@@ -207,21 +226,13 @@ __device__ __forceinline__ int chunks_fixed(const BatchMat* __restrict__ Mp, con
         for (int q = 0; q < K; ++q) acc[q] = fma(v[h][j], g[h][j][q], acc[q]);
       if (r[h] < 0) continue;
       double* out = Mp->C + (int64_t)r[h] * Mp->ldc;
-      if (VEC && K >= 2) {
-#pragma unroll
-        for (int q = 0; q + 1 < K; q += 2)
-          if (q < k) st_c(reinterpret_cast<double2*>(out + q), make_double2(acc[q], acc[q + 1]));
-      } else {
-#pragma unroll
-        for (int q = 0; q < K; ++q)
-          if (q < k) st_c(out + q, acc[q]);
-      }
+      store_row<K, VEC>(out, k, acc);
     }
   }
   return c;
 }
 
-template <int K, bool VEC>
+template <int K, int VEC>
 __device__ __forceinline__ void batch_chunks(const BatchMat* __restrict__ Mp, const BatchSell& S,
                                              const BatchItem& item, int k, int lane) {
   struct {
@@ -282,15 +293,7 @@ __device__ __forceinline__ void batch_chunks(const BatchMat* __restrict__ Mp, co
     }
     if (r >= 0) {
       double* out = Mp->C + (int64_t)r * Mp->ldc;
-      if (VEC && K >= 2) {
-#pragma unroll
-        for (int q = 0; q + 1 < K; q += 2)
-          if (q < k) st_c(reinterpret_cast<double2*>(out + q), make_double2(acc[q], acc[q + 1]));
-      } else {
-#pragma unroll
-        for (int q = 0; q < K; ++q)
-          if (q < k) st_c(out + q, acc[q]);
-      }
+      store_row<K, VEC>(out, k, acc);
     }
   }
 }
@@ -318,7 +321,7 @@ __device__ __forceinline__ int next_item(int it, int nw, int dynamic, int* count
 }
 
 // Persistent kernel over row items (modes 0-2).
-template <int K, bool VEC>
+template <int K, int VEC>
 __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
     k_batch_rows(const BatchMat* __restrict__ mats, const BatchItem* __restrict__ items, int n_items,
                  const int2* __restrict__ rowlist, int* __restrict__ counter, int dynamic, int k) {
@@ -337,7 +340,7 @@ __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
 // one member stay next to each other in the list, so a member's B block is
 // gathered while it is resident in L2 (two separate kernels, one per mode,
 // would stream every B block twice).
-template <int K, bool VEC>
+template <int K, int VEC>
 __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
     k_batch(const BatchMat* __restrict__ mats, const BatchItem* __restrict__ items, int n_items,
             const int2* __restrict__ rowlist, BatchSell sell, int* __restrict__ counter, int dynamic, int k) {
@@ -355,34 +358,45 @@ __global__ void __launch_bounds__(kBatchThreads, BatchMinCtas<K>::value)
   }
 }
 
-template <bool VEC>
+template <int VEC>
 static const void* batch_rows_kernel_t(int k) {
-  if (k <= 1) return (const void*)k_batch_rows<1, false>;
-  if (k <= 2) return (const void*)k_batch_rows<2, VEC>;
-  if (k == 3) return (const void*)k_batch_rows<3, false>;
+  if constexpr (VEC == 1) {
+    if (k == 1) return (const void*)k_batch_rows<1, 1>;
+    if (k == 3) return (const void*)k_batch_rows<3, 1>;
+  }
+  if constexpr (VEC <= 2)
+    if (k <= 2) return (const void*)k_batch_rows<2, VEC>;
   if (k <= 4) return (const void*)k_batch_rows<4, VEC>;
   if (k <= 8) return (const void*)k_batch_rows<8, VEC>;
   return (const void*)k_batch_rows<16, VEC>;
 }
 
-template <bool VEC>
+template <int VEC>
 static const void* batch_kernel_t(int k) {
-  if (k <= 1) return (const void*)k_batch<1, false>;
-  if (k <= 2) return (const void*)k_batch<2, VEC>;
-  if (k == 3) return (const void*)k_batch<3, false>;  // (as four columns, one masked: 603.6 us for 512 members, 562.1 so)
+  if constexpr (VEC == 1) {
+    if (k == 1) return (const void*)k_batch<1, 1>;
+    if (k == 3) return (const void*)k_batch<3, 1>;  // (as four columns, one masked: 603.6 us for 512 members, 562.1 so)
+  }
+  if constexpr (VEC <= 2)
+    if (k <= 2) return (const void*)k_batch<2, VEC>;
   if (k <= 4) return (const void*)k_batch<4, VEC>;
   if (k <= 8) return (const void*)k_batch<8, VEC>;
   return (const void*)k_batch<16, VEC>;
 }
 
-// The kernels for k right-hand sides; vec: every member's B and C rows are
-// 16-byte aligned and k is even (16-byte loads and stores).  The rows-only
+// The kernels for k right-hand sides in accesses of vec doubles.  The rows-only
 // variant serves work lists without sorted chunks.
-static inline const void* batch_rows_kernel(int k, bool vec) {
-  return vec ? batch_rows_kernel_t<true>(k) : batch_rows_kernel_t<false>(k);
+static inline const void* batch_rows_kernel(int k, int vec) {
+  return vec == 4 ? batch_rows_kernel_t<4>(k) : vec == 2 ? batch_rows_kernel_t<2>(k) : batch_rows_kernel_t<1>(k);
 }
-static inline const void* batch_kernel(int k, bool vec) {
-  return vec ? batch_kernel_t<true>(k) : batch_kernel_t<false>(k);
+static inline const void* batch_kernel(int k, int vec) {
+  return vec == 4 ? batch_kernel_t<4>(k) : vec == 2 ? batch_kernel_t<2>(k) : batch_kernel_t<1>(k);
+}
+
+// Doubles per access (at most `most`) that k columns of a member with these operands allow.
+static inline int batch_access(int most, int k, const double* B, int64_t ldb, const double* C, int64_t ldc) {
+  while (most > 1 && (k % most || ldb % most || ldc % most || ((uintptr_t)B | (uintptr_t)C) % (8 * most))) most /= 2;
+  return most;
 }
 
 }  // namespace spmv

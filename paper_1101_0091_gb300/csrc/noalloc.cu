@@ -69,7 +69,7 @@ extern "C" spmv_status spmv_batch_apply_noalloc(int32_t count, const int64_t* n_
   BatchMat* table = reinterpret_cast<BatchMat*>(g_noalloc_host + kNoAllocCounterBytes);
   BatchItem* items = reinterpret_cast<BatchItem*>(g_noalloc_host + kNoAllocItemsOffset);
   size_t n_items = 0;
-  bool vec = (k % 2 == 0);
+  int vec = 4;
   for (int m = 0; m < count; ++m) {
     const int L = lanes ? lanes[m] : 1;
     if (L != 1 && L != 2 && L != 4 && L != 8 && L != 16 && L != 32)
@@ -80,7 +80,7 @@ extern "C" spmv_status spmv_batch_apply_noalloc(int32_t count, const int64_t* n_
     if (n_rows[m] > 0 && (!row_ptr_dev[m] || !col_dev[m] || !val_dev[m] || !B_dev[m] || !C_dev[m]))
       return fail(SPMV_ERR_ARG, "NULL row_ptr, col, val, B or C of member " + std::to_string(m) + " (it has rows)");
     table[m] = BatchMat{row_ptr_dev[m], col_dev[m], val_dev[m], B_dev[m], C_dev[m], lb, lc, n_rows[m]};
-    vec = vec && lb % 2 == 0 && lc % 2 == 0 && (uintptr_t)B_dev[m] % 16 == 0 && (uintptr_t)C_dev[m] % 16 == 0;
+    vec = batch_access(vec, k, B_dev[m], lb, C_dev[m], lc);
     const int64_t per = (int64_t)(32 / L) * kNoAllocPasses;
     for (int64_t r0 = 0; r0 < n_rows[m]; r0 += per) {
       if (n_items == kNoAllocMaxItems)
