@@ -253,44 +253,46 @@ __device__ __forceinline__ void batch_chunks(const BatchMat* __restrict__ Mp, co
     double acc[K];
 #pragma unroll
     for (int q = 0; q < K; ++q) acc[q] = 0.0;
-    constexpr int NB = K <= 2 ? 4 / K : 1;  // gathers issued before their FMAs
-    if (NB == 1) {
-      // one slot per step, software-pipelined: the next slot's val/col load is in flight
-      // while this slot's gathers are, so only the gathers stay on the critical path
-      double v = len > 0 ? ldcs(S.val + base) : 0.0;
-      int32_t cc = len > 0 ? ldcs(S.col + base) : 0;
-      for (int j = 0; j < len; ++j) {
-        double g[K];
-        gather_row<K, VEC>(M.B + (int64_t)cc * M.ldb, k, g);
-        const int64_t nxt = base + (int64_t)(j + 1 < len ? j + 1 : j) * 32;
-        const double v_n = ldcs(S.val + nxt);
-        const int32_t c_n = ldcs(S.col + nxt);
+    // NB slots a step, software-pipelined: the next step's values and columns are in flight while this
+    // step's gathers are, so only the gathers stay on the critical path.  512 members, against four / two slots
+    // without the pipeline at k = 1 / 2 and one slot with it at k = 4: 287 -> 281, 334 -> 330, 476 -> 468 us.
+    constexpr int NB = K == 1 ? 4 : K <= 4 ? 2 : 1;
+    double v[NB];
+    int32_t cc[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      v[u] = u < len ? ldcs(S.val + base + u * 32) : 0.0;
+      cc[u] = u < len ? ldcs(S.col + base + u * 32) : 0;
+    }
+    int j = 0;
+    for (; j + NB <= len; j += NB) {
+      double g[NB][K], vn[NB];
+      int32_t cn[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) gather_row<K, VEC>(M.B + (int64_t)cc[u] * M.ldb, k, g[u]);
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int64_t nxt = base + (int64_t)(j + NB + u < len ? j + NB + u : j) * 32;
+        vn[u] = ldcs(S.val + nxt);
+        cn[u] = ldcs(S.col + nxt);
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
 #pragma unroll
         for (int q = 0; q < K; ++q)
-          if (q < k) acc[q] = fma(v, g[q], acc[q]);
-        v = v_n;
-        cc = c_n;
-      }
-    } else {
-      for (int j = 0; j < len; j += NB) {
-        double v[NB];
-        const double* b[NB];
+          if (q < k) acc[q] = fma(v[u], g[u][q], acc[q]);
 #pragma unroll
-        for (int u = 0; u < NB; ++u) {
-          const int64_t slot = base + (int64_t)((j + u < len) ? j + u : j) * 32;
-          v[u] = ldcs(S.val + slot);
-          b[u] = M.B + (int64_t)ldcs(S.col + slot) * M.ldb;
-        }
-        double g[NB][K];
-#pragma unroll
-        for (int u = 0; u < NB; ++u) gather_row<K, VEC>(b[u], k, g[u]);
-#pragma unroll
-        for (int u = 0; u < NB; ++u)
-#pragma unroll
-          for (int q = 0; q < K; ++q)
-            if (j + u < len && q < k) acc[q] = fma(v[u], g[u][q], acc[q]);
-      }
+      for (int u = 0; u < NB; ++u) v[u] = vn[u], cc[u] = cn[u];
     }
+#pragma unroll
+    for (int u = 0; u < NB - 1; ++u)
+      if (j + u < len) {
+        double g[K];
+        gather_row<K, VEC>(M.B + (int64_t)cc[u] * M.ldb, k, g);
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+          if (q < k) acc[q] = fma(v[u], g[q], acc[q]);
+      }
     if (r >= 0) {
       double* out = Mp->C + (int64_t)r * Mp->ldc;
       store_row<K, VEC>(out, k, acc);
