@@ -15,8 +15,8 @@
 // order, so every W gives the same bits.  Here a lane stops at its row's own
 // length (from the CRS row_ptr): a warp's rows are fewer than a chunk's, and the
 // padding that they leave out is FP64 work, which bounds these products (600,011-row
-// eigenproblem matrix, k = 6: 106.3 -> 96.7 us, FP64 floor 79).  One vector is bound by
-// the SMs' requests to L2 on scattered matrices (2,000,003 rows: 95.7 us, request
+// eigenproblem matrix, k = 6: 106.3 -> 96.7 us, now 93.9, FP64 floor 79).  One vector is bound by
+// the SMs' requests to L2 on scattered matrices (2,000,003 rows: 92.3 us, request
 // floor 73); there the two dependent loads in front of each row cost more than
 // its padding (99.9 us).
 #include "device.cuh"
@@ -58,25 +58,42 @@ __global__ void __launch_bounds__(kThreads)
   const int64_t base = __ldg(chunk_ptr + c) + t;
   grid_wait();
   double acc = 0.0;
-  // batches of NB slots: all gathers of a batch are issued before its FMAs (len is the warp's, so
-  // the last slots take a branch, not masked multiply-adds)
+  // batches of NB slots, software-pipelined: all gathers of a batch are issued before its FMAs, and behind
+  // them the next batch's values and columns (len is the warp's, so the last slots take a branch, not
+  // masked multiply-adds).  Without and with the pipeline: eigenproblem matrices of 400,009 / 2,000,003 rows
+  // 23.9 -> 22.8, 93.3 -> 92.3 us; 130^3 Poisson 40.4 -> 36.3 (FP32 values 35.0 -> 29.7; HBM floor 33 and 24).
   constexpr int NB = 2;
+  VT v[NB];
+  int32_t cc[NB];
+#pragma unroll
+  for (int u = 0; u < NB; ++u) {
+    v[u] = VT();
+    cc[u] = 0;
+    if (u < len) {
+      v[u] = ldcs(val + base + u * kSellC);
+      cc[u] = ldcs(col + base + u * kSellC);
+    }
+  }
   int j = 0;
   for (; j + NB <= len; j += NB) {
-    double v[NB], g[NB];
+    double g[NB];
+    VT vn[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) g[u] = B[(int64_t)cc[u] * ldb];
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const int64_t slot = base + (int64_t)(j + u) * kSellC;
-      v[u] = to_f64(ldcs(val + slot));
-      g[u] = B[(int64_t)ldcs(col + slot) * ldb];
+      const int64_t nxt = base + (int64_t)(j + NB + u < len ? j + NB + u : j) * kSellC;
+      vn[u] = ldcs(val + nxt);
+      cc[u] = ldcs(col + nxt);
     }
 #pragma unroll
-    for (int u = 0; u < NB; ++u) acc = fma(v[u], g[u], acc);
+    for (int u = 0; u < NB; ++u) acc = fma(to_f64(v[u]), g[u], acc);
+#pragma unroll
+    for (int u = 0; u < NB; ++u) v[u] = vn[u];
   }
-  for (; j < len; ++j) {
-    const int64_t slot = base + (int64_t)j * kSellC;
-    acc = fma(to_f64(ldcs(val + slot)), B[(int64_t)ldcs(col + slot) * ldb], acc);
-  }
+#pragma unroll
+  for (int u = 0; u < NB - 1; ++u)
+    if (j + u < len) acc = fma(to_f64(v[u]), B[(int64_t)cc[u] * ldb], acc);
   if (r >= n_rows) return;
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
 }
@@ -111,12 +128,34 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   const double* Bc = B + c0;
   const VT* vp = val + base;
   const int32_t* cp = col + base;
-  for (int j = 0; j < len; ++j) {
-    const double v = to_f64(ldcs(vp + j * kSellC));
-    double g[W];
-    load_cols(Bc + (int64_t)ldcs(cp + j * kSellC) * ldb, g);
+  double g[W];
+  if constexpr (W == 2 || W == 3) {
+    // The next slot's value and column are in flight while this slot's gathers are: 600,011 rows, k = 6
+    // 94.8 -> 93.7 us; 400,009 rows, k = 2 / 3 / 4 28.6 -> 27.7, 44.5 -> 42.5, 46.0 -> 45.5; 130^3 Poisson, k = 2 / 4
+    // 61.2 -> 56.9, 109.1 -> 105.5.  Not with one column a lane (100,003 rows, k = 4: 15.8 -> 16.8) nor with five
+    // (400,009 rows, k = 5: 63.2 -> 65.4) or seven (Poisson, FP32 values 179.5 -> 182.3).
+    if (len > 0) {
+      VT v = ldcs(vp);
+      int32_t c = ldcs(cp);
+      for (int j = 1; j < len; ++j) {
+        load_cols(Bc + (int64_t)c * ldb, g);
+        const VT vn = ldcs(vp + j * kSellC);
+        c = ldcs(cp + j * kSellC);
 #pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
+        for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
+        v = vn;
+      }
+      load_cols(Bc + (int64_t)c * ldb, g);
+#pragma unroll
+      for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
+    }
+  } else {
+    for (int j = 0; j < len; ++j) {
+      const double v = to_f64(ldcs(vp + j * kSellC));
+      load_cols(Bc + (int64_t)ldcs(cp + j * kSellC) * ldb, g);
+#pragma unroll
+      for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
+    }
   }
   store_cols(C + (int64_t)row * ldc + c0, acc);
 }
