@@ -97,11 +97,20 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 }
 
 // Programmatic dependent launch (launch_dependent, internal.h): grid_dependents lets the next kernel of
-// the stream be launched as soon as every CTA of this one has got here, so that its CTAs take the slots
-// that this kernel's last ones leave; grid_wait holds a kernel launched that way until the work before
-// it is complete and visible.  Before grid_wait a kernel reads its plan's own arrays only, and what
-// earlier work may have written (B, the solvers' vectors and scalars) is read with plain loads: a
+// the stream be launched as soon as every CTA of this one has got here (or has exited), so that its CTAs
+// take the slots that this kernel's last ones leave; grid_wait holds a kernel launched that way until the
+// work before it is complete and visible.  Before grid_wait a kernel reads its plan's own arrays only, and
+// what earlier work may have written (B, the solvers' vectors and scalars) is read with plain loads: a
 // read-only load (ld.global.nc, __ldg, const __restrict__) could be moved above the wait.
+//
+// grid_dependents comes after grid_wait, never before: ahead of it, products that fit on the chip several
+// times over are launched on top of one another, and the last ones crowd onto the SMs that empty first
+// (256^2 Laplacian in a CUDA graph 3.9 us, 2.2 now; eigenproblem matrix of 50,001 rows 9.5 us, 6.5 now).  The
+// kernels whose CTAs differ most in time, or that fit on the chip at once, call it in front of their
+// stores, for the same reason: eigenproblem matrix of 200,003 rows 15.0 -> 11.4 us, 27-point stencil 48^3
+// 13.9 -> 9.1, 400^2 Laplacian 4.5 -> 3.5.  Larger grids of even work overlap more of the next launch with
+// their last wave and call it at once (131 x 127 x 129 Poisson, k = 3: 77.8 us, in front of the stores 80.0).
+constexpr unsigned kOneWave = 152 * 8;  // CTAs of kThreads that the chip holds
 __device__ __forceinline__ void grid_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

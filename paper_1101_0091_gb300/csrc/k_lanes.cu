@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(kThreads, 8)
     k_crs_row(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
               int64_t ldc, int prefetch) {
-  grid_dependents();
   if (threadIdx.x == 0 && prefetch > 0)
     prefetch_rows(((int64_t)blockIdx.x + prefetch) * kThreads, kThreads, n_rows, row_ptr, col, val);
   const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
@@ -133,6 +132,7 @@ __global__ void __launch_bounds__(kThreads, 8)
   int j = __ldg(row_ptr + g);
   const int re = __ldg(row_ptr + g + 1);
   grid_wait();
+  if (gridDim.x > 4 * kOneWave) grid_dependents();
   double acc[1] = {0.0};
   for (; j + 4 <= re; j += 4) {
     const VT* vj = val + j;
@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     }
   }
   add_tail(re - j, v, x, acc);
+  grid_dependents();
   C[g * ldc] = acc[0];
 }
 
@@ -164,12 +165,12 @@ template <typename VT>
 __global__ void __launch_bounds__(kThreads, 8)
     k_crs_halo(int64_t n_rows, const int32_t* __restrict__ rows, const int32_t* __restrict__ row_ptr,
                const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B, double* C) {
-  grid_dependents();
   const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (g >= n_rows) return;
   const int64_t row = __ldg(rows + g);
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   grid_wait();
+  grid_dependents();
   const double c = C[row];
   double acc = 0.0;
   for (int j = rs; j < re; ++j) acc = fma(to_f64(ldg(val + j)), B[ldg(col + j)], acc);
@@ -182,7 +183,6 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_crs_cols(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc, int G, int prefetch) {
-  grid_dependents();
   const int rpc = kThreads / G;  // rows per CTA
   if (threadIdx.x == 0 && prefetch > 0)
     prefetch_rows(((int64_t)blockIdx.x + prefetch) * rpc, rpc, n_rows, row_ptr, col, val);
@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   const int c0 = ((int)threadIdx.x - r * G) * W;  // first column of this lane
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   grid_wait();
+  if (gridDim.x > kOneWave) grid_dependents();
   double acc[W];
 #pragma unroll
   for (int q = 0; q < W; ++q) acc[q] = 0.0;
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[q] = fma(v, gv[q], acc[q]);
   }
+  grid_dependents();
   store_cols(C + g * ldc + c0, acc);
 }
 
@@ -251,7 +253,6 @@ __global__ void __launch_bounds__(kWideThreads, (W == 4 ? 12 : 20))
     k_crs_wide(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc) {
-  grid_dependents();
   const int64_t g = (int64_t)blockIdx.x * kWideThreads + threadIdx.x;
   if (g >= n_rows) return;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
@@ -300,6 +301,7 @@ __global__ void __launch_bounds__(kWideThreads, (W == 4 ? 12 : 20))
       ca[u] = cb[u];
     }
   }
+  grid_dependents();
   store_cols(C + g * ldc, acc);
 }
 
@@ -361,7 +363,6 @@ __global__ void __launch_bounds__(kThreads, 8)
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
                int64_t ldc, int k, int short_row, int prefetch) {
   __shared__ double sh[kThreads];
-  grid_dependents();
   constexpr int WARPS = kThreads / 32;
   const int tid = (int)threadIdx.x;
   int64_t blk = blockIdx.x;
@@ -386,6 +387,7 @@ __global__ void __launch_bounds__(kThreads, 8)
   if (r >= rpc || g >= n_rows) return;
   const int rs = __ldg(row_ptr + g), re = __ldg(row_ptr + g + 1);
   grid_wait();
+  grid_dependents();
   if (re - rs > short_row) return;
   const double* Bc = B + (tid - r * k);
   double acc = 0.0;

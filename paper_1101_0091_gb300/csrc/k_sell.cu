@@ -45,7 +45,6 @@ __global__ void __launch_bounds__(kThreads)
            const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
            const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B,
            int64_t ldb, double* C, int64_t ldc, int prefetch) {
-  grid_dependents();
   constexpr int CPC = kThreads / kSellC;  // chunks per CTA
   // bring the slots of the CTA `prefetch` positions ahead into L2
   if (threadIdx.x == 0 && prefetch > 0)
@@ -94,6 +93,7 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
   for (int u = 0; u < NB - 1; ++u)
     if (j + u < len) acc = fma(to_f64(v[u]), B[(int64_t)cc[u] * ldb], acc);
+  grid_dependents();
   if (r >= n_rows) return;
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
 }
@@ -105,7 +105,6 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
                 const int32_t* __restrict__ col, const VT* __restrict__ val, const double* B,
                 int64_t ldb, double* C, int64_t ldc, int G, int prefetch) {
-  grid_dependents();
   const int rpc = kThreads / G;  // sorted rows per CTA
   if (threadIdx.x == 0 && prefetch > 0) {
     // the chunks that start in the rows of the CTA `prefetch` positions ahead
@@ -157,6 +156,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
       for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
     }
   }
+  grid_dependents();
   store_cols(C + (int64_t)row * ldc + c0, acc);
 }
 

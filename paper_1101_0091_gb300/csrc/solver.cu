@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(kVecThreads) k_cg_init(int64_t n, int k, const
                                                          double* P, double* rr_partial,
                                                          double* bb_partial) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   double rr[G::KC], bb[G::KC];
 #pragma unroll
@@ -260,8 +260,8 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads) k_cg_begin(int k, const double* rr_partial, const double* bb_partial,
                                                           unsigned n_partials, CgScalars* S, double rtol2) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   __shared__ int n_active;
   const int c = threadIdx.x;
@@ -286,8 +286,8 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2) k_cg_dot(int64_t n, int k, const double* P,
                                                            const double* Q, double* partial) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   double acc[G::KC];
 #pragma unroll
@@ -313,8 +313,8 @@ __global__ void __launch_bounds__(kVecThreads, 2)
     k_cg_update(int64_t n, int k, double* R, const double* Q, const double* pq_partial,
                 double* rr_partial, CgScalars* S) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   __shared__ double s_alpha[kMaxCols];
   __shared__ int s_run[kMaxCols];
@@ -373,8 +373,8 @@ __global__ void __launch_bounds__(kVecThreads, 2)
     k_cg_direction(int64_t n, int k, double* X, const double* R, double* P,
                    const double* rr_partial, CgScalars* S) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   __shared__ double s_alpha[kMaxCols], s_beta[kMaxCols];
   __shared__ int s_run[kMaxCols], s_next[kMaxCols];
@@ -441,8 +441,8 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, const double* V0,
                                                             double* partial) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   double acc[G::KC];
 #pragma unroll
@@ -471,8 +471,8 @@ __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_alpha(int64_t n, int k, double* W, const double* u, const double* u_prev, const double* uu_partial,
                double* wu_partial, LzScalars* S, double* beta_out) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   __shared__ double s_inv[kMaxCols], s_prev[kMaxCols];
   Walk<G> w(n, k);
@@ -528,8 +528,8 @@ __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_beta(int64_t n, int k, double* W, const double* u, const double* wu_partial, double* uu_partial,
               LzScalars* S, double* alpha_out) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   __shared__ double s_a[kMaxCols];
   Walk<G> w(n, k);
@@ -579,8 +579,8 @@ template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads) k_lz_end(int k, const double* uu_partial, unsigned n_partials,
                                                         const LzScalars* S, double* beta_out) {
   using G = Seg<K, MODE>;
-  grid_dependents();
   grid_wait();
+  grid_dependents();
   __shared__ VecShared sh;
   const double uu = read_partials<G>(uu_partial, n_partials, k, sh);
   if ((int)threadIdx.x < k) beta_out[threadIdx.x] = S->live_old[threadIdx.x] ? sqrt(uu) : 0.0;
