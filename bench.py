@@ -703,9 +703,9 @@ def ordering_forms(A, torch, spmv, pm, timer, stream, B, C, workload, steps=100)
 
 def cg_bytes_per_iteration(pm, A, k: int) -> int:
     """Algorithmic bytes of one CG iteration of the library: the SpMM's V_min
-    (P read, Q written) + alpha (read P, Q) + update (read X, P, R, Q; write
-    X, R) + direction (read R, P; write P): V_min + 88 k n bytes."""
-    return pm.gpu_min_traffic(A.n_rows, A.n_cols, A.nnz, k=k).bytes_min + 88 * k * A.n_rows
+    (P read, Q written) + alpha (read P, Q) + update (read R, Q; write R) +
+    direction (read X, R, P; write X, P): V_min + 80 k n bytes."""
+    return pm.gpu_min_traffic(A.n_rows, A.n_cols, A.nnz, k=k).bytes_min + 80 * k * A.n_rows
 
 
 def cg_forms(A, torch, spmv, pm, stream, iters: int = 50):
@@ -718,7 +718,7 @@ def cg_forms(A, torch, spmv, pm, stream, iters: int = 50):
     out = {"method": "CG (Hestenes-Stiefel), k independent columns, graph-replayed iterations",
            "iterations": iters,
            "bound": "SpMM at max(HBM, FP64-pipe) time of its V_min and 2k nnz flops, plus the vector "
-                    "kernels' 88 k n bytes at the measured copy peak (the kernels run one after another)"}
+                    "kernels' 80 k n bytes at the measured copy peak (the kernels run one after another)"}
     for k in (1, 4, 8, 16):
         # k = 1 is HBM-bound; k >= 2 is FP64-pipe-bound, where CRS_L1 runs its column-split form
         with spmv.Plan.from_csr(A, variant=spmv.SPMV_CRS_L1) as p:
@@ -739,7 +739,7 @@ def cg_forms(A, torch, spmv, pm, stream, iters: int = 50):
         byts = cg_bytes_per_iteration(pm, A, k)
         spmm = pm.gpu_min_traffic(A.n_rows, A.n_cols, A.nnz, k=k)
         t_bound = (max(spmm.bytes_min / (hbm * 1e9), spmm.flops / (fp64_peak() * 1e9))
-                   + 88 * k * A.n_rows / (hbm * 1e9))
+                   + 80 * k * A.n_rows / (hbm * 1e9))
         out[f"k{k}"] = {"plan_variant": "crs_l1",
                         "us_per_iteration": round(t_it * 1e6, 1), "gflops": round(flops / t_it / 1e9, 1),
                         "hbm_gbs": round(byts / t_it / 1e9, 1), "bytes_per_iteration": byts,
@@ -754,8 +754,8 @@ def cg_forms(A, torch, spmv, pm, stream, iters: int = 50):
 def lanczos_forms(A, torch, spmv, pm, stream, m: int = 30):
     """Lanczos (no reorthogonalisation) on k start vectors through the
     selector's SELL-32-4096 plan: time per step.  Bytes per step: V_min(k) +
-    alpha (read W, v, v_prev; write W) + beta (read W, v; write W) + scale
-    (read W; write v) = V_min + 72 k n."""
+    alpha (read W, v, v_prev; write W) + beta (read W, v; write W) = V_min +
+    56 k n."""
     import gen
     hbm, _ = measured_hbm()
     out = {"method": "Lanczos three-term recurrence, k independent start vectors", "steps": m}
@@ -773,9 +773,9 @@ def lanczos_forms(A, torch, spmv, pm, stream, m: int = 30):
                     ts.append(time.perf_counter() - t0)
             t_it = min(ts) / m
             spmm = pm.gpu_min_traffic(A.n_rows, A.n_cols, A.nnz, k=k)
-            byts = spmm.bytes_min + 72 * k * A.n_rows
+            byts = spmm.bytes_min + 56 * k * A.n_rows
             t_bound = (max(spmm.bytes_min / (hbm * 1e9), spmm.flops / (fp64_peak() * 1e9))
-                       + 72 * k * A.n_rows / (hbm * 1e9))
+                       + 56 * k * A.n_rows / (hbm * 1e9))
             out[f"k{k}"] = {"us_per_step": round(t_it * 1e6, 1),
                             "gflops": round((2 * k * A.nnz + 8 * k * A.n_rows) / t_it / 1e9, 1),
                             "hbm_gbs": round(byts / t_it / 1e9, 1), "bound_us": round(t_bound * 1e6, 1),
