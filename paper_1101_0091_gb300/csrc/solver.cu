@@ -462,10 +462,9 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, co
 
 // The Lanczos vectors stay unscaled: u_j = |u_j| v_j, where |u_j| = beta_{j-1} and inv_j = 1 / |u_j| (0 for
 // a column that has stopped).  W (= A u_j) becomes A v_j - beta_{j-1} v_{j-1} = inv_j W - (beta_{j-1}
-// inv_{j-1}) u_{j-1}; column sums of W.u_j.  The pass that divided W by its norm is gone (k = 4, 500,009 rows:
-// 92.2 -> 89.2 us a step; seven vector
-// passes instead of nine).  beta_{j-1} comes from the partials of u_j.u_j; it is stored to
-// beta_out unless that is NULL (j = 1: |V0|, every column live before).
+// inv_{j-1}) u_{j-1}; column sums of W.u_j.  The pass that divided W by its norm is gone (seven vector passes
+// instead of nine; k = 4, 500,009 rows: 92.2 -> 89.2 us a step).  beta_{j-1} comes from the partials of
+// u_j.u_j; it is stored to beta_out unless that is NULL (j = 1: |V0|, every column live before).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_alpha(int64_t n, int k, double* W, const double* u, const double* u_prev, const double* uu_partial,
