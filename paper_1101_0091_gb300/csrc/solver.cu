@@ -28,8 +28,8 @@ constexpr int kMaxCols = 16;
 
 // Per-column scalars.  Every CTA of a kernel reads them and CTA 0 writes, so no kernel writes a field
 // that it reads: k_cg_direction writes rr, active, iters and n_active, k_cg_update the others, with
-// copies (rr_old) or working sets (running) of what k_cg_direction needs; k_lz_alpha writes inv and
-// live, k_lz_beta their copies.
+// copies (rr_old) or working sets (running) of what k_cg_direction needs; k_lz_alpha writes uu, scale
+// and live, k_lz_beta their copies.
 struct CgScalars {
   double rr[kMaxCols], rr_old[kMaxCols], tol2[kMaxCols], alpha[kMaxCols];
   int active[kMaxCols], running[kMaxCols], iters[kMaxCols], breakdown[kMaxCols];
@@ -37,7 +37,7 @@ struct CgScalars {
 };
 
 struct LzScalars {
-  double inv[kMaxCols], inv_old[kMaxCols];
+  double uu[kMaxCols], uu_old[kMaxCols], scale[kMaxCols], scale_old[kMaxCols];
   int live[kMaxCols], live_old[kMaxCols];
 };
 
@@ -460,11 +460,17 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, co
   write_partial<G>(acc, k, partial, sh);
 }
 
-// The Lanczos vectors stay unscaled: u_j = |u_j| v_j, where |u_j| = beta_{j-1} and inv_j = 1 / |u_j| (0 for
-// a column that has stopped).  W (= A u_j) becomes A v_j - beta_{j-1} v_{j-1} = inv_j W - (beta_{j-1}
-// inv_{j-1}) u_{j-1}; column sums of W.u_j.  The pass that divided W by its norm is gone (seven vector passes
-// instead of nine; k = 4, 500,009 rows: 92.2 -> 89.2 us a step).  beta_{j-1} comes from the partials of
-// u_j.u_j; it is stored to beta_out unless that is NULL (j = 1: |V0|, every column live before).
+// The beta of the step before, from uu = u_j.u_j.
+__device__ __forceinline__ double last_beta(const LzScalars* S, int c, double uu) {
+  return S->live_old[c] ? sqrt(uu / S->uu_old[c]) / S->scale_old[c] : 0.0;
+}
+
+// The Lanczos vectors are not normalised: u_j = |u_j| v_j, and the pass that divided by the norm is gone
+// (seven vector passes instead of nine; k = 4, 500,009 rows: 92.2 -> 89.2 us a step).  W (= A u_j) is scaled by
+// s_j, a power of two near 1 / |u_j| (0 for a column that has stopped), so that nothing is rounded, and
+// becomes s_j |u_j| (A v_j - beta_{j-1} v_{j-1}) = s_j W - (s_j u_j.u_j / s_{j-1} u_{j-1}.u_{j-1}) u_{j-1}; column sums
+// of W.u_j.  Each column scalar is one quotient of such sums: its error is alike in every row.  beta_{j-1} is
+// |u_j| / (s_{j-1} |u_{j-1}|), stored to beta_out unless that is NULL (j = 1: |V0|, every column live before).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_alpha(int64_t n, int k, double* W, const double* u, const double* u_prev, const double* uu_partial,
@@ -482,14 +488,15 @@ __global__ void __launch_bounds__(kVecThreads, 2)
   const int c = threadIdx.x;
   if (c < k) {
     const bool first = beta_out == nullptr;
-    const double b = first || S->live_old[c] ? sqrt(uu) : 0.0;
-    const bool live = b > 0.0;
-    s_inv[c] = live ? 1.0 / b : 0.0;
-    s_prev[c] = !first && live ? b * S->inv_old[c] : 0.0;
+    const bool live = (first || S->live_old[c]) && uu > 0.0;
+    const double scale = live ? ldexp(1.0, -(ilogb(uu) >> 1)) : 0.0;
+    s_inv[c] = scale;
+    s_prev[c] = !first && live ? scale * uu / (S->scale_old[c] * S->uu_old[c]) : 0.0;
     if (blockIdx.x == 0) {
-      if (!first) beta_out[c] = b;
+      if (!first) beta_out[c] = last_beta(S, c, uu);
       S->live[c] = live;
-      S->inv[c] = s_inv[c];
+      S->scale[c] = scale;
+      S->uu[c] = uu;
     }
   }
   __syncthreads();
@@ -521,7 +528,8 @@ __global__ void __launch_bounds__(kVecThreads, 2)
   write_partial<G>(acc, k, wu_partial, sh);
 }
 
-// alpha_j = W.v_j (live columns), stored to alpha_out; W = W - alpha_j v_j = u_{j+1}; column sums of W.W.
+// alpha_j = W.u_j / (s_j u_j.u_j) (live columns), stored to alpha_out; W = W - (W.u_j / u_j.u_j) u_j = u_{j+1}; column
+// sums of W.W.
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_beta(int64_t n, int k, double* W, const double* u, const double* wu_partial, double* uu_partial,
@@ -538,11 +546,12 @@ __global__ void __launch_bounds__(kVecThreads, 2)
   const double wu = read_partials<G>(wu_partial, gridDim.x, k, sh);
   const int c = threadIdx.x;
   if (c < k) {
-    const double inv = S->inv[c], alpha = S->live[c] ? wu * inv : 0.0;
-    s_a[c] = alpha * inv;
+    const bool live = S->live[c];
+    s_a[c] = live ? wu / S->uu[c] : 0.0;
     if (blockIdx.x == 0) {
-      alpha_out[c] = alpha;
-      S->inv_old[c] = inv;
+      alpha_out[c] = live ? wu / (S->scale[c] * S->uu[c]) : 0.0;
+      S->uu_old[c] = S->uu[c];
+      S->scale_old[c] = S->scale[c];
       S->live_old[c] = S->live[c];
     }
   }
@@ -582,7 +591,7 @@ __global__ void __launch_bounds__(kVecThreads) k_lz_end(int k, const double* uu_
   grid_dependents();
   __shared__ VecShared sh;
   const double uu = read_partials<G>(uu_partial, n_partials, k, sh);
-  if ((int)threadIdx.x < k) beta_out[threadIdx.x] = S->live_old[threadIdx.x] ? sqrt(uu) : 0.0;
+  if ((int)threadIdx.x < k) beta_out[threadIdx.x] = last_beta(S, threadIdx.x, uu);
 }
 
 // ---------------------------------------------------------------- dispatch
