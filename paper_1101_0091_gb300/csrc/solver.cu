@@ -460,9 +460,57 @@ __global__ void __launch_bounds__(kVecThreads, 2) k_lz_norm(int64_t n, int k, co
   write_partial<G>(acc, k, partial, sh);
 }
 
-// The beta of the step before, from uu = u_j.u_j.
+// A power of two near 1 / sqrt(uu): a vector of squared norm uu > 0 is scaled by it without rounding, to a
+// squared norm of 1 .. 4.
+__device__ __forceinline__ double unit_scale(double uu) { return ldexp(1.0, -(ilogb(uu) >> 1)); }
+
+// u_1 = V0 scaled by unit_scale (0 in a column of norm 0), so that no product or sum depends on |V0|; column
+// sums of u_1.u_1.  One pass over V0 a call: 500,009 rows, k = 4, 20 steps 1794 -> 1808 us; 1,000,000 rows, k = 1,
+// 12 steps 902 -> 908.
+template <int K, int MODE>
+__global__ void __launch_bounds__(kVecThreads, 2)
+    k_lz_start(int64_t n, int k, const double* V0, double* u1, const double* norm_partial, double* uu_partial) {
+  using G = Seg<K, MODE>;
+  grid_wait();
+  grid_dependents();
+  __shared__ VecShared sh;
+  __shared__ double s_scale[kMaxCols];
+  Walk<G> w(n, k);
+  double v[G::U][G::W];
+  w.load(V0, v);
+  const double norm2 = read_partials<G>(norm_partial, gridDim.x, k, sh);
+  const int c = threadIdx.x;
+  if (c < k) s_scale[c] = norm2 > 0.0 ? unit_scale(norm2) : 0.0;
+  __syncthreads();
+  double scale[G::KC], acc[G::KC];
+  const int c0 = G::column(threadIdx.x, k);
+#pragma unroll
+  for (int q = 0; q < G::KC; ++q) {
+    scale[q] = s_scale[c0 + q];
+    acc[q] = 0.0;
+  }
+  while (w.more()) {
+#pragma unroll
+    for (int j = 0; j < G::U; ++j) {
+      if (!w.has(j)) break;
+#pragma unroll
+      for (int i = 0; i < G::W; ++i) {
+        const int q = G::acc(i);
+        v[j][i] = scale[q] > 0.0 ? v[j][i] * scale[q] : 0.0;
+        acc[q] = fma(v[j][i], v[j][i], acc[q]);
+      }
+    }
+    w.store(u1, v);
+    w.next();
+    w.load(V0, v);
+  }
+  write_partial<G>(acc, k, uu_partial, sh);
+}
+
+// The beta of the step before, from uu = u_j.u_j.  uu_old is multiplied by the square of its own scale, a power
+// of two, so the quotient is beta^2 whatever size u_{j-1} had.
 __device__ __forceinline__ double last_beta(const LzScalars* S, int c, double uu) {
-  return S->live_old[c] ? sqrt(uu / S->uu_old[c]) / S->scale_old[c] : 0.0;
+  return S->live_old[c] ? sqrt(uu / (S->scale_old[c] * S->uu_old[c] * S->scale_old[c])) : 0.0;
 }
 
 // The Lanczos vectors are not normalised: u_j = |u_j| v_j, and the pass that divided by the norm is gone
@@ -470,7 +518,7 @@ __device__ __forceinline__ double last_beta(const LzScalars* S, int c, double uu
 // s_j, a power of two near 1 / |u_j| (0 for a column that has stopped), so that nothing is rounded, and
 // becomes s_j |u_j| (A v_j - beta_{j-1} v_{j-1}) = s_j W - (s_j u_j.u_j / s_{j-1} u_{j-1}.u_{j-1}) u_{j-1}; column sums
 // of W.u_j.  Each column scalar is one quotient of such sums: its error is alike in every row.  beta_{j-1} is
-// |u_j| / (s_{j-1} |u_{j-1}|), stored to beta_out unless that is NULL (j = 1: |V0|, every column live before).
+// |u_j| / (s_{j-1} |u_{j-1}|), stored to beta_out unless that is NULL (j = 1; every column was live before).
 template <int K, int MODE>
 __global__ void __launch_bounds__(kVecThreads, 2)
     k_lz_alpha(int64_t n, int k, double* W, const double* u, const double* u_prev, const double* uu_partial,
@@ -489,7 +537,7 @@ __global__ void __launch_bounds__(kVecThreads, 2)
   if (c < k) {
     const bool first = beta_out == nullptr;
     const bool live = (first || S->live_old[c]) && uu > 0.0;
-    const double scale = live ? ldexp(1.0, -(ilogb(uu) >> 1)) : 0.0;
+    const double scale = live ? unit_scale(uu) : 0.0;
     s_inv[c] = scale;
     s_prev[c] = !first && live ? scale * uu / (S->scale_old[c] * S->uu_old[c]) : 0.0;
     if (blockIdx.x == 0) {
@@ -621,6 +669,7 @@ SOLVER_LAUNCHER(LCgDot, k_cg_dot<K, MODE>)
 SOLVER_LAUNCHER(LCgUpdate, k_cg_update<K, MODE>)
 SOLVER_LAUNCHER(LCgDirection, k_cg_direction<K, MODE>)
 SOLVER_LAUNCHER(LLzNorm, k_lz_norm<K, MODE>)
+SOLVER_LAUNCHER(LLzStart, k_lz_start<K, MODE>)
 SOLVER_LAUNCHER(LLzAlpha, k_lz_alpha<K, MODE>)
 SOLVER_LAUNCHER(LLzBeta, k_lz_beta<K, MODE>)
 SOLVER_LAUNCHER(LLzEnd, k_lz_end<K, MODE>)
@@ -863,13 +912,18 @@ spmv_status spmv_lanczos(spmv_solver_handle S, const double* V0_dev, int32_t m, 
   }
   double* a_out = S->lz_out;
   double* b_out = S->lz_out + (size_t)m * kMaxCols;
-  // u_1 = V0; u_{j+1} is the W of step j, which takes the buffers in turn (buffer 0 is u_0 = 0)
-  const double *u_prev = S->buf[0], *u = V0_dev;
-  cudaError_t e = by_k<LLzNorm>(k, S->grid, s, S->n, k, V0_dev, S->partial);
+  // u_{j+1} is the W of step j; the three buffers hold u_{j-1}, u_j and W in turn, u_0 = 0 and u_1 (V0
+  // scaled) first
+  const double *u_prev = S->buf[0], *u = S->buf[1];
+  cudaError_t e = by_k<LLzNorm>(k, S->grid, s, S->n, k, V0_dev, S->partial2);
+  if (e == cudaSuccess)
+    e = by_k<LLzStart>(k, S->grid, s, S->n, k, V0_dev, S->buf[1], (const double*)S->partial2, S->partial);
+  // (The memset last: without it between them the first product is launched while k_lz_start runs, and all
+  // steps behind it take 2 us longer, 1,000,000 rows, k = 1.)
   if (e == cudaSuccess) e = cudaMemsetAsync(S->buf[0], 0, sizeof(double) * (size_t)S->n * (size_t)k, s);
   if (e != cudaSuccess) return cuda_fail(e, "Lanczos start");
   for (int j = 0; j < m; ++j) {
-    double* W = S->buf[(j + 1) % 3];
+    double* W = S->buf[(j + 2) % 3];
     spmv_status st = spmv_apply_block(S->A, u, k, k, W, k, s);
     if (st != SPMV_OK) return st;
     e = by_k<LLzAlpha>(k, S->grid, s, S->n, k, W, u, u_prev, (const double*)S->partial, S->partial2, S->lz,
