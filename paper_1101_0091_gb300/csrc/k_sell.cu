@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
 #pragma unroll
   for (int q = 0; q < W; ++q) acc[q] = 0.0;
   const double* Bc = B + c0;
-  const VT* vp = val + base;
+  const VT* vp = val + base;  // (advanced slot by slot: 32 slots of a row of 2^26 entries are out of 32 bits)
   const int32_t* cp = col + base;
   double g[W];
   if constexpr (W == 2 || W == 3) {
@@ -138,8 +138,10 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
       int32_t c = ldcs(cp);
       for (int j = 1; j < len; ++j) {
         load_cols(Bc + (int64_t)c * ldb, g);
-        const VT vn = ldcs(vp + j * kSellC);
-        c = ldcs(cp + j * kSellC);
+        vp += kSellC;
+        cp += kSellC;
+        const VT vn = ldcs(vp);
+        c = ldcs(cp);
 #pragma unroll
         for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
         v = vn;
@@ -150,8 +152,10 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     }
   } else {
     for (int j = 0; j < len; ++j) {
-      const double v = to_f64(ldcs(vp + j * kSellC));
-      load_cols(Bc + (int64_t)ldcs(cp + j * kSellC) * ldb, g);
+      const double v = to_f64(ldcs(vp));
+      load_cols(Bc + (int64_t)ldcs(cp) * ldb, g);
+      vp += kSellC;
+      cp += kSellC;
 #pragma unroll
       for (int q = 0; q < W; ++q) acc[q] = fma(v, g[q], acc[q]);
     }
