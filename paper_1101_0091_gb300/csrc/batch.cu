@@ -45,8 +45,8 @@ static int adaptive_lanes(int64_t len) {
 
 // Items of about item_nnz work units (a row counts max(len, 1)) and at most
 // 64 warp passes.  Contiguous rows [p0, p1) (mode 0), or positions [p0, p1) of
-// the row list, all of length len (mode 1) or of at most len (mode 2).  An item's
-// len is its longest row.
+// the row list, all of length len (mode 1) or of at most len (modes 2 and 4).  An item's
+// len is its longest row (modes 2 and 4: the longest of the rows cut together).
 static void cut_items(const int32_t* rp, int64_t p0, int64_t p1, int mat, int L, int mode, int64_t len,
                       int item_nnz, std::vector<BatchItem>& out) {
   const int64_t rows_cap = (int64_t)(32 / L) * 64;
@@ -62,7 +62,7 @@ static void cut_items(const int32_t* rp, int64_t p0, int64_t p1, int mat, int L,
       if (mode == 0) longest = 0;
     }
     if (mode == 0) longest = std::max<int64_t>(longest, rp[p + 1] - rp[p]);
-    work += mode == 1 ? std::max<int64_t>(len, 1) : (mode == 2 ? len : std::max<int64_t>(rp[p + 1] - rp[p], 1));
+    work += mode == 1 ? std::max<int64_t>(len, 1) : (mode != 0 ? len : std::max<int64_t>(rp[p + 1] - rp[p], 1));
   }
   if (p1 > s) emit(p1);
 }
@@ -181,7 +181,7 @@ void build_batch_items(const int32_t* rp, int64_t n_rows, int mat, int policy, i
       while (e <= maxlen && adaptive_lanes(maxlen - e) == L && maxlen - e > 32) ++e;
     const int64_t p0 = start[(size_t)d], p1 = start[(size_t)e];
     if (p1 > p0 && !(long_only && len <= kSortedMaxLen))
-      cut_items(rp, base + p0, base + p1, mat, L, len > 32 ? 2 : 1, len, item_nnz, out);
+      cut_items(rp, base + p0, base + p1, mat, L, len > 32 ? listed_mode(rp[n_rows]) : 1, len, item_nnz, out);
     d = e;
   }
 }

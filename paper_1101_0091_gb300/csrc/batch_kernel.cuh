@@ -19,7 +19,8 @@ struct BatchMat {
 // Work item.  mode 0: rows [p0, p1) of member `mat`, bounds from row_ptr.
 // mode 1: the rows listed at positions [p0, p1) of the (row, first entry)
 // list, all of length `len` (the length-binned rows of the adaptive policy).
-// mode 2: listed rows of unequal lengths (ends from row_ptr).
+// mode 2: listed rows of unequal lengths (ends from row_ptr); mode 4 the same, of a member whose
+// entries end within a long step of 2^31 - 1 (listed_mode).
 // mode 3: chunks [p0, p1) of the length-sorted SELL-32 copy (sorted policy),
 // all of length `len`, stored back to back from slot `base`: one lane per row,
 // slots column-major inside a chunk.
@@ -30,6 +31,9 @@ struct BatchItem {
   int32_t pad;
   int64_t base;
 };
+
+// At k = 2 mode 2 steps by up to 4 entries on each of 32 lanes, counted in 32 bits.
+inline int listed_mode(int64_t nnz) { return nnz <= INT32_MAX - 4 * 32 ? 2 : 4; }
 
 // Length-sorted SELL-32 copy of the short rows of the members with the sorted
 // policy: chunk c holds 32 rows (row index perm[32c + t], -1 for padding) of

@@ -38,8 +38,11 @@ static thread_local dim3 threadIdx;
 static dim3 blockIdx(0), gridDim(1);
 static std::barrier<>*cta_barrier, *warp_barrier;
 template <typename T> T __ldg(const T* p) { return *p; }
+template <typename T> void __stcs(T* p, T x) { *p = x; }
 static inline unsigned __activemask() { return 1; }
 static inline int __any_sync(unsigned, int x) { return x; }
+static inline int atomicAdd(int* p, int x) { return *p += x; }
+static inline int __shfl_sync(unsigned, int x, int) { return x; }
 static inline int __clz(int x) { return __builtin_clz(x); }
 static inline void __syncwarp() { warp_barrier->arrive_and_wait(); }
 static inline void __syncthreads() { cta_barrier->arrive_and_wait(); }
@@ -116,6 +119,82 @@ int main() {
 }
 """
 
+# Rows that end at 2^31 - 1, the largest nnz of a plan.
+LANES = r"""
+static const double* val;
+static const int32_t* col;
+static const int last = INT_MAX;
+template <typename F> static int row(int len, int ldb, int k, int threads, bool sync, F f) {
+  int32_t row_ptr[2] = {last - len, last};
+  static double B[2 * 4], C[4];
+  for (int i = 0; i < 8; ++i) B[i] = i < ldb ? 0 : 100 + i;
+  for (double& c : C) c = 0;
+  cta(0, threads, sync, [&] { f(row_ptr, B, C); });
+  const int n = len < 40 ? len : 40;  // the mapping ends in 40 entries of value 1, column 1
+  for (int q = 0; q < k; ++q) CHECK(C[q], n * B[ldb + q]);
+  return 0;
+}
+int main() {
+  double* v = mapped<double>(last + 5ll);
+  int32_t* c = mapped<int32_t>(last + 5ll);
+  for (int i = 0; i < 40; ++i) v[last - 1ll - i] = c[last - 1ll - i] = 1;
+  val = v, col = c;
+  int bad = 0;
+  for (int len : {1, 2, 3, 4, 5, 6, 7, 8, 9, 31}) {
+    bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_row<double, true>(1, rp, col, val, B, 1, C, 1, 0);
+    });
+    bad |= row(len, 2, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_row<double, false>(1, rp, col, val, B, 2, C, 1, 0);
+    });
+    bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_wide<double, 1>(1, rp, col, val, B, 1, C, 1);
+    });
+    bad |= row(len, 4, 4, 1, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_wide<double, 4>(1, rp, col, val, B, 4, C, 4);
+    });
+    bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {  // a lane row of k_crs_long
+      spmv::k_crs_long<double>(nullptr, 0, 0, 1, rp, col, val, B, 1, C, 1, 1, 32, 0);
+    });
+    bad |= row(len, 2, 2, 2, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_cols<double, 1>(1, rp, col, val, B, 2, C, 2, 2, 0);
+    });
+  }
+  static int32_t zero = 0;
+  for (int k : {1, 3})
+    for (int len : {40, 70, 300, 1500, 5000})
+      for (int n_cta : {0, 1})  // the row on a warp, on a CTA
+        bad |= row(len, k, k, n_cta ? 256 : 32, true, [&](int32_t* rp, double* B, double* C) {
+          spmv::k_crs_long<double>(&zero, 1, n_cta, 1, rp, col, val, B, k, C, k, k, 12, 0);
+        });
+  return bad;
+}
+"""
+
+# Rows that end 64 entries below: as far as the steps of one entry a lane go.
+BATCH = r"""
+int main() {
+  const int last = INT_MAX - 64;
+  double* v = mapped<double>(last);
+  int32_t* c = mapped<int32_t>(last);
+  static double B[4], C[4];
+  for (int len : {50, 127, 128, 129, 700}) {
+    int32_t rp[2] = {last - len, last};
+    int2 list[1] = {{0, last - len}};
+    spmv::BatchMat m = {rp, c, v, B, C, 2, 2, 1};
+    for (int lanes : {2, 4, 8, 16, 32})
+      for (int lane = 0; lane < 32; ++lane) {
+        spmv::BatchItem one = {0, 0, 1, len, (int16_t)lanes, (int16_t)spmv::listed_mode(last), 0, 0};
+        spmv::batch_row_item<2, 2>(&m, list, one, 2, lane);
+        spmv::batch_row_item<2, 1>(&m, list, one, 2, lane);
+      }
+  }
+  return spmv::listed_mode(last - 64) != 2;  // (the sum over the lanes is stubbed: only the reads are checked)
+}
+"""
+
+headers = pytest.mark.skipif(not os.path.exists("/usr/local/cuda/include/cuda_runtime.h"), reason="no CUDA headers")
+
 
 def run_on_host(tmp_path, source, harness):
     text = open(os.path.join(CSRC, source)).read()
@@ -135,6 +214,16 @@ def run_on_host(tmp_path, source, harness):
     assert r.returncode == 0, (r.returncode, r.stdout, r.stderr)
 
 
-@pytest.mark.skipif(not os.path.exists("/usr/local/cuda/include/cuda_runtime.h"), reason="no CUDA headers")
+@headers
 def test_sell_slots_behind_2_31(tmp_path):
     run_on_host(tmp_path, "k_sell.cu", SELL)
+
+
+@headers
+def test_crs_rows_that_end_at_2_31(tmp_path):
+    run_on_host(tmp_path, "k_lanes.cu", LANES)
+
+
+@headers
+def test_batch_rows_that_end_at_2_31(tmp_path):
+    run_on_host(tmp_path, "batch_kernel.cuh", BATCH)
