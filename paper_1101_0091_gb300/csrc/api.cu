@@ -90,6 +90,7 @@ struct spmv_plan {
   uint64_t generation = 0;  // bumped whenever the kernel, its arrays or its launch parameters change
   spmv_options opt{};
   int variant = SPMV_CRS_STAGED;
+  int requested = SPMV_VARIANT_AUTO;  // as asked for: AUTO's CRS_L1 is not an explicit one's kernel (long_rows)
   // what AUTO runs: SELL-32-256 on matrices whose rows gather at scattered
   // addresses (and pack well into SELL), CRS_L1 otherwise
   double scattered = 0.0;
@@ -360,7 +361,7 @@ static spmv_status build_sym_dev(spmv_plan* p) {
 }
 
 static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
-  const bool is_auto = variant == SPMV_VARIANT_AUTO;
+  const int requested = variant;
   if (variant == SPMV_VARIANT_AUTO) {
     variant = p->auto_sell ? SPMV_SELL : SPMV_CRS_L1;
     sigma = p->auto_sell ? 256 : sigma;
@@ -380,7 +381,8 @@ static spmv_status prepare_variant(spmv_plan* p, int variant, int sigma) {
     spmv_status st = build_sym_dev(p);
     if (st != SPMV_OK) return st;
   }
-  p->A.long_rows = is_auto ? p->long_rows : LongRows{};
+  p->A.long_rows = requested == SPMV_VARIANT_AUTO ? p->long_rows : LongRows{};
+  p->requested = requested;
   p->variant = variant;
   ++p->generation;
   return SPMV_OK;
@@ -740,7 +742,7 @@ spmv_status spmv_autotune(spmv_handle h, int32_t k, const double* B_dev, int64_t
   if (h->host.n_rows > 0 && (!C_dev || (!B_dev && h->host.n_cols > 0))) return fail(SPMV_ERR_ARG, "NULL buffer");
   DeviceGuard g(h->device);
   cudaStream_t s = (cudaStream_t)stream;
-  const int keep_variant = h->variant, keep_sigma = h->sell.perm ? h->sell.sigma : 1;
+  const int keep_variant = h->requested, keep_sigma = h->sell.perm ? h->sell.sigma : 1;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   SPMV_CUDA(cudaEventCreate(&e0));
   cudaError_t ce = cudaEventCreate(&e1);
