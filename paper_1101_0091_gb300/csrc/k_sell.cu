@@ -98,8 +98,28 @@ __global__ void __launch_bounds__(kThreads)
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
 }
 
+// W columns of a block row: 16-byte accesses (A16, even W) or 8-byte ones.
+template <int W, bool A16>
+__device__ __forceinline__ void load_row(const double* b, double (&g)[W]) {
+  if constexpr (A16) {
+    load_cols(b, g);
+  } else {
+#pragma unroll
+    for (int q = 0; q < W; ++q) g[q] = b[q];
+  }
+}
+
+// Slots of a lane's step in k_sell_cols, whose values and columns are loaded behind the gathers of the step
+// before (0: no such pipeline).  Means over rows of 1 .. 200 entries, 20,000 .. 2,000,000 of them, in units
+// of the fastest of 0 / 1 / 2 slots: doubles one column 1.06 / 1.02 / 1.03, two in 16 bytes 1.03 / 1.03 / 1.02
+// (eigenproblem matrices of 600,011 and 2,000,003 rows, k = 6, 94.8 / 93.8 / 95.1 and 300 / 297 / 300 us), two, three
+// and four in 8 bytes 1.05 / 1.02 / 1.01, four in 16 bytes 1.02 / 1.01 / 1.04, five and seven 1.04 / 1.01 / 1.04;
+// floats one column 1.02 / 1.09 / 1.10, two 1.03 / 1.05 / 1.01, three and four 1.03 / 1.02 / 1.02.
+template <typename VT, int W, bool A16>
+constexpr int kSellStep = sizeof(VT) == 4 ? (W == 1 ? 0 : W == 2 ? 2 : 1) : (!A16 && W >= 2 && W <= 4 ? 2 : 1);
+
 // k columns of a sorted row on G = k / W lanes, W columns each (as k_crs_cols).
-template <typename VT, int W>
+template <typename VT, int W, bool A16>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm, const int32_t* __restrict__ row_ptr,
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
@@ -127,17 +147,54 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   const double* Bc = B + c0;
   const VT* vp = val + base;  // (advanced slot by slot: 32 slots of a row of 2^26 entries are out of 32 bits)
   const int32_t* cp = col + base;
-  double g[W];
-  if constexpr (W == 2 || W == 3) {
-    // The next slot's value and column are in flight while this slot's gathers are: 600,011 rows, k = 6
-    // 94.8 -> 93.7 us; 400,009 rows, k = 2 / 3 / 4 28.6 -> 27.7, 44.5 -> 42.5, 46.0 -> 45.5; 130^3 Poisson, k = 2 / 4
-    // 61.2 -> 56.9, 109.1 -> 105.5.  Not with one column a lane (100,003 rows, k = 4: 15.8 -> 16.8) nor with five
-    // (400,009 rows, k = 5: 63.2 -> 65.4) or seven (Poisson, FP32 values 179.5 -> 182.3).
+  constexpr int NB = kSellStep<VT, W, A16>;
+  if constexpr (NB == 2) {
+    VT v[NB];
+    int32_t cc[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      v[u] = VT();
+      cc[u] = 0;
+      if (u < len) {
+        v[u] = ldcs(vp + u * kSellC);
+        cc[u] = ldcs(cp + u * kSellC);
+      }
+    }
+    int j = 0;
+    for (; j + NB <= len; j += NB) {
+      double g[NB][W];
+      VT vn[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) load_row<W, A16>(Bc + (int64_t)cc[u] * ldb, g[u]);
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int64_t nxt = (int64_t)(j + NB + u < len ? j + NB + u : j) * kSellC;
+        vn[u] = ldcs(vp + nxt);
+        cc[u] = ldcs(cp + nxt);
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+#pragma unroll
+        for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v[u]), g[u][q], acc[q]);
+#pragma unroll
+      for (int u = 0; u < NB; ++u) v[u] = vn[u];
+    }
+#pragma unroll
+    for (int u = 0; u < NB - 1; ++u)
+      if (j + u < len) {
+        double g[W];
+        load_row<W, A16>(Bc + (int64_t)cc[u] * ldb, g);
+#pragma unroll
+        for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v[u]), g[q], acc[q]);
+      }
+  } else if constexpr (NB == 1) {
+    double g[W];
     if (len > 0) {
       VT v = ldcs(vp);
       int32_t c = ldcs(cp);
+#pragma unroll 4
       for (int j = 1; j < len; ++j) {
-        load_cols(Bc + (int64_t)c * ldb, g);
+        load_row<W, A16>(Bc + (int64_t)c * ldb, g);
         vp += kSellC;
         cp += kSellC;
         const VT vn = ldcs(vp);
@@ -146,14 +203,15 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
         for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
         v = vn;
       }
-      load_cols(Bc + (int64_t)c * ldb, g);
+      load_row<W, A16>(Bc + (int64_t)c * ldb, g);
 #pragma unroll
       for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
     }
   } else {
+    double g[W];
     for (int j = 0; j < len; ++j) {
       const double v = to_f64(ldcs(vp));
-      load_cols(Bc + (int64_t)ldcs(cp) * ldb, g);
+      load_row<W, A16>(Bc + (int64_t)ldcs(cp) * ldb, g);
       vp += kSellC;
       cp += kSellC;
 #pragma unroll
@@ -161,16 +219,44 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     }
   }
   grid_dependents();
-  store_cols(C + (int64_t)row * ldc + c0, acc);
+  double* out = C + (int64_t)row * ldc + c0;
+  if constexpr (A16) {
+    store_cols(out, acc);
+  } else {
+#pragma unroll
+    for (int q = 0; q < W; ++q) out[q] = acc[q];
+  }
 }
 
-template <typename VT, int W>
+template <typename VT, int W, bool A16 = (W % 2 == 0)>
 static cudaError_t launch_cols(const SellDev& S, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                                int k, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (S.n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_sell_cols<VT, W>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.row_ptr, S.chunk_ptr,
-                          S.chunk_len, S.col, val, B, ldb, C, ldc, G, S.prefetch);
+  return launch_dependent(k_sell_cols<VT, W, A16>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm,
+                          S.row_ptr, S.chunk_ptr, S.chunk_len, S.col, val, B, ldb, C, ldc, G, S.prefetch);
+}
+
+// Columns per lane of a block product.  Several read a row's slots and its B rows in fewer, longer accesses, as
+// long as the threads still fill the GPU.
+static int sell_cols(const SellDev& S, int k, bool a16) {
+  const int64_t n = S.n_rows;
+  // Four for many short rows (in an uneven chunk the padding is idle FP64 time, more of it the more rows a warp
+  // holds).  Two -> four columns, k = 16: 1,500,000 rows of 2 / 5 / 8 entries 168 -> 121, 271 -> 205, 341 -> 319 us,
+  // 300,000 rows of 3 34.6 -> 27.2, of 13 106.6 -> 106.6; eigenproblem matrix of 600,011 rows (12.8 a row), k = 8,
+  // 120.4 -> 126.2; of 60,000 rows, one -> four, 15.3 -> 19.8.
+  if (k % 4 == 0 && n * (k / 4) >= 1000000 && S.slots <= 9 * n) return 4;
+  // Two: k = 2 always (one -> two columns: 20,000 rows of 48 / 200 entries 21.9 -> 15.4, 57.8 -> 43.6 us, 200,000
+  // rows of 4 or 60 39.9 -> 32.8, eigenproblem matrices of 60,000 / 150,000 rows 9.3 -> 9.4, 16.6 -> 15.0), other k
+  // from as many threads on as k_crs_cols (k = 8, 60,000 / 150,000 rows 15.3 -> 17.8, 33.4 -> 34.2).
+  if (a16 && k % 2 == 0 && (k == 2 || n * (k / 2) >= kMinColThreads)) return 2;
+  // 8-byte accesses.  One -> two columns: 1,500,000 rows, k = 2, of 1 / 2 / 3 / 5 / 8 entries 23.2 -> 19.9, 32.5 ->
+  // 30.4, 37.2 -> 36.3, 44.1 -> 50.0, 63.2 -> 70.9 us, k = 4, of 8 entries 118 -> 94.
+  if (!(a16 && k % 2 == 0))
+    for (int w : {7, 5, 3})
+      if (k % w == 0 && n * (k / w) >= kMinColThreads) return w;
+  if (!a16 && k % 2 == 0 && n * (k / 2) >= kMinColThreads && (k > 2 || S.slots <= 3 * n)) return 2;
+  return 1;
 }
 
 template <typename VT>
@@ -178,13 +264,17 @@ static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int6
                           int k, cudaStream_t s) {
   if (S.n_chunks == 0) return cudaSuccess;
   if (k > 1) {
-    // two columns per lane at most: 600,011-row eigenproblem matrix, k = 4 / 8 / 16, four -> two columns 71.6 ->
-    // 66.2, 126.5 -> 120.4, 232.1 -> 227.8 us (fewer rows per warp: less is added for the chunk's padding)
-    switch (cols_per_lane(k, rows_on_16_bytes(B, ldb, C, ldc), S.n_rows, 2, true)) {
+    const bool a16 = rows_on_16_bytes(B, ldb, C, ldc);
+    switch (sell_cols(S, k, a16)) {
       case 7: return launch_cols<VT, 7>(S, val, B, ldb, C, ldc, k, s);
       case 5: return launch_cols<VT, 5>(S, val, B, ldb, C, ldc, k, s);
+      case 4:
+        return a16 ? launch_cols<VT, 4>(S, val, B, ldb, C, ldc, k, s)
+                   : launch_cols<VT, 4, false>(S, val, B, ldb, C, ldc, k, s);
       case 3: return launch_cols<VT, 3>(S, val, B, ldb, C, ldc, k, s);
-      case 2: return launch_cols<VT, 2>(S, val, B, ldb, C, ldc, k, s);
+      case 2:
+        return a16 ? launch_cols<VT, 2>(S, val, B, ldb, C, ldc, k, s)
+                   : launch_cols<VT, 2, false>(S, val, B, ldb, C, ldc, k, s);
       default: return launch_cols<VT, 1>(S, val, B, ldb, C, ldc, k, s);
     }
   }
