@@ -323,9 +323,11 @@ static spmv_status build_graph(spmv_batch_plan* b) {
   return capture_graph(b, b->d_mats, b->vec, &b->graph, &b->exec);
 }
 
-// Rounds of dependent loads that a warp runs through for an item (chunks of rows
-// with up to two entries go four and two at a time, with up to four one at a time,
-// longer ones one slot a round; other items count each pass as their longest row).
+// What an item takes, relative to others: about the rounds of dependent loads that a warp runs through (chunks of
+// rows with one / two entries count four and two at a time, with up to four one at a time, longer ones a
+// slot each; other items each pass as their longest row).  Counted as the kernels step (their slots and
+// entries a round by k) the order is no better: 512-member mix cut to 96, k = 2 / 4 / 8 87.4 -> 90.5, 121.9 -> 121.5,
+// 259.9 -> 260.3 us; 40 members of rows of 60 .. 200, k = 3 / 4 131.4 -> 139.3, 164 -> 171.
 static int64_t item_rounds(const BatchItem& it) {
   const int64_t n = it.p1 - it.p0;
   if (it.mode == 3) return it.len <= 1 ? n / 4 : it.len == 2 ? n / 2 : it.len <= 4 ? n : n * it.len;
@@ -355,9 +357,15 @@ static spmv_status rebuild(spmv_batch_plan* b) {
   // starts last is run out alone.  512 members, k = 2 / 4: 368 -> 355, 499 -> 491 us;
   // 96 members 96.5 -> 84.2, 119.6 -> 111.7 us; 32 members, k = 8: 131 -> 112 us.
   // Twice as many lose more to the gathers from DRAM than they gain (k = 4).
+  // Not if all items are in flight at once: then none starts late, and neighbours of falling length load the SMs
+  // unevenly (200 members of 2000 rows, sorted, k = 6 / 8 / 12: 53.9 -> 48.1, 55.6 -> 49.8, 85.2 -> 79.2 us).
   const size_t warps = (size_t)b->num_sms * b->cfg.ctas_per_sm * (kBatchThreads / 32);
-  std::stable_sort(items.end() - std::min(items.size(), warps), items.end(),
-                   [](const BatchItem& x, const BatchItem& y) { return item_rounds(x) > item_rounds(y); });
+  int resident = 0;
+  SPMV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, batch_kernel(b->k, b->vec), kBatchThreads, 0));
+  const size_t in_flight = (size_t)b->num_sms * std::min(b->cfg.ctas_per_sm, resident) * (kBatchThreads / 32);
+  if (items.size() > in_flight)
+    std::stable_sort(items.end() - std::min(items.size(), warps), items.end(),
+                     [](const BatchItem& x, const BatchItem& y) { return item_rounds(x) > item_rounds(y); });
   b->n_chunk_items = std::count_if(items.begin(), items.end(), [](const BatchItem& it) { return it.mode == 3; });
   if (b->d_items) cudaFree(b->d_items);
   if (b->d_rowlist) cudaFree(b->d_rowlist);
