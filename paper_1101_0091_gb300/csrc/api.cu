@@ -261,18 +261,16 @@ static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const R
   return list;
 }
 
-// long_rows (NULL for the parts of a split, which run one vector) receives the list of list_long_rows,
+// long_rows (NULL for the parts of a split) receives the list of list_long_rows,
 // uploaded behind row_ptr.
 static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n_cols, const int32_t* rp,
                               const int32_t* col, const double* val, int64_t nnz, LongRows* long_rows) {
   int32_t *drp, *dcol;
   double* dval;
   std::vector<int32_t> list;
-  if (long_rows) {
-    const RowStats stats = row_stats(rp, n_rows);
-    M->lane_cols = lane_cols(stats, nnz);
-    list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
-  }
+  const RowStats stats = row_stats(rp, n_rows);
+  M->lane_cols = lane_cols(stats, nnz);
+  if (long_rows) list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
   SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, (int64_t)list.size()));
   if (!list.empty()) {
     SPMV_CUDA(cudaMemcpy(drp + n_rows + 1, list.data(), sizeof(int32_t) * list.size(), cudaMemcpyHostToDevice));

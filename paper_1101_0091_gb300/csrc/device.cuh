@@ -177,11 +177,11 @@ inline int cols_per_lane(int k, bool a16, int64_t n_rows, int even, bool odd) {
   return 1;
 }
 
-// W consecutive columns of a block row: 16-byte accesses for W = 2, 4, else 8-byte ones.  (Plain loads:
-// see grid_wait.)
-template <int W>
+// W consecutive columns of a block row: 16-byte accesses where the rows start on 16 bytes (A16, even W), else
+// 8-byte ones.  (Plain loads: see grid_wait.)
+template <int W, bool A16 = (W % 2 == 0)>
 __device__ __forceinline__ void load_cols(const double* b, double (&g)[W]) {
-  if constexpr (W % 2 == 1) {
+  if constexpr (!A16) {
 #pragma unroll
     for (int q = 0; q < W; ++q) g[q] = b[q];
   } else {
@@ -193,9 +193,9 @@ __device__ __forceinline__ void load_cols(const double* b, double (&g)[W]) {
     }
   }
 }
-template <int W>
+template <int W, bool A16 = (W % 2 == 0)>
 __device__ __forceinline__ void store_cols(double* c, const double (&a)[W]) {
-  if constexpr (W % 2 == 1) {
+  if constexpr (!A16) {
 #pragma unroll
     for (int q = 0; q < W; ++q) c[q] = a[q];
   } else {

@@ -121,8 +121,11 @@ __device__ __forceinline__ void add_tail(int r, const VT* v, const double (*x)[W
 // cost what it padded: 280^3 Poisson (7 entries a row) 326.5 -> 323.2 us (HBM-bound), with FP32 values
 // 303.9 -> 272.4 us; 1500^2 Laplacian 39.0 -> 33.2 us; 3,000,000 rows of 5 entries 48.9 -> 41.1 us.  The
 // two pipes together bound it: 7 multiply-adds per row are 0.74 of the HBM time at 280^3, with FP32
-// values 0.99 of it.
-template <typename VT, bool UNIT>  // UNIT: ldb = 1 (its multiplication and two registers saved)
+// values 0.99 of it.  Among uneven rows a warp waits for its longest anyway, and with FP32 values the
+// batches are masked (MASKED): 1,500,000 rows of 0 .. 12 / 4 .. 9 / 10 .. 30 entries 42.0 -> 35.1,
+// 42.6 -> 35.8, 53.9 -> 42.4 us, power-law rows of up to 16 35.0 -> 30.7.  (Doubles of the first, second and last: 44.3 -> 40.9,
+// 39.0 -> 40.8, 32.6 -> 37.0; not masked.)
+template <typename VT, bool UNIT, bool MASKED>  // UNIT: ldb = 1 (its multiplication and two registers saved)
 __global__ void __launch_bounds__(kThreads, 8)
     k_crs_row(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
@@ -136,6 +139,24 @@ __global__ void __launch_bounds__(kThreads, 8)
   grid_wait();
   if (gridDim.x > 4 * kOneWave) grid_dependents();
   double acc[1] = {0.0};
+  if constexpr (MASKED) {
+    for (int left = re - j; left > 0; left -= 4, j = (int)((uint32_t)j + 4)) {
+      double v[4], x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = u < left ? j + u : j;
+        v[u] = to_f64(ldg(val + i));
+        const double* b = UNIT ? B + ldg(col + i) : B + (int64_t)ldg(col + i) * ldb;
+        x[u] = u < left ? *b : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (u < left) acc[0] = fma(v[u], x[u], acc[0]);
+    }
+    grid_dependents();
+    C[g * ldc] = acc[0];
+    return;
+  }
   for (; re - j >= 4; j += 4) {
     const VT* vj = val + j;
     const int32_t* cj = col + j;
@@ -179,8 +200,8 @@ __global__ void __launch_bounds__(kThreads, 8)
   C[row] = c + acc;
 }
 
-// k columns of a row on G = k / W lanes, W columns each (W = 4 or 2 with 16-byte accesses, else 1).
-template <typename VT, int W>
+// k columns of a row on G = k / W lanes, W columns each (A16: the blocks' rows start on 16 bytes; even W).
+template <typename VT, int W, bool A16>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_crs_cols(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
@@ -202,20 +223,20 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   for (int j = rs; j < re; ++j) {
     const double v = to_f64(ldg(val + j));
     double gv[W];
-    load_cols(Bc + (int64_t)ldg(col + j) * ldb, gv);
+    load_cols<W, A16>(Bc + (int64_t)ldg(col + j) * ldb, gv);
 #pragma unroll
     for (int q = 0; q < W; ++q) acc[q] = fma(v, gv[q], acc[q]);
   }
   grid_dependents();
-  store_cols(C + g * ldc + c0, acc);
+  store_cols<W, A16>(C + g * ldc + c0, acc);
 }
 
-template <typename VT, int W>
+template <typename VT, int W, bool A16 = (W % 2 == 0)>
 static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int32_t* col, const VT* val,
                                const double* B, int64_t ldb, double* C, int64_t ldc, int k, int pf, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_crs_cols<VT, W>, (unsigned)grid, kThreads, s, n_rows, row_ptr, col, val, B, ldb, C, ldc, G,
+  return launch_dependent(k_crs_cols<VT, W, A16>, (unsigned)grid, kThreads, s, n_rows, row_ptr, col, val, B, ldb, C, ldc, G,
                           pf);
 }
 
@@ -463,22 +484,38 @@ static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64
   const int pf = A.prefetch;
   const bool a16 = rows_on_16_bytes(B, ldb, C, ldc);
   if (A.long_rows.n > 0) return launch_long(A, val, B, ldb, C, ldc, k, s);
+  const bool even = A.lane_cols == 4;
   if (k == 1) {
-    if (A.nnz >= kWideRow * n) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
-    return launch_dependent(ldb == 1 ? k_crs_row<VT, true> : k_crs_row<VT, false>,
-                            (unsigned)((n + kThreads - 1) / kThreads), kThreads, s, n, rp, col, val, B, ldb, C, ldc, pf);
+    const bool masked = sizeof(VT) == 4 && !even;
+    if (!masked && A.nnz >= kWideRow * n) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
+    auto* row = masked ? (ldb == 1 ? k_crs_row<VT, true, sizeof(VT) == 4> : k_crs_row<VT, false, sizeof(VT) == 4>)
+                       : (ldb == 1 ? k_crs_row<VT, true, false> : k_crs_row<VT, false, false>);
+    return launch_dependent(row, (unsigned)((n + kThreads - 1) / kThreads), kThreads, s, n, rp, col, val, B, ldb, C,
+                            ldc, pf);
   }
+  // (uneven rows: a row's columns on one lane keep its warp waiting for its longest row.  Rows of 10 .. 30 entries,
+  // 300,000 of them, k = 2 / 4: 51.8 / 97.2 us on k_crs_wide, 37.6 / 65.3 on k_crs_cols)
   const bool long_average = A.nnz >= kWideRowCols * n;
-  if (long_average && a16 && k == 2) return launch_wide<VT, 2>(A, val, B, ldb, C, ldc, s);
-  if (long_average && a16 && k == 4) return launch_wide<VT, 4>(A, val, B, ldb, C, ldc, s);
+  if (long_average && even && a16 && k == 2) return launch_wide<VT, 2>(A, val, B, ldb, C, ldc, s);
+  if (long_average && even && a16 && k == 4) return launch_wide<VT, 4>(A, val, B, ldb, C, ldc, s);
   // (rows of 16 and more entries: one column per lane rather than 3, 5 or 7; the lanes of a row share its
   // uncoalesced entries.  27-point stencil on 60^3, k = 3 / 5, one / several: 32.5 / 34.8, 51.4 / 54.9 us)
-  switch (cols_per_lane(k, a16, n, A.lane_cols, A.lane_cols > 1 && !long_average)) {
+  int w = cols_per_lane(k, a16, n, A.lane_cols, A.lane_cols > 1 && !long_average);
+  // Short rows gain by two columns from fewer threads on where they are uneven (100,000 / 300,000 rows of 4 .. 9
+  // entries, k = 4 / 2, one -> two columns 13.0 -> 10.6, 18.2 -> 14.1 us; of 0 .. 12 13.0 -> 13.5, 18.2 -> 18.0; 30,000
+  // of 0 .. 12, k = 16, 11.2 -> 12.9), and in
+  // 8-byte accesses too (1,500,000 rows of 4 .. 9, k = 4, ld = 5 150.4 -> 113.1, of 1 49.0 -> 38.6, 160^3 Poisson 199.5 ->
+  // 192.3; 300,000 rows of 8 18.4 -> 20.0).
+  if (w == 1 && k % 2 == 0 && A.lane_cols > 1 && A.nnz < kWideRow * n && (even ? n * (k / 2) >= kMinColThreads : n >= 100000))
+    w = 2;
+  switch (w) {
     case 7: return launch_cols<VT, 7>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
     case 5: return launch_cols<VT, 5>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
     case 4: return launch_cols<VT, 4>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
     case 3: return launch_cols<VT, 3>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
-    case 2: return launch_cols<VT, 2>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
+    case 2:
+      return a16 ? launch_cols<VT, 2>(n, rp, col, val, B, ldb, C, ldc, k, pf, s)
+                 : launch_cols<VT, 2, false>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
     default: return launch_cols<VT, 1>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
   }
 }

@@ -98,17 +98,6 @@ __global__ void __launch_bounds__(kThreads)
   C[(int64_t)__ldg(perm + r) * ldc] = acc;
 }
 
-// W columns of a block row: 16-byte accesses (A16, even W) or 8-byte ones.
-template <int W, bool A16>
-__device__ __forceinline__ void load_row(const double* b, double (&g)[W]) {
-  if constexpr (A16) {
-    load_cols(b, g);
-  } else {
-#pragma unroll
-    for (int q = 0; q < W; ++q) g[q] = b[q];
-  }
-}
-
 // Slots of a lane's step in k_sell_cols, whose values and columns are loaded behind the gathers of the step
 // before (0: no such pipeline).  Means over rows of 1 .. 200 entries, 20,000 .. 2,000,000 of them, in units
 // of the fastest of 0 / 1 / 2 slots: doubles one column 1.06 / 1.02 / 1.03, two in 16 bytes 1.03 / 1.03 / 1.02
@@ -165,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
       double g[NB][W];
       VT vn[NB];
 #pragma unroll
-      for (int u = 0; u < NB; ++u) load_row<W, A16>(Bc + (int64_t)cc[u] * ldb, g[u]);
+      for (int u = 0; u < NB; ++u) load_cols<W, A16>(Bc + (int64_t)cc[u] * ldb, g[u]);
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
         const int64_t nxt = (int64_t)(j + NB + u < len ? j + NB + u : j) * kSellC;
@@ -183,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     for (int u = 0; u < NB - 1; ++u)
       if (j + u < len) {
         double g[W];
-        load_row<W, A16>(Bc + (int64_t)cc[u] * ldb, g);
+        load_cols<W, A16>(Bc + (int64_t)cc[u] * ldb, g);
 #pragma unroll
         for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v[u]), g[q], acc[q]);
       }
@@ -194,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
       int32_t c = ldcs(cp);
 #pragma unroll 4
       for (int j = 1; j < len; ++j) {
-        load_row<W, A16>(Bc + (int64_t)c * ldb, g);
+        load_cols<W, A16>(Bc + (int64_t)c * ldb, g);
         vp += kSellC;
         cp += kSellC;
         const VT vn = ldcs(vp);
@@ -203,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
         for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
         v = vn;
       }
-      load_row<W, A16>(Bc + (int64_t)c * ldb, g);
+      load_cols<W, A16>(Bc + (int64_t)c * ldb, g);
 #pragma unroll
       for (int q = 0; q < W; ++q) acc[q] = fma(to_f64(v), g[q], acc[q]);
     }
@@ -211,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     double g[W];
     for (int j = 0; j < len; ++j) {
       const double v = to_f64(ldcs(vp));
-      load_row<W, A16>(Bc + (int64_t)ldcs(cp) * ldb, g);
+      load_cols<W, A16>(Bc + (int64_t)ldcs(cp) * ldb, g);
       vp += kSellC;
       cp += kSellC;
 #pragma unroll
@@ -219,13 +208,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     }
   }
   grid_dependents();
-  double* out = C + (int64_t)row * ldc + c0;
-  if constexpr (A16) {
-    store_cols(out, acc);
-  } else {
-#pragma unroll
-    for (int q = 0; q < W; ++q) out[q] = acc[q];
-  }
+  store_cols<W, A16>(C + (int64_t)row * ldc + c0, acc);
 }
 
 template <typename VT, int W, bool A16 = (W % 2 == 0)>

@@ -58,8 +58,8 @@ inline double to_f64(f32n v) { return v.v; }
 template <typename T> T ldg(const T* p) { return *p; }
 template <typename T> T ldcs(const T* p) { return *p; }
 template <typename T> void ldg4(const T* p, T (&x)[4]) { for (int i = 0; i < 4; ++i) x[i] = p[i]; }
-template <int W> void load_cols(const double* b, double (&g)[W]) { for (int q = 0; q < W; ++q) g[q] = b[q]; }
-template <int W> void store_cols(double* c, const double (&a)[W]) { for (int q = 0; q < W; ++q) c[q] = a[q]; }
+template <int W, bool = false> void load_cols(const double* b, double (&g)[W]) { for (int q = 0; q < W; ++q) g[q] = b[q]; }
+template <int W, bool = false> void store_cols(double* c, const double (&a)[W]) { for (int q = 0; q < W; ++q) c[q] = a[q]; }
 inline double warp_sum_xor(double x, int) { return x; }
 inline bool rows_on_16_bytes(const double*, int64_t, const double*, int64_t) { return true; }
 inline int cols_per_lane(int, bool, int64_t, int, bool) { return 1; }
@@ -142,10 +142,13 @@ int main() {
   int bad = 0;
   for (int len : {1, 2, 3, 4, 5, 6, 7, 8, 9, 31}) {
     bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
-      spmv::k_crs_row<double, true>(1, rp, col, val, B, 1, C, 1, 0);
+      spmv::k_crs_row<double, true, false>(1, rp, col, val, B, 1, C, 1, 0);
     });
     bad |= row(len, 2, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
-      spmv::k_crs_row<double, false>(1, rp, col, val, B, 2, C, 1, 0);
+      spmv::k_crs_row<double, false, false>(1, rp, col, val, B, 2, C, 1, 0);
+    });
+    bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
+      spmv::k_crs_row<double, true, true>(1, rp, col, val, B, 1, C, 1, 0);
     });
     bad |= row(len, 1, 1, 1, false, [&](int32_t* rp, double* B, double* C) {
       spmv::k_crs_wide<double, 1>(1, rp, col, val, B, 1, C, 1);
@@ -157,7 +160,7 @@ int main() {
       spmv::k_crs_long<double>(nullptr, 0, 0, 1, rp, col, val, B, 1, C, 1, 1, 32, 0);
     });
     bad |= row(len, 2, 2, 2, false, [&](int32_t* rp, double* B, double* C) {
-      spmv::k_crs_cols<double, 1>(1, rp, col, val, B, 2, C, 2, 2, 0);
+      spmv::k_crs_cols<double, 1, false>(1, rp, col, val, B, 2, C, 2, 2, 0);
     });
   }
   static int32_t zero = 0;
