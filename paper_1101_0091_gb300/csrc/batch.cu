@@ -323,6 +323,8 @@ static spmv_status build_graph(spmv_batch_plan* b) {
   return capture_graph(b, b->d_mats, b->vec, &b->graph, &b->exec);
 }
 
+constexpr int64_t kL1Bytes = 256 << 10;  // of an SM (with its shared memory)
+
 // What an item takes, relative to others: about the rounds of dependent loads that a warp runs through (chunks of
 // rows with one / two entries count four and two at a time, with up to four one at a time, longer ones a
 // slot each; other items each pass as their longest row).  Counted as the kernels step (their slots and
@@ -357,13 +359,16 @@ static spmv_status rebuild(spmv_batch_plan* b) {
   // starts last is run out alone.  512 members, k = 2 / 4: 368 -> 355, 499 -> 491 us;
   // 96 members 96.5 -> 84.2, 119.6 -> 111.7 us; 32 members, k = 8: 131 -> 112 us.
   // Twice as many lose more to the gathers from DRAM than they gain (k = 4).
-  // Not if all items are in flight at once: then none starts late, and neighbours of falling length load the SMs
-  // unevenly (200 members of 2000 rows, sorted, k = 6 / 8 / 12: 53.9 -> 48.1, 55.6 -> 49.8, 85.2 -> 79.2 us).
+  // Not if all items are in flight at once and the members are small: then none starts late, and neighbours of one
+  // member share its B in L1 (200 members of 2000 rows, sorted, k = 6 / 8 / 12: 53.9 -> 48.1, 55.6 -> 49.8, 85.2 -> 79.2 us;
+  // 27 members of 1000 .. 200,000 rows, k = 2, in flight at once: 42.6 in order of length, 43.8 not).
   const size_t warps = (size_t)b->num_sms * b->cfg.ctas_per_sm * (kBatchThreads / 32);
   int resident = 0;
   SPMV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, batch_kernel(b->k, b->vec), kBatchThreads, 0));
   const size_t in_flight = (size_t)b->num_sms * std::min(b->cfg.ctas_per_sm, resident) * (kBatchThreads / 32);
-  if (items.size() > in_flight)
+  int64_t b_bytes = 0;
+  for (spmv_handle p : b->plans) b_bytes += 8 * (int64_t)b->k * plan_csr(p)->n_cols;
+  if (items.size() > in_flight || b_bytes > kL1Bytes * (int64_t)b->plans.size())
     std::stable_sort(items.end() - std::min(items.size(), warps), items.end(),
                      [](const BatchItem& x, const BatchItem& y) { return item_rounds(x) > item_rounds(y); });
   b->n_chunk_items = std::count_if(items.begin(), items.end(), [](const BatchItem& it) { return it.mode == 3; });
