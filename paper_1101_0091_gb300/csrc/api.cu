@@ -253,11 +253,29 @@ static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const R
   const int64_t few = std::max<int64_t>(kManyLongRows, (int64_t)(kAutoOverShare * (double)n));
   const int64_t most = (int64_t)(kAutoLongShare * (double)n);
   if (s.longest <= kAutoLongestRow || s.n_long > most) return list;
-  *short_row = s.n_over <= std::min(few, most) ? kShortRow : kShortRowWide;
-  for (int64_t i = 0; i < n; ++i)
-    if (rp[i + 1] - rp[i] > *short_row) list.push_back((int32_t)i);
-  std::stable_sort(list.begin(), list.end(),
-                   [rp](int32_t a, int32_t b) { return rp[a + 1] - rp[a] > rp[b + 1] - rp[b]; });
+  const bool all = s.n_over <= std::min(few, most);
+  *short_row = all ? kShortRow : kShortRowWide;
+  const size_t count = (size_t)(all ? s.n_over : s.n_long);
+  std::vector<int32_t> rows(count + 1);  // (one more: every row is written, the long ones are kept)
+  size_t m = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    rows[m] = (int32_t)i;
+    m += rp[i + 1] - rp[i] > *short_row;
+  }
+  rows.resize(count);
+  // By falling length: a counting sort, with one bucket for the longest, which are sorted by comparison (a sort of
+  // them all: creating the plan of 1,000,000 power-law rows 15.4 ms, 13.9 so, 13.0 without a list).
+  constexpr int32_t kBuckets = 1024;
+  auto len = [rp](int32_t i) { return rp[i + 1] - rp[i]; };
+  std::vector<size_t> at(kBuckets + 1, 0);  // at[b]: rows of min(len, kBuckets - 1) > b, then where the next one goes
+  for (int32_t i : rows)
+    if (const int32_t b = std::min(len(i), kBuckets - 1)) ++at[b - 1];
+  for (int b = kBuckets - 2; b >= 0; --b) at[b] += at[b + 1];
+  const size_t n_longest = at[kBuckets - 2];
+  list.resize(rows.size());
+  for (int32_t i : rows) list[at[std::min(len(i), kBuckets - 1)]++] = i;
+  std::stable_sort(list.begin(), list.begin() + (int64_t)n_longest,
+                   [&](int32_t a, int32_t b) { return len(a) > len(b); });
   return list;
 }
 
@@ -270,7 +288,11 @@ static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n
   std::vector<int32_t> list;
   const RowStats stats = row_stats(rp, n_rows);
   M->lane_cols = lane_cols(stats, nnz);
-  if (long_rows) list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
+  try {
+    if (long_rows) list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
+  } catch (const std::bad_alloc&) {
+    return fail(SPMV_ERR_OOM, "host allocation failed");
+  }
   SPMV_CUDA(upload(p->arena, &drp, rp, n_rows + 1, (int64_t)list.size()));
   if (!list.empty()) {
     SPMV_CUDA(cudaMemcpy(drp + n_rows + 1, list.data(), sizeof(int32_t) * list.size(), cudaMemcpyHostToDevice));
