@@ -755,7 +755,8 @@ def lanczos_forms(A, torch, spmv, pm, stream, m: int = 30):
     """Lanczos (no reorthogonalisation) on k start vectors through the
     selector's SELL-32-4096 plan: time per step.  Bytes per step: V_min(k) +
     alpha (read W, v, v_prev; write W) + beta (read W, v; write W) = V_min +
-    56 k n."""
+    56 k n (the start's passes, over V0 twice and one cleared vector, are in the
+    measured time and not in the bound)."""
     import gen
     hbm, _ = measured_hbm()
     out = {"method": "Lanczos three-term recurrence, k independent start vectors", "steps": m}

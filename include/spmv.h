@@ -61,7 +61,14 @@ typedef enum {
                            /* are gathered at scattered addresses (entry (i, c) is regular when */
                            /* row i-1 holds column c-1 or row i+1 holds c+1) and SELL-32-256     */
                            /* stores at least 0.85 nonzeros per slot; CRS_L1 otherwise (a tuner  */
-                           /* or the cost model may switch)                                      */
+                           /* or the cost model may switch).  AUTO's CRS_L1 gives the long rows  */
+                           /* of a matrix that has few of them (the longest of more than 28      */
+                           /* entries, at most a quarter long) a warp or a CTA each.  Their sums */
+                           /* are formed in a fixed order that depends on k, so a column of a    */
+                           /* block equals the single-vector product to rounding there, bit for  */
+                           /* bit in all other rows.  spmv_info.variant reads CRS_L1 for this    */
+                           /* form and for an explicit CRS_L1, which keeps every row on one      */
+                           /* lane: keep 0 (AUTO), not the number read back, to restore it       */
   SPMV_CRS_STAGED = 1,     /* thread per row; each CTA's contiguous val/col tile is brought     */
                            /* into shared memory by one bulk copy (cp.async.bulk + mbarrier);   */
                            /* rows longer than 64 go to warp-per-row blocks                      */
@@ -448,7 +455,8 @@ spmv_status spmv_model_select_guarded(spmv_model_handle m, const double* feature
  * right-hand sides (spmv_features) go through the network (n_in must be 34),
  * output o stands for variant variants[o] with SELL sigma sigmas[o] (host
  * arrays of the network's n_out entries), and the plan switches to the
- * output with the smallest prediction as spmv_set_variant would.  *choice
+ * output with the smallest prediction as spmv_set_variant would (CRS_L1 then
+ * means the explicit one; see SPMV_VARIANT_AUTO).  *choice
  * (host) receives o.  Synchronises the stream. */
 spmv_status spmv_select(spmv_handle h, spmv_model_handle m, int32_t k, const int32_t* variants,
                         const int32_t* sigmas, int32_t* choice, void* stream);
@@ -460,7 +468,9 @@ spmv_status spmv_select(spmv_handle h, spmv_model_handle m, int32_t k, const int
  * switches to the candidate with the smallest median time.  *best (host)
  * receives its index; times_ms[n] (host, may be NULL) the medians, +inf for
  * a candidate the plan cannot build (e.g. SYM on an unsymmetric matrix).
- * Returns SPMV_ERR_UNSUPPORTED if no candidate builds.  Synchronous. */
+ * Variant 0 (AUTO) may be a candidate; on matrices with long rows it is not the
+ * kernel of an explicit CRS_L1.  Returns SPMV_ERR_UNSUPPORTED if no candidate
+ * builds; the plan then keeps the variant it was asked for before.  Synchronous. */
 spmv_status spmv_autotune(spmv_handle h, int32_t k, const double* B_dev, int64_t ldb, double* C_dev, int64_t ldc,
                           const int32_t* variants, const int32_t* sigmas, int32_t n, int32_t reps, int32_t* best,
                           float* times_ms, void* stream);
@@ -515,7 +525,9 @@ spmv_status spmv_cg_solve(spmv_solver_handle s, const double* B_dev, double* X_d
 /* m steps of the Lanczos three-term recurrence (no reorthogonalisation) from
  * the k columns of V0_dev: v_1 = v0/|v0|; w = A v_j - beta_{j-1} v_{j-1};
  * alpha_j = w.v_j; w -= alpha_j v_j; beta_j = |w|; v_{j+1} = w / beta_j.  A
- * column whose beta reaches 0 stops (zeros from there on).  alpha_host and
+ * column whose beta reaches 0 stops (zeros from there on).  |v0|^2 has to be
+ * a normal number; within that its size does not matter (scaled by a power of
+ * two it gives the same bits).  alpha_host and
  * beta_host are m x k row-major host arrays; the Ritz values are the
  * eigenvalues of the tridiagonal matrix with alpha_1..m on the diagonal and
  * beta_1..m-1 beside it.  Synchronous. */

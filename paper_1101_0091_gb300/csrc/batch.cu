@@ -360,8 +360,8 @@ static spmv_status rebuild(spmv_batch_plan* b) {
   // 96 members 96.5 -> 84.2, 119.6 -> 111.7 us; 32 members, k = 8: 131 -> 112 us.
   // Twice as many lose more to the gathers from DRAM than they gain (k = 4).
   // Not if all items are in flight at once and the members are small: then none starts late, and neighbours of one
-  // member share its B in L1 (200 members of 2000 rows, sorted, k = 6 / 8 / 12: 53.9 -> 48.1, 55.6 -> 49.8, 85.2 -> 79.2 us;
-  // 27 members of 1000 .. 200,000 rows, k = 2, in flight at once: 42.6 in order of length, 43.8 not).
+  // member share its B in L1 (200 members of 2000 rows, sorted, k = 6 / 8 / 12: 53.9 -> 48.1, 55.6 -> 49.8, 85.2 ->
+  // 79.2 us; 27 members of 1000 .. 200,000 rows, k = 2, in flight at once: 42.6 in order of length, 43.8 not).
   const size_t warps = (size_t)b->num_sms * b->cfg.ctas_per_sm * (kBatchThreads / 32);
   int resident = 0;
   SPMV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, batch_kernel(b->k, b->vec), kBatchThreads, 0));

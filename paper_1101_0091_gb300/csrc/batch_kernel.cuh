@@ -174,8 +174,8 @@ __device__ __forceinline__ void batch_rows(const BatchMat* __restrict__ Mp, cons
 template <int K, int VEC>
 __device__ __forceinline__ void batch_row_item(const BatchMat* __restrict__ Mp, const int2* __restrict__ rowlist,
                                                const BatchItem& item, int k, int lane) {
-  if (K == 2 && item.mode == 2) {
-    switch (item.lanes) {
+  if constexpr (K == 2) {
+    if (item.mode == 2) switch (item.lanes) {
       case 2: batch_rows<2, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
       case 4: batch_rows<4, K, VEC, 4>(Mp, rowlist, item, k, lane); return;
       case 8: batch_rows<8, K, VEC, 4>(Mp, rowlist, item, k, lane); return;

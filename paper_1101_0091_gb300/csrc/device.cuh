@@ -110,7 +110,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 // stores, for the same reason: eigenproblem matrix of 200,003 rows 15.0 -> 11.4 us, 27-point stencil 48^3
 // 13.9 -> 9.1, 400^2 Laplacian 4.5 -> 3.5.  Larger grids of even work overlap more of the next launch with
 // their last wave and call it at once (131 x 127 x 129 Poisson, k = 3: 77.8 us, in front of the stores 80.0).
-constexpr unsigned kOneWave = 152 * 8;  // CTAs of kThreads that the chip holds
+// The lines: k_crs_cols at one wave of kOneWave CTAs, k_crs_row at four, between which it does not matter
+// (at once / in front of the stores: 800^2 and 1000^2 Laplacians 7.66 / 7.66, 11.1 / 10.9 us; 72^3, 90^3 and 100^3
+// Poisson 6.6 / 6.9, 11.1 / 11.2, 17.2 / 17.0).  (k_crs_cols of several columns holds six CTAs, not eight: up to
+// 1.3 of its waves count as one.)
+constexpr unsigned kOneWave = 152 * 8;  // CTAs of kThreads that the chip holds, eight per SM
 __device__ __forceinline__ void grid_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -155,15 +159,14 @@ inline bool rows_on_16_bytes(const double* B, int64_t ldb, const double* C, int6
   return ldb % 2 == 0 && ldc % 2 == 0 && (((uintptr_t)B | (uintptr_t)C) & 15) == 0;
 }
 
-// Columns per lane of the column-split kernels (k_crs_cols, k_sell_cols) for k right-hand sides over
+// Columns per lane of k_crs_cols (k_sell_cols has its own rule, sell_cols) for k right-hand sides over
 // n_rows rows: up to `even` (4 or 2; 16-byte accesses) where k divides by it and the rows start on 16
 // bytes (a16), 3, 5 or 7 in 8-byte accesses where k divides by one of those and `odd` allows it, else 1.
 // These products are bound by the FP64 pipe (a warp's FMA occupies an SM for 16 cycles), so a lane per
 // column costs little that the pipe does not hide; a masked kernel of 4, 8 or 16 columns on one lane
 // issued the masked FMAs as well (k = 3 on a 131 x 127 x 129 Poisson matrix: 107.9 us masked, 79.7 with
 // one column per lane, FP64 floor 71).  Several columns per lane read the row's entries fewer times
-// (128^3 Poisson, k = 3 / 7 / 15, one -> several: 78.5 -> 76.1, 178.7 -> 170.5, 374.1 -> 362.3 us;
-// 600,011-row eigenproblem matrix in SELL, k = 6 / 9: 114.7 -> 94.4, 173.9 -> 140.9 us) as long as the
+// (128^3 Poisson, k = 3 / 7 / 15, one -> several: 78.5 -> 76.1, 178.7 -> 170.5, 374.1 -> 362.3 us) as long as the
 // threads still fill the GPU: at 60,000 rows, k = 4, four / two / one columns took 23.8 / 16.7 / 14.1 us, k = 5
 // five / one 30.7 / 13.5 us, hence kMinColThreads (the GPU holds 311,296 threads).
 constexpr int64_t kMinColThreads = 400000;

@@ -122,9 +122,9 @@ __device__ __forceinline__ void add_tail(int r, const VT* v, const double (*x)[W
 // 303.9 -> 272.4 us; 1500^2 Laplacian 39.0 -> 33.2 us; 3,000,000 rows of 5 entries 48.9 -> 41.1 us.  The
 // two pipes together bound it: 7 multiply-adds per row are 0.74 of the HBM time at 280^3, with FP32
 // values 0.99 of it.  Among uneven rows a warp waits for its longest anyway, and with FP32 values the
-// batches are masked (MASKED): 1,500,000 rows of 0 .. 12 / 4 .. 9 / 10 .. 30 entries 42.0 -> 35.1,
-// 42.6 -> 35.8, 53.9 -> 42.4 us, power-law rows of up to 16 35.0 -> 30.7.  (Doubles of the first, second and last: 44.3 -> 40.9,
-// 39.0 -> 40.8, 32.6 -> 37.0; not masked.)
+// batches are masked (MASKED): 1,500,000 rows of 0 .. 12 / 4 .. 9 / 10 .. 30 entries 42.0 -> 35.1, 42.6 ->
+// 35.8, 53.9 -> 42.4 us, power-law rows of up to 16 35.0 -> 30.7.  (Doubles of the first, second and last: 44.3 ->
+// 40.9, 39.0 -> 40.8, 32.6 -> 37.0; not masked.)
 template <typename VT, bool UNIT, bool MASKED>  // UNIT: ldb = 1 (its multiplication and two registers saved)
 __global__ void __launch_bounds__(kThreads, 8)
     k_crs_row(int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -236,8 +236,8 @@ static cudaError_t launch_cols(int64_t n_rows, const int32_t* row_ptr, const int
                                const double* B, int64_t ldb, double* C, int64_t ldc, int k, int pf, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_crs_cols<VT, W, A16>, (unsigned)grid, kThreads, s, n_rows, row_ptr, col, val, B, ldb, C, ldc, G,
-                          pf);
+  return launch_dependent(k_crs_cols<VT, W, A16>, (unsigned)grid, kThreads, s, n_rows, row_ptr, col, val, B, ldb, C,
+                          ldc, G, pf);
 }
 
 // out[i] = (a, b)[i + phase], i < 4, phase < 4: four consecutive entries that straddle two aligned groups.
@@ -336,8 +336,8 @@ template <typename VT, int W>
 static cudaError_t launch_wide(const CsrDev& A, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                                cudaStream_t s) {
   const int64_t grid = (A.n_rows + kWideThreads - 1) / kWideThreads;
-  return launch_dependent(k_crs_wide<VT, W>, (unsigned)grid, kWideThreads, s, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
-                          ldc);
+  return launch_dependent(k_crs_wide<VT, W>, (unsigned)grid, kWideThreads, s, A.n_rows, A.row_ptr, A.col, val, B,
+                          ldb, C, ldc);
 }
 
 // One row on NT threads (a warp or the CTA; thread t of them): EP entry lanes, a power of two, times
@@ -388,9 +388,9 @@ __device__ __forceinline__ void long_row(int row, int t, int k, const int32_t* _
 // four columns per lane 121.9 / 171.5 us, one 69.6 / 112.6).
 template <typename VT>
 __global__ void __launch_bounds__(kThreads, 8)
-    k_crs_long(const int32_t* __restrict__ long_rows, int n_long, int n_cta, int64_t n_rows, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-               const VT* __restrict__ val, const double* B, int64_t ldb, double* C,
-               int64_t ldc, int k, int short_row, int prefetch) {
+    k_crs_long(const int32_t* __restrict__ long_rows, int n_long, int n_cta, int64_t n_rows,
+               const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const VT* __restrict__ val,
+               const double* B, int64_t ldb, double* C, int64_t ldc, int k, int short_row, int prefetch) {
   __shared__ double sh[kThreads];
   constexpr int WARPS = kThreads / 32;
   const int tid = (int)threadIdx.x;
@@ -444,8 +444,8 @@ static cudaError_t launch_long(const CsrDev& A, const VT* val, const double* B, 
   const LongRows& lr = A.long_rows;
   const int rpc = kThreads / k, warps = kThreads / 32, n_cta = lr.n_cta[k];
   const int64_t grid = n_cta + (lr.n - n_cta + warps - 1) / warps + (A.n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_crs_long<VT>, (unsigned)grid, kThreads, s, lr.rows, lr.n, n_cta, A.n_rows, A.row_ptr, A.col, val, B, ldb, C,
-                          ldc, k, lr.short_row, A.prefetch);
+  return launch_dependent(k_crs_long<VT>, (unsigned)grid, kThreads, s, lr.rows, lr.n, n_cta, A.n_rows, A.row_ptr,
+                          A.col, val, B, ldb, C, ldc, k, lr.short_row, A.prefetch);
 }
 
 template <typename VT, int L, int K>
@@ -504,10 +504,10 @@ static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64
   // Short rows gain by two columns from fewer threads on where they are uneven (100,000 / 300,000 rows of 4 .. 9
   // entries, k = 4 / 2, one -> two columns 13.0 -> 10.6, 18.2 -> 14.1 us; of 0 .. 12 13.0 -> 13.5, 18.2 -> 18.0; 30,000
   // of 0 .. 12, k = 16, 11.2 -> 12.9), and in
-  // 8-byte accesses too (1,500,000 rows of 4 .. 9, k = 4, ld = 5 150.4 -> 113.1, of 1 49.0 -> 38.6, 160^3 Poisson 199.5 ->
-  // 192.3; 300,000 rows of 8 18.4 -> 20.0).
-  if (w == 1 && k % 2 == 0 && A.lane_cols > 1 && A.nnz < kWideRow * n && (even ? n * (k / 2) >= kMinColThreads : n >= 100000))
-    w = 2;
+  // 8-byte accesses too (1,500,000 rows of 4 .. 9, k = 4, ld = 5 150.4 -> 113.1, of 1 49.0 -> 38.6, 160^3 Poisson
+  // 199.5 -> 192.3; 300,000 rows of 8 18.4 -> 20.0).
+  const bool many = even ? n * (k / 2) >= kMinColThreads : n >= 100000;
+  if (w == 1 && k % 2 == 0 && A.lane_cols > 1 && A.nnz < kWideRow * n && many) w = 2;
   switch (w) {
     case 7: return launch_cols<VT, 7>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);
     case 5: return launch_cols<VT, 5>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);

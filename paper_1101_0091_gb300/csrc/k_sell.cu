@@ -10,7 +10,7 @@
 // slots) small.
 //
 // A block of k >= 2 columns runs k_sell_cols: each sorted row is shared by
-// G = k / W lanes with W columns each (cols_per_lane), and the G lanes of a row
+// G = k / W lanes with W columns each (sell_cols), and the G lanes of a row
 // read one contiguous piece of its B row; a row's slots are still summed in
 // order, so every W gives the same bits.  Here a lane stops at its row's own
 // length (from the CRS row_ptr): a warp's rows are fewer than a chunk's, and the
@@ -262,8 +262,8 @@ static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int6
     }
   }
   const int64_t grid = (S.n_chunks * kSellC + kThreads - 1) / kThreads;
-  return launch_dependent(k_sell<VT>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.chunk_ptr, S.chunk_len,
-                          S.col, val, B, ldb, C, ldc, S.prefetch);
+  return launch_dependent(k_sell<VT>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm, S.chunk_ptr,
+                          S.chunk_len, S.col, val, B, ldb, C, ldc, S.prefetch);
 }
 
 cudaError_t launch_sell(const SellDev& S, bool fp32, const double* B, int64_t ldb, double* C, int64_t ldc, int k,

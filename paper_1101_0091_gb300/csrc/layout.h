@@ -58,7 +58,7 @@ struct CsrDev {
   int prefetch = 0;                 // CTAs ahead whose val/col slices are prefetched into L2 (0 = off)
   bool val32_special = false;       // val32 holds a subnormal, infinite or NaN float
   int lane_cols = 4;                // most columns of a block that a lane of CRS_L1 takes (see upload_csr)
-  LongRows long_rows;               // listed (n_cta + n_warp > 0) when AUTO splits the long rows off CRS_L1
+  LongRows long_rows;               // listed (n > 0) when AUTO splits the long rows off CRS_L1
 };
 
 struct SellDev {

@@ -31,7 +31,7 @@ from . import _binding_model as bm
 
 PLAN_VARIANTS = [("crs_l1", 2, 1), ("crs_l2", 3, 1), ("crs_l4", 4, 1), ("crs_l8", 5, 1), ("crs_l32", 7, 1),
                  ("crs_staged", 1, 1), ("sell_s1", 8, 1), ("sell_s256", 8, 256), ("sell_s4096", 8, 4096)]
-PLAN_DEFAULT = 0          # CRS_L1, plain CRS (AUTO runs it on all but scattered matrices)
+PLAN_DEFAULT = 0          # CRS_L1, plain CRS: AUTO's kernel but for scattered matrices and those with long rows
 BATCH_POLICIES = [("l1", 0), ("l2", 1), ("l4", 2), ("l8", 3), ("l32", 4), ("adapt", 5), ("sorted", 6)]
 BATCH_DEFAULT = 6         # sorted, the batch's default policy
 BATCH_MARGIN = 0.25       # guard margin of an uncalibrated batch model (a predicted gain above ~28 %)
