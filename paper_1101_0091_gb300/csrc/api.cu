@@ -194,6 +194,8 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
   p->sell.n_rows = p->host.n_rows;
   p->sell.n_chunks = S.n_chunks;
   p->sell.slots = S.slots;
+  p->sell.nnz = p->host.nnz;
+  for (int32_t len : S.chunk_len) p->sell.longest = std::max(p->sell.longest, len);
   p->sell.sigma = sigma;
   p->sell.perm = perm;
   p->sell.row_ptr = p->A.row_ptr;
@@ -288,6 +290,7 @@ static spmv_status upload_csr(spmv_plan* p, CsrDev* M, int64_t n_rows, int64_t n
   std::vector<int32_t> list;
   const RowStats stats = row_stats(rp, n_rows);
   M->lane_cols = lane_cols(stats, nnz);
+  M->longest = stats.longest;
   try {
     if (long_rows) list = list_long_rows(rp, n_rows, stats, &long_rows->short_row);
   } catch (const std::bad_alloc&) {

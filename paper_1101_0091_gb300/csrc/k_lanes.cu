@@ -486,7 +486,9 @@ static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64
   if (A.long_rows.n > 0) return launch_long(A, val, B, ldb, C, ldc, k, s);
   const bool even = A.lane_cols == 4;
   if (k == 1) {
-    const bool masked = sizeof(VT) == 4 && !even;
+    // (not with longer rows: 200,000 rows of 4 or 60 entries 28.8 -> 35.5 us masked, power-law rows of up to 2000
+    // 173 -> 211)
+    const bool masked = sizeof(VT) == 4 && !even && A.longest <= kShortRowWide;
     if (!masked && A.nnz >= kWideRow * n) return launch_wide<VT, 1>(A, val, B, ldb, C, ldc, s);
     auto* row = masked ? (ldb == 1 ? k_crs_row<VT, true, sizeof(VT) == 4> : k_crs_row<VT, false, sizeof(VT) == 4>)
                        : (ldb == 1 ? k_crs_row<VT, true, false> : k_crs_row<VT, false, false>);
@@ -505,8 +507,9 @@ static cudaError_t crs_l1(const CsrDev& A, const VT* val, const double* B, int64
   // entries, k = 4 / 2, one -> two columns 13.0 -> 10.6, 18.2 -> 14.1 us; of 0 .. 12 13.0 -> 13.5, 18.2 -> 18.0; 30,000
   // of 0 .. 12, k = 16, 11.2 -> 12.9), and in
   // 8-byte accesses too (1,500,000 rows of 4 .. 9, k = 4, ld = 5 150.4 -> 113.1, of 1 49.0 -> 38.6, 160^3 Poisson
-  // 199.5 -> 192.3; 300,000 rows of 8 18.4 -> 20.0).
-  const bool many = even ? n * (k / 2) >= kMinColThreads : n >= 100000;
+  // 199.5 -> 192.3; 300,000 rows of 8 18.4 -> 20.0).  Not where one long row is walked by its lanes alone (100,000
+  // rows of 4 and one of 4000, k = 2: 446 -> 620).
+  const bool many = even ? n * (k / 2) >= kMinColThreads : n >= 100000 && A.longest <= kWalkedRow;
   if (w == 1 && k % 2 == 0 && A.lane_cols > 1 && A.nnz < kWideRow * n && many) w = 2;
   switch (w) {
     case 7: return launch_cols<VT, 7>(n, rp, col, val, B, ldb, C, ldc, k, pf, s);

@@ -104,11 +104,14 @@ __global__ void __launch_bounds__(kThreads)
 // (eigenproblem matrices of 600,011 and 2,000,003 rows, k = 6, 94.8 / 93.8 / 95.1 and 300 / 297 / 300 us), two, three
 // and four in 8 bytes 1.05 / 1.02 / 1.01, four in 16 bytes 1.02 / 1.01 / 1.04, five and seven 1.04 / 1.01 / 1.04;
 // floats one column 1.02 / 1.09 / 1.10, two 1.03 / 1.05 / 1.01, three and four 1.03 / 1.02 / 1.02.
-template <typename VT, int W, bool A16>
-constexpr int kSellStep = sizeof(VT) == 4 ? (W == 1 ? 0 : W == 2 ? 2 : 1) : (!A16 && W >= 2 && W <= 4 ? 2 : 1);
+// Two columns where a long row bounds the product (LONG, kWalkedRow): unrolled slots without the pipeline, 200,000
+// power-law rows of up to 2000, k = 2 / 4 561 -> 523, 575 -> 525 us (FP32 values, k = 2, 456 -> 400).
+template <typename VT, int W, bool A16, bool LONG>
+constexpr int kSellStep = LONG ? 0
+                          : sizeof(VT) == 4 ? (W == 1 ? 0 : W == 2 ? 2 : 1) : (!A16 && W >= 2 && W <= 4 ? 2 : 1);
 
 // k columns of a sorted row on G = k / W lanes, W columns each (as k_crs_cols).
-template <typename VT, int W, bool A16>
+template <typename VT, int W, bool A16, bool LONG>
 __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     k_sell_cols(int64_t n_rows, int64_t n_chunks, const int32_t* __restrict__ perm, const int32_t* __restrict__ row_ptr,
                 const int64_t* __restrict__ chunk_ptr, const int32_t* __restrict__ chunk_len,
@@ -136,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   const double* Bc = B + c0;
   const VT* vp = val + base;  // (advanced slot by slot: 32 slots of a row of 2^26 entries are out of 32 bits)
   const int32_t* cp = col + base;
-  constexpr int NB = kSellStep<VT, W, A16>;
+  constexpr int NB = kSellStep<VT, W, A16, LONG>;
   if constexpr (NB == 2) {
     VT v[NB];
     int32_t cc[NB];
@@ -198,6 +201,7 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
     }
   } else {
     double g[W];
+#pragma unroll 4
     for (int j = 0; j < len; ++j) {
       const double v = to_f64(ldcs(vp));
       load_cols<W, A16>(Bc + (int64_t)ldcs(cp) * ldb, g);
@@ -211,12 +215,12 @@ __global__ void __launch_bounds__(kThreads, (W == 1 ? 8 : 6))
   store_cols<W, A16>(C + (int64_t)row * ldc + c0, acc);
 }
 
-template <typename VT, int W, bool A16 = (W % 2 == 0)>
+template <typename VT, int W, bool A16 = (W % 2 == 0), bool LONG = false>
 static cudaError_t launch_cols(const SellDev& S, const VT* val, const double* B, int64_t ldb, double* C, int64_t ldc,
                                int k, cudaStream_t s) {
   const int G = k / W, rpc = kThreads / G;
   const int64_t grid = (S.n_rows + rpc - 1) / rpc;
-  return launch_dependent(k_sell_cols<VT, W, A16>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm,
+  return launch_dependent(k_sell_cols<VT, W, A16, LONG>, (unsigned)grid, kThreads, s, S.n_rows, S.n_chunks, S.perm,
                           S.row_ptr, S.chunk_ptr, S.chunk_len, S.col, val, B, ldb, C, ldc, G, S.prefetch);
 }
 
@@ -228,17 +232,23 @@ static int sell_cols(const SellDev& S, int k, bool a16) {
   // holds).  Two -> four columns, k = 16: 1,500,000 rows of 2 / 5 / 8 entries 168 -> 121, 271 -> 205, 341 -> 319 us,
   // 300,000 rows of 3 34.6 -> 27.2, of 13 106.6 -> 106.6; eigenproblem matrix of 600,011 rows (12.8 a row), k = 8,
   // 120.4 -> 126.2; of 60,000 rows, one -> four, 15.3 -> 19.8.
-  if (k % 4 == 0 && n * (k / 4) >= 1000000 && S.slots <= 9 * n) return 4;
-  // Two: k = 2 always (one -> two columns: 20,000 rows of 48 / 200 entries 21.9 -> 15.4, 57.8 -> 43.6 us, 200,000
-  // rows of 4 or 60 39.9 -> 32.8, eigenproblem matrices of 60,000 / 150,000 rows 9.3 -> 9.4, 16.6 -> 15.0), other k
-  // from as many threads on as k_crs_cols (k = 8, 60,000 / 150,000 rows 15.3 -> 17.8, 33.4 -> 34.2).
-  if (a16 && k % 2 == 0 && (k == 2 || n * (k / 2) >= kMinColThreads)) return 2;
+  // (1,000,000 power-law rows of up to 2000, k = 4 679 -> 1079.)
+  if (k % 4 == 0 && n * (k / 4) >= 1000000 && S.slots <= 9 * n && S.longest <= kWalkedRow) return 4;
+  // Two: k = 2 from 100,000 rows on or in long rows (one -> two columns: 20,000 rows of 48 / 200 entries 21.9 -> 15.4,
+  // 57.8 -> 43.6 us, 200,000 rows of 4 or 60 39.9 -> 32.8, eigenproblem matrices of 60,000 / 150,000 rows 9.3 -> 9.4,
+  // 16.6 -> 15.0, 300^2 Laplacian 4.0 -> 4.7), other k from as many threads on as k_crs_cols (k = 8, 60,000 / 150,000
+  // rows 15.3 -> 17.8, 33.4 -> 34.2).
+  const bool wide2 = k == 2 ? n >= 100000 || S.slots >= 24 * n : n * (k / 2) >= kMinColThreads;
+  if (a16 && k % 2 == 0 && wide2) return 2;
   // 8-byte accesses.  One -> two columns: 1,500,000 rows, k = 2, of 1 / 2 / 3 / 5 / 8 entries 23.2 -> 19.9, 32.5 ->
-  // 30.4, 37.2 -> 36.3, 44.1 -> 50.0, 63.2 -> 70.9 us, k = 4, of 8 entries 118 -> 94.
+  // 30.4, 37.2 -> 36.3, 44.1 -> 50.0, 63.2 -> 70.9 us, k = 4, of 8 entries 118 -> 94; unsorted rows of 4 or 60, k = 16,
+  // 180 -> 208.
   if (!(a16 && k % 2 == 0))
     for (int w : {7, 5, 3})
       if (k % w == 0 && n * (k / w) >= kMinColThreads) return w;
-  if (!a16 && k % 2 == 0 && n * (k / 2) >= kMinColThreads && (k > 2 || S.slots <= 3 * n)) return 2;
+  if (!a16 && k % 2 == 0 && n * (k / 2) >= kMinColThreads && (k > 2 || S.slots <= 3 * n) &&
+      (double)S.nnz >= kAutoSellFill * (double)S.slots)
+    return 2;
   return 1;
 }
 
@@ -256,6 +266,9 @@ static cudaError_t sell_k(const SellDev& S, const VT* val, const double* B, int6
                    : launch_cols<VT, 4, false>(S, val, B, ldb, C, ldc, k, s);
       case 3: return launch_cols<VT, 3>(S, val, B, ldb, C, ldc, k, s);
       case 2:
+        if (S.longest > kWalkedRow)
+          return a16 ? launch_cols<VT, 2, true, true>(S, val, B, ldb, C, ldc, k, s)
+                     : launch_cols<VT, 2, false, true>(S, val, B, ldb, C, ldc, k, s);
         return a16 ? launch_cols<VT, 2>(S, val, B, ldb, C, ldc, k, s)
                    : launch_cols<VT, 2, false>(S, val, B, ldb, C, ldc, k, s);
       default: return launch_cols<VT, 1>(S, val, B, ldb, C, ldc, k, s);

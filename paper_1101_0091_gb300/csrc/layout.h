@@ -40,6 +40,9 @@ struct LongRows {
   int n = 0, short_row = 0, n_cta[kMaxK + 1] = {};
 };
 
+// Products of matrices with a longer row than this are bound by the thread that walks it, where a row has one.
+constexpr int kWalkedRow = 64;
+
 // CRS_L1 reads the rows in aligned groups of four entries from this many entries per row on average
 // (kWideRowCols for blocks of two or four columns).
 constexpr int64_t kWideRow = 8;
@@ -58,12 +61,14 @@ struct CsrDev {
   int prefetch = 0;                 // CTAs ahead whose val/col slices are prefetched into L2 (0 = off)
   bool val32_special = false;       // val32 holds a subnormal, infinite or NaN float
   int lane_cols = 4;                // most columns of a block that a lane of CRS_L1 takes (see upload_csr)
+  int32_t longest = 0;              // entries of the longest row
   LongRows long_rows;               // listed (n > 0) when AUTO splits the long rows off CRS_L1
 };
 
 struct SellDev {
-  int64_t n_rows = 0, n_chunks = 0, slots = 0;
+  int64_t n_rows = 0, n_chunks = 0, slots = 0, nnz = 0;
   int sigma = 0;
+  int32_t longest = 0;              // slots per row of the longest chunk
   const int32_t* perm = nullptr;
   const int32_t* row_ptr = nullptr;  // of the CRS matrix (row lengths)
   const int64_t* chunk_ptr = nullptr;

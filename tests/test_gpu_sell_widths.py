@@ -44,3 +44,29 @@ def test_widths(lib, n, lo, hi, k, fp32):
     for y in ys:
         assert np.array_equal(y, want)
     assert_close(want, A, B, f32val=fp32)
+
+
+@pytest.mark.parametrize("longest", [64, 65, 300])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_one_long_row(lib, longest, fp32):
+    """Two columns per lane in unrolled slots from a row of more than 64 entries on."""
+    A = quick(200_001, 1, 3, seed=longest)
+    lens = np.diff(A.row_ptr)
+    lens[77_777] = longest
+    rp = np.zeros(A.n_rows + 1, np.int32)
+    rp[1:] = np.cumsum(lens)
+    rng = np.random.default_rng(longest)
+    A = gen.CSR(A.n_rows, A.n_cols, rp, rng.integers(0, A.n_cols, rp[-1]).astype(np.int32), rng.uniform(-1, 1, rp[-1]))
+    import torch
+    for k, ld in ((2, 2), (4, 4), (4, 5), (6, 6)):
+        B = gen.rhs_block(A.n_cols, k, seed=k)
+        Bd = torch.full((A.n_cols, ld), 7.0, dtype=torch.float64, device="cuda")
+        Bd[:, :k] = dev(B)
+        got = []
+        for variant in (lib.SPMV_SELL, lib.SPMV_CRS_L1):
+            with lib.Plan.from_csr(A, val_fp32=fp32, variant=variant, sell_sigma=256) as p:
+                C = torch.full((A.n_rows, ld), 7.0, dtype=torch.float64, device="cuda")
+                p.apply_block(Bd, C, k)
+                got.append(host(C))
+        assert np.array_equal(got[0], got[1]) and np.all(got[0][:, k:] == 7.0)
+        assert_close(np.ascontiguousarray(got[0][:, :k]), A, B, f32val=fp32)

@@ -94,7 +94,7 @@ template <int W> static int run(const double* val, const int32_t* col, int64_t* 
   const int k = W == 1 ? 2 : W;
   for (int i = 0; i < 16; ++i) B[i] = i < k ? 1 : 100 + i;
   cta(0, 1, false, [&] {
-    spmv::k_sell_cols<double, W, W % 2 == 0>(32, 1, perm, row_ptr, chunk_ptr, chunk_len, col, val, B, k, C, k, k / W, 0);
+    spmv::k_sell_cols<double, W, W % 2 == 0, false>(32, 1, perm, row_ptr, chunk_ptr, chunk_len, col, val, B, k, C, k, k / W, 0);
   });
   for (int q = 0; q < W; ++q) CHECK(C[q], 3.0 + 2 * B[k + q]);
   return 0;
