@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 8)
     C[g * ldc] = acc[0];
     return;
   }
-  for (; re - j >= 4; j += 4) {
+  for (; (uint32_t)j + 4 <= (uint32_t)re; j += 4) {
     const VT* vj = val + j;
     const int32_t* cj = col + j;
     double v[4], x[4];
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 8)
 #pragma unroll
   for (int u = 0; u < 3; ++u) {
     v[u] = x[u][0] = 0.0;
-    if (u < re - j) {
+    if ((uint32_t)j + u < (uint32_t)re) {
       v[u] = to_f64(ldg(val + j + u));
       x[u][0] = *(UNIT ? B + ldg(col + j + u) : B + (int64_t)ldg(col + j + u) * ldb);
     }
