@@ -216,29 +216,6 @@ static spmv_status build_sell_dev(spmv_plan* p, int sigma) {
   return SPMV_OK;
 }
 
-// What the choice of a CRS_L1 kernel needs of the row lengths, in one pass.
-struct RowStats {
-  int32_t longest = 0;
-  int64_t n_over = 0, n_long = 0;  // rows of more than kShortRow and of more than kShortRowWide entries
-  int64_t slots = 0;               // 32 x the longest row of every 32 consecutive rows
-};
-static RowStats row_stats(const int32_t* rp, int64_t n) {
-  RowStats s;
-  for (int64_t r0 = 0; r0 < n; r0 += 32) {
-    const int64_t r1 = std::min(r0 + 32, n);
-    int32_t most = 0;
-    for (int64_t i = r0; i < r1; ++i) {
-      const int32_t len = rp[i + 1] - rp[i];
-      most = std::max(most, len);
-      s.n_over += len > kShortRow;
-      s.n_long += len > kShortRowWide;
-    }
-    s.longest = std::max(s.longest, most);
-    s.slots += 32 * (int64_t)most;
-  }
-  return s;
-}
-
 // Columns of a block per lane: the more of them, the fewer times a row's entries are read, but the more
 // rows a warp holds and waits for the longest of.  By the share of a warp's slots that hold entries
 // (1,000,000 rows; four / two / one columns): 1.00 (3D Poisson, k = 16) 184.6 / 186.3 / 190.5 us; 0.72
@@ -246,39 +223,6 @@ static RowStats row_stats(const int32_t* rp, int64_t n) {
 // (power-law up to 40, k = 4) 118.3 / 85.2 / 66.4.
 static int lane_cols(const RowStats& s, int64_t nnz) {
   return nnz >= 0.95 * s.slots ? 4 : nnz >= 0.3 * s.slots ? 2 : 1;
-}
-
-// The long rows (LongRows), longest first (ties by row); none when no row exceeds kAutoLongestRow or when
-// more than kAutoLongShare of the rows are long.
-static std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s, int* short_row) {
-  std::vector<int32_t> list;
-  const int64_t few = std::max<int64_t>(kManyLongRows, (int64_t)(kAutoOverShare * (double)n));
-  const int64_t most = (int64_t)(kAutoLongShare * (double)n);
-  if (s.longest <= kAutoLongestRow || s.n_long > most) return list;
-  const bool all = s.n_over <= std::min(few, most);
-  *short_row = all ? kShortRow : kShortRowWide;
-  const size_t count = (size_t)(all ? s.n_over : s.n_long);
-  std::vector<int32_t> rows(count + 1);  // (one more: every row is written, the long ones are kept)
-  size_t m = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    rows[m] = (int32_t)i;
-    m += rp[i + 1] - rp[i] > *short_row;
-  }
-  rows.resize(count);
-  // By falling length: a counting sort, with one bucket for the longest, which are sorted by comparison (a sort of
-  // them all: creating the plan of 1,000,000 power-law rows 15.4 ms, 13.9 so, 13.0 without a list).
-  constexpr int32_t kBuckets = 1024;
-  auto len = [rp](int32_t i) { return rp[i + 1] - rp[i]; };
-  std::vector<size_t> at(kBuckets + 1, 0);  // at[b]: rows of min(len, kBuckets - 1) > b, then where the next one goes
-  for (int32_t i : rows)
-    if (const int32_t b = std::min(len(i), kBuckets - 1)) ++at[b - 1];
-  for (int b = kBuckets - 2; b >= 0; --b) at[b] += at[b + 1];
-  const size_t n_longest = at[kBuckets - 2];
-  list.resize(rows.size());
-  for (int32_t i : rows) list[at[std::min(len(i), kBuckets - 1)]++] = i;
-  std::stable_sort(list.begin(), list.begin() + (int64_t)n_longest,
-                   [&](int32_t a, int32_t b) { return len(a) > len(b); });
-  return list;
 }
 
 // long_rows (NULL for the parts of a split) receives the list of list_long_rows,

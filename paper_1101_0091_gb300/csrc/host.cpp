@@ -201,6 +201,58 @@ double sell_fill(const int32_t* rp, int64_t n_rows, int64_t sigma) {
   return slots ? (double)nnz / (double)slots : 1.0;
 }
 
+RowStats row_stats(const int32_t* rp, int64_t n) {
+  RowStats s;
+  auto rows = [&](const int32_t* p, int m) {  // 32 rows at most, in 32 bits: vector code for m = 32
+    int32_t most = 0, over = 0, lng = 0;
+    for (int i = 0; i < m; ++i) {
+      const int32_t len = p[i + 1] - p[i];
+      most = len > most ? len : most;
+      over += len > kShortRow;
+      lng += len > kShortRowWide;
+    }
+    s.n_over += over;
+    s.n_long += lng;
+    s.longest = std::max(s.longest, most);
+    s.slots += 32 * (int64_t)most;
+  };
+  int64_t r = 0;
+  for (; r + 32 <= n; r += 32) rows(rp + r, 32);
+  if (r < n) rows(rp + r, (int)(n - r));
+  return s;
+}
+
+std::vector<int32_t> list_long_rows(const int32_t* rp, int64_t n, const RowStats& s, int* short_row) {
+  std::vector<int32_t> list;
+  const int64_t few = std::max<int64_t>(kManyLongRows, (int64_t)(kAutoOverShare * (double)n));
+  const int64_t most = (int64_t)(kAutoLongShare * (double)n);
+  if (s.longest <= kAutoLongestRow || s.n_long > most) return list;
+  const bool all = s.n_over <= std::min(few, most);
+  *short_row = all ? kShortRow : kShortRowWide;
+  const size_t count = (size_t)(all ? s.n_over : s.n_long);
+  std::vector<int32_t> rows(count + 1);  // (one more: every row is written, the long ones are kept)
+  size_t m = 0;
+  for (int64_t i = 0; i < n; ++i) {
+    rows[m] = (int32_t)i;
+    m += rp[i + 1] - rp[i] > *short_row;
+  }
+  rows.resize(count);
+  // By falling length: a counting sort, with one bucket for the longest, which are sorted by comparison (a sort of
+  // them all: creating the plan of 1,000,000 power-law rows 15.4 ms, 13.9 so, 13.0 without a list).
+  constexpr int32_t kBuckets = 1024;
+  auto len = [rp](int32_t i) { return rp[i + 1] - rp[i]; };
+  std::vector<size_t> at(kBuckets + 1, 0);  // at[b]: rows of min(len, kBuckets - 1) > b, then where the next one goes
+  for (int32_t i : rows)
+    if (const int32_t b = std::min(len(i), kBuckets - 1)) ++at[b - 1];
+  for (int b = kBuckets - 2; b >= 0; --b) at[b] += at[b + 1];
+  const size_t n_longest = at[kBuckets - 2];
+  list.resize(rows.size());
+  for (int32_t i : rows) list[at[std::min(len(i), kBuckets - 1)]++] = i;
+  std::stable_sort(list.begin(), list.begin() + (int64_t)n_longest,
+                   [&](int32_t a, int32_t b) { return len(a) > len(b); });
+  return list;
+}
+
 // Local/halo split at column h (Sec. 3.1): local = entries with col < h over all
 // rows, halo = entries with col >= h over the ascending list of rows that have
 // any; in-row order kept, global column indices.

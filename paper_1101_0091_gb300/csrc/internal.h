@@ -109,6 +109,17 @@ constexpr double kAutoOverShare = 0.03;
 double scattered_fraction(const int32_t* row_ptr, const int32_t* col, int64_t n_rows);
 // Nonzeros over stored slots of SELL-32-sigma, from the row lengths.
 double sell_fill(const int32_t* row_ptr, int64_t n_rows, int64_t sigma);
+// What the choice of a CRS_L1 kernel needs of the row lengths, in one pass.
+struct RowStats {
+  int32_t longest = 0;
+  int64_t n_over = 0, n_long = 0;  // rows of more than kShortRow and of more than kShortRowWide entries
+  int64_t slots = 0;               // 32 x the longest row of every 32 consecutive rows
+};
+RowStats row_stats(const int32_t* row_ptr, int64_t n_rows);
+// The long rows (LongRows), longest first (ties by row); none when no row exceeds kAutoLongestRow or when
+// more than kAutoLongShare of the rows are long.
+std::vector<int32_t> list_long_rows(const int32_t* row_ptr, int64_t n_rows, const RowStats& s, int* short_row);
+
 void compute_features(int64_t n_rows, int64_t n_cols, const int32_t* row_ptr, const int32_t* col,
                       int k, double* f);
 
